@@ -115,8 +115,10 @@ mt_status mt_graph_copy_csr(const mt_graph* g, int32_t* row_ptr, int32_t* col, v
  * the device: each of the 2^(k(k-1)) keys is canonicalised by the minimum over
  * all k! vertex orderings, the connected canonical masks are ranked, and each
  * key's slot receives its dense class id, or 0xFFFFFFFF for a disconnected
- * pattern.  Device memory: 4 * 2^(k(k-1)) bytes (4 GiB for k = 6) plus
- * 2^(k(k-1))/4 bytes of scratch freed before return.
+ * pattern.  (At k = 6 only the keys whose first five vertices are in canonical
+ * order are walked; the others' slots are copies of theirs.)  Device memory:
+ * 4 * 2^(k(k-1)) bytes (4 GiB for k = 6) plus at most 2^(k(k-1))/4 bytes of
+ * scratch freed before return.
  * Key layout ("extension-order key", used by the counting kernels): the k
  * vertices are listed in the order the enumerator adds them; position p >= 1
  * owns the 2p bits starting at k(k-1) - p(p+1) (the last position in the
@@ -137,8 +139,8 @@ mt_status mt_table_build(int k, void* stream, mt_table** out);
  * fields for the vertices of X are permuted, the sixth vertex's field for the
  * fifth is not), which leaves the class of the whole unchanged.  Slot
  * (class of X) << 18 | relabelled fifth word << 10 | relabelled sixth word
- * holds the dense id.  Built from the full table, which is freed before return
- * (peak device memory: the full table's).  Class ids and class masks are the
+ * holds the dense id.  Scratch while it builds: about 220 MB, freed before
+ * return.  Class ids and class masks are the
  * full table's.  Counting with a compact table supports the per-subgraph
  * method only (MT_METHOD_CELLS gives MT_EUNSUPPORTED); mt_table_entries reads
  * compact slots.  Synchronises `stream`.

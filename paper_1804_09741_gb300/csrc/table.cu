@@ -15,6 +15,10 @@
 // A popcount prefix over the bitmap then ranks the connected canonical masks
 // (dense id = rank), and a last pass replaces each slot by the id of its
 // canonical mask, or 0xFFFFFFFF for disconnected patterns.
+//
+// At k = 6 steps 2 and 3 run over the 9,608 x 2^10 keys whose first five
+// vertices are in canonical order only, and the other rows of the table are
+// permuted copies (see "k = 6 through its 5-vertex prefixes").
 #include <algorithm>
 #include <numeric>
 #include <vector>
@@ -37,7 +41,7 @@ struct mt_table {
 
 namespace mt {
 
-__constant__ uint8_t c_sjt[720];  // transposition positions p (swap p, p+1)
+__constant__ uint8_t c_sjt[7][720];  // per k: transposition positions p (swap p, p+1)
 
 // Positions of the adjacent transpositions that take the identity through all
 // k! permutations (Steinhaus-Johnson-Trotter with directions).
@@ -125,7 +129,7 @@ __global__ void __launch_bounds__(256) k_canon(uint32_t* table, uint32_t* bitmap
     const uint64_t x0 = key_to_matrix((uint32_t)key, K);
     uint64_t x = x0, best = x0;
     for (int s = 0; s < nsteps; ++s) {
-      x = swap_adjacent(x, c_sjt[s]);
+      x = swap_adjacent(x, c_sjt[K][s]);
       best = x < best ? x : best;
     }
     const uint32_t canon = matrix_to_mask(best, K);
@@ -135,16 +139,21 @@ __global__ void __launch_bounds__(256) k_canon(uint32_t* table, uint32_t* bitmap
   }
 }
 
-// prefix[w] = number of set bits in bitmap[0..w); tile sums first.
+// prefix[q] = number of set bits in the bitmap's 128-bit groups 0..q-1 (one
+// uint4 each; a rank adds the group's own words); tile sums first.
 constexpr int kScanThreads = 256, kScanPer = 16, kScanTile = kScanThreads * kScanPer;
 
-__global__ void k_tile_popc(const uint32_t* bitmap, size_t nwords, int32_t* tile_sum) {
+__device__ __forceinline__ int popc4(uint4 v) {
+  return __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+}
+
+__global__ void k_tile_popc(const uint4* bitmap, size_t ngroups, int32_t* tile_sum) {
   __shared__ int red[kScanThreads / 32];
   const size_t base = (size_t)blockIdx.x * kScanTile;
   int s = 0;
   for (int i = 0; i < kScanPer; ++i) {
     size_t w = base + (size_t)i * kScanThreads + threadIdx.x;
-    if (w < nwords) s += __popc(bitmap[w]);
+    if (w < ngroups) s += popc4(bitmap[w]);
   }
   for (int d = 16; d; d >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
@@ -161,144 +170,366 @@ __global__ void __launch_bounds__(1024) k_scan_single(int32_t* data, int count) 
   block_exclusive_scan(data, count, tmp);
 }
 
-__global__ void k_tile_prefix(const uint32_t* bitmap, size_t nwords, const int32_t* tile_off,
+// A warp scans 32 consecutive groups at a time, so its reads and writes are
+// coalesced; the tile's warps take the tile's slices in order.
+__global__ void k_tile_prefix(const uint4* bitmap, size_t ngroups, const int32_t* tile_off,
                               int32_t* prefix) {
-  __shared__ int wsum[kScanThreads / 32 + 1];
-  const size_t base = (size_t)blockIdx.x * kScanTile + (size_t)threadIdx.x * kScanPer;
-  int loc[kScanPer];
-  int s = 0;
-  for (int i = 0; i < kScanPer; ++i) {
-    const size_t w = base + i;
-    loc[i] = s;
-    s += w < nwords ? __popc(bitmap[w]) : 0;
-  }
+  constexpr int kWarps = kScanThreads / 32, kSlice = kScanTile / kWarps;
+  __shared__ int wsum[kWarps];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int inc = warp_incl_scan(s);
-  if (lane == 31) wsum[wid] = inc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int acc = 0;
-    for (int i = 0; i < kScanThreads / 32; ++i) {
-      int t = wsum[i];
-      wsum[i] = acc;
-      acc += t;
-    }
+  const size_t base = (size_t)blockIdx.x * kScanTile + (size_t)wid * kSlice;
+  int loc[kSlice / 32];
+  int s = 0;
+  for (int i = 0; i < kSlice / 32; ++i) {
+    const size_t w = base + (size_t)i * 32 + lane;
+    const int c = w < ngroups ? popc4(bitmap[w]) : 0;
+    const int inc = warp_incl_scan(c);
+    loc[i] = s + inc - c;
+    s += __shfl_sync(0xFFFFFFFFu, inc, 31);
   }
+  if (lane == 0) wsum[wid] = s;
   __syncthreads();
-  const int off = tile_off[blockIdx.x] + wsum[wid] + inc - s;
-  for (int i = 0; i < kScanPer; ++i) {
-    const size_t w = base + i;
-    if (w < nwords) prefix[w] = off + loc[i];
+  int off = tile_off[blockIdx.x];
+  for (int i = 0; i < wid; ++i) off += wsum[i];
+  for (int i = 0; i < kSlice / 32; ++i) {
+    const size_t w = base + (size_t)i * 32 + lane;
+    if (w < ngroups) prefix[w] = off + loc[i];
   }
 }
 
-__global__ void k_assign(uint32_t* table, uint64_t nkeys, const uint32_t* bitmap,
+// Rank of bit c among the set bits, or kNoClass when it is not set.
+__device__ __forceinline__ uint32_t rank_of(const uint4* bitmap, const int32_t* prefix,
+                                            uint32_t c) {
+  const uint4 v = bitmap[c >> 7];
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  const uint32_t at = (c >> 5) & 3u, bit = 1u << (c & 31u);
+  uint32_t r = (uint32_t)prefix[c >> 7], own = 0;
+#pragma unroll
+  for (uint32_t i = 0; i < 4; ++i) {
+    if (i < at) r += __popc(w[i]);
+    if (i == at) own = w[i];
+  }
+  return (own & bit) ? r + __popc(own & (bit - 1u)) : kNoClass;
+}
+
+// table[key] = rank of the canonical mask that k_canon or k_sub_canon left there.
+__global__ void k_assign(uint32_t* table, uint64_t nkeys, const uint4* bitmap,
                          const int32_t* prefix) {
   for (uint64_t key = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; key < nkeys;
-       key += (uint64_t)gridDim.x * blockDim.x) {
-    const uint32_t c = table[key];
-    const uint32_t w = bitmap[c >> 5];
-    const uint32_t bit = 1u << (c & 31u);
-    table[key] = (w & bit) ? (uint32_t)prefix[c >> 5] + __popc(w & (bit - 1u)) : kNoClass;
+       key += (uint64_t)gridDim.x * blockDim.x)
+    table[key] = rank_of(bitmap, prefix, table[key]);
+}
+
+// The set bits of the bitmap in ascending order.
+__global__ void k_bit_list(const uint4* bitmap, size_t ngroups, const int32_t* prefix,
+                           uint32_t* out, uint32_t count) {
+  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < ngroups;
+       q += (size_t)gridDim.x * blockDim.x) {
+    const uint4 v = bitmap[q];
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    uint32_t r = (uint32_t)prefix[q];
+    for (int i = 0; i < 4; ++i)
+      for (uint32_t bits = w[i]; bits; bits &= bits - 1u, ++r)
+        if (r < count) out[r] = (uint32_t)(q * 128 + i * 32 + __ffs(bits) - 1);
   }
 }
 
-__global__ void k_class_list(const uint32_t* bitmap, size_t nwords, const int32_t* prefix,
-                             uint32_t* out, uint32_t classes) {
-  for (size_t w = blockIdx.x * (size_t)blockDim.x + threadIdx.x; w < nwords;
-       w += (size_t)gridDim.x * blockDim.x) {
-    uint32_t bits = bitmap[w];
-    int r = prefix[w];
-    while (bits) {
-      const int b = __ffs(bits) - 1;
-      if ((uint32_t)r < classes) out[r] = (uint32_t)(w * 32 + b);
-      ++r;
-      bits &= bits - 1u;
+static cudaError_t launch_rank(const uint32_t* bitmap, size_t ngroups, int32_t* tiles,
+                               int32_t* prefix, cudaStream_t s) {
+  const unsigned ntiles = (unsigned)((ngroups + kScanTile - 1) / kScanTile);
+  const uint4* bits = (const uint4*)bitmap;
+  k_tile_popc<<<ntiles, kScanThreads, 0, s>>>(bits, ngroups, tiles);
+  k_scan_single<<<1, 1024, 0, s>>>(tiles, (int)ntiles);
+  k_tile_prefix<<<ntiles, kScanThreads, 0, s>>>(bits, ngroups, tiles, prefix);
+  return cudaGetLastError();
+}
+
+// --------------------------------------------- k = 6 through its 5-vertex prefixes
+//
+// A 6-vertex key is a 5-vertex prefix X (key bits 10..29, itself a 5-vertex
+// extension-order key) and the sixth vertex's word z (bits 0..9).  Relabelling
+// X into the canonical order of its own class and z's fields with it leaves the
+// class of the whole unchanged, so only 9,608 x 2^10 of the 2^30 keys (one
+// prefix per 5-vertex digraph, connected or not) go through the k! orderings;
+// every other row of 1,024 slots is one of theirs with its slots permuted.
+// Measured on a GB300, table, count and read-out of one 800-vertex graph: 910
+// ms with all 2^30 keys walked (893 ms of it k_canon<6>), 18.4 ms this way.
+
+constexpr int kP5Keys = 1 << 20;      // 5-vertex prefix keys
+constexpr uint32_t kP5Classes = 9608; // 5-vertex digraphs up to isomorphism
+constexpr int kP5Low = 10;            // bits of the sixth vertex's word
+
+// For every prefix key: its canonical mask and the ordering sigma that reaches
+// it (new position i holds old vertex sigma(i), 3 bits each); marks the
+// canonical masks.
+__global__ void __launch_bounds__(256) k_prefix5(uint32_t* canon, uint16_t* sigma,
+                                                 uint32_t* bitmap, int nsteps) {
+  const uint32_t xk = blockIdx.x * blockDim.x + threadIdx.x;
+  if (xk >= (uint32_t)kP5Keys) return;
+  const uint64_t x0 = key_to_matrix(xk, 5);
+  uint64_t x = x0, best = x0;
+  uint32_t at = 0 | (1 << 3) | (2 << 6) | (3 << 9) | (4 << 12), best_at = at;
+  for (int s = 0; s < nsteps; ++s) {
+    const int p = c_sjt[5][s];
+    x = swap_adjacent(x, p);
+    const uint32_t t = ((at >> (3 * p)) ^ (at >> (3 * p + 3))) & 7u;
+    at ^= (t << (3 * p)) | (t << (3 * p + 3));
+    if (x < best) {
+      best = x;
+      best_at = at;
     }
   }
+  const uint32_t c = matrix_to_mask(best, 5);
+  canon[xk] = c;
+  sigma[xk] = (uint16_t)best_at;
+  if (best == x0) atomicOr(&bitmap[c >> 5], 1u << (c & 31u));
+}
+
+// 5-vertex canonical mask -> the prefix key with that very matrix.
+__device__ __forceinline__ uint32_t mask5_to_key(uint32_t mask) {
+  uint32_t key = 0;
+  for (int p = 1; p < 5; ++p)
+    for (int q = 0; q < p; ++q) {
+      const int off = 20 - p * (p + 1) + 2 * q;
+      key |= ((mask >> (q * 4 + p - 1)) & 1u) << off;        // q -> p
+      key |= ((mask >> (p * 4 + q)) & 1u) << (off + 1);      // p -> q
+    }
+  return key;
+}
+
+// Canonical masks of the 6-vertex keys above the class prefixes (sub[class][z]);
+// marks the connected ones.  Disconnected patterns get mask 0, which is not
+// connected and so is never marked.
+__global__ void __launch_bounds__(256) k_sub_canon(uint32_t* sub, const uint32_t* masks5,
+                                                   uint32_t* bitmap, int nsteps) {
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (kP5Classes << kP5Low)) return;
+  const uint32_t key =
+      (mask5_to_key(masks5[i >> kP5Low]) << kP5Low) | (i & ((1u << kP5Low) - 1u));
+  const uint64_t x0 = key_to_matrix(key, 6);
+  uint32_t c = 0;
+  if (matrix_connected(x0, 6)) {
+    uint64_t x = x0, best = x0;
+    for (int s = 0; s < nsteps; ++s) {
+      x = swap_adjacent(x, c_sjt[6][s]);
+      best = x < best ? x : best;
+    }
+    c = matrix_to_mask(best, 6);
+    const uint32_t bit = 1u << (c & 31u);
+    // about six keys share a mask: most find the bit set
+    if (!(*(volatile uint32_t*)&bitmap[c >> 5] & bit)) atomicOr(&bitmap[c >> 5], bit);
+  }
+  sub[i] = c;
+}
+
+// out[row * 1024 + z] = sub[class of the row's prefix][z relabelled]; row r's
+// prefix key is r, or prefix_of[r >> 8] << 8 | (r & 255) for the compact form's
+// rows.  One warp per row, four neighbouring slots per lane and store.
+__global__ void __launch_bounds__(256) k_expand(uint32_t* __restrict__ out,
+                                                const uint32_t* __restrict__ sub,
+                                                const uint32_t* __restrict__ class5,
+                                                const uint16_t* __restrict__ sigma,
+                                                const int32_t* __restrict__ prefix_of,
+                                                uint32_t nrows) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+  for (uint32_t r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < nrows; r += warps) {
+    const uint32_t xk = prefix_of ? ((uint32_t)prefix_of[r >> 8] << 8) | (r & 255u) : r;
+    const uint32_t* row = sub + ((size_t)class5[xk] << kP5Low);
+    const uint32_t sg = sigma[xk];
+    int to[5];  // where z's field q goes
+#pragma unroll
+    for (int q = 0; q < 5; ++q) to[q] = 0;
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+#pragma unroll
+      for (int q = 0; q < 5; ++q)
+        if (((sg >> (3 * i)) & 7u) == (uint32_t)q) to[q] = 2 * i;
+    // z = step * 128 + lane * 4 + t: t is field 0, the lane fields 1, 2 and the
+    // low bit of 3, the step the high bit of 3 and field 4
+    const uint32_t zl = ((lane & 3u) << to[1]) | (((lane >> 2) & 3u) << to[2]) |
+                        ((uint32_t)(lane >> 4) << to[3]);
+    uint4* o = (uint4*)(out + ((size_t)r << kP5Low)) + lane;
+#pragma unroll
+    for (int step = 0; step < 8; ++step) {
+      const uint32_t z = zl | ((uint32_t)(step & 1) << (to[3] + 1)) |
+                         ((uint32_t)(step >> 1) << to[4]);
+      uint4 v;
+      v.x = __ldg(row + z);
+      v.y = __ldg(row + (z | (1u << to[0])));
+      v.z = __ldg(row + (z | (2u << to[0])));
+      v.w = __ldg(row + (z | (3u << to[0])));
+      o[step * 32] = v;
+    }
+  }
+}
+
+// Upload k's transposition sequence (always the same bytes), after checking that
+// the walk visits every ordering exactly once.
+static mt_status upload_sjt(int k, cudaStream_t s, int* nsteps) {
+  const std::vector<uint8_t> seq = sjt_sequence(k);
+  std::vector<uint32_t> seen;
+  uint32_t p = 0x543210u & ((1u << (4 * k)) - 1u);  // 4 bits per position
+  seen.push_back(p);
+  for (uint8_t q : seq) {
+    const uint32_t t = ((p >> (4 * q)) ^ (p >> (4 * q + 4))) & 15u;
+    p ^= (t << (4 * q)) | (t << (4 * q + 4));
+    seen.push_back(p);
+  }
+  std::sort(seen.begin(), seen.end());
+  size_t fact = 1;
+  for (int i = 2; i <= k; ++i) fact *= i;
+  if (seq.size() + 1 != fact || std::unique(seen.begin(), seen.end()) != seen.end())
+    return MT_ECUDA;
+  MT_CUDA_TRY(cudaMemcpyToSymbolAsync(c_sjt, seq.data(), seq.size(), (size_t)k * 720,
+                                      cudaMemcpyHostToDevice, s));
+  *nsteps = (int)seq.size();
+  return MT_OK;
+}
+
+static int sm_count() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
+// Scratch of one build, one stream-ordered allocation.
+struct TableScratch {
+  char* mem = nullptr;
+  size_t off = 0, bytes = 0;
+  uint32_t *bitmap = nullptr, *bitmap5 = nullptr;  // connected 6- (or k-), 5-vertex masks
+  size_t ngroups = 0, ngroups5 = 0, zeroed = 0;
+  int32_t *prefix = nullptr, *prefix5 = nullptr, *tiles = nullptr;
+  uint32_t *sub = nullptr, *class5 = nullptr, *masks5 = nullptr;
+  uint16_t* sigma = nullptr;
+  int32_t* reps = nullptr;  // compact form: representative 4-vertex prefix keys
+};
+
+static cudaError_t scratch_alloc(TableScratch* x, int k, cudaStream_t s) {
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    const size_t o = off;
+    off += (bytes + 255) & ~(size_t)255;
+    return o;
+  };
+  x->ngroups = (size_t)std::max<uint64_t>((1ull << (k * (k - 1))) / 128, 1);
+  x->ngroups5 = k == 6 ? kP5Keys / 128 : 0;
+  const size_t tiles = (x->ngroups + kScanTile - 1) / kScanTile;
+  const size_t o_b = take(x->ngroups * 16), o_b5 = take(x->ngroups5 * 16);
+  x->zeroed = off;
+  const size_t o_p = take(x->ngroups * 4), o_p5 = take(x->ngroups5 * 4), o_t = take(tiles * 4);
+  const size_t o_s = take(k == 6 ? ((size_t)kP5Classes << kP5Low) * 4 : 0);
+  const size_t o_c = take(k == 6 ? (size_t)kP5Keys * 4 : 0);
+  const size_t o_m = take(k == 6 ? (size_t)kP5Classes * 4 : 0);
+  const size_t o_g = take(k == 6 ? (size_t)kP5Keys * 2 : 0);
+  const size_t o_r = take(k == 6 ? 256 * 4 : 0);
+  cudaError_t e = cudaMallocAsync((void**)&x->mem, off, s);
+  if (e != cudaSuccess) return e;
+  x->bitmap = (uint32_t*)(x->mem + o_b);
+  x->bitmap5 = (uint32_t*)(x->mem + o_b5);
+  x->prefix = (int32_t*)(x->mem + o_p);
+  x->prefix5 = (int32_t*)(x->mem + o_p5);
+  x->tiles = (int32_t*)(x->mem + o_t);
+  x->sub = (uint32_t*)(x->mem + o_s);
+  x->class5 = (uint32_t*)(x->mem + o_c);
+  x->masks5 = (uint32_t*)(x->mem + o_m);
+  x->sigma = (uint16_t*)(x->mem + o_g);
+  x->reps = (int32_t*)(x->mem + o_r);
+  return cudaMemsetAsync(x->mem, 0, x->zeroed, s);
+}
+
+// The 5-vertex classes and the dense ids above them (x->sub, x->class5,
+// x->sigma), and the class list.
+static cudaError_t launch_sub6(const TableScratch& x, uint32_t* class_masks, int nsteps5,
+                               int nsteps6, int sms, cudaStream_t s) {
+  k_prefix5<<<kP5Keys / 256, 256, 0, s>>>(x.class5, x.sigma, x.bitmap5, nsteps5);
+  cudaError_t e = launch_rank(x.bitmap5, x.ngroups5, x.tiles, x.prefix5, s);
+  if (e != cudaSuccess) return e;
+  const uint4* b5 = (const uint4*)x.bitmap5;
+  const uint4* b6 = (const uint4*)x.bitmap;
+  k_bit_list<<<32, 256, 0, s>>>(b5, x.ngroups5, x.prefix5, x.masks5, kP5Classes);
+  k_assign<<<sms * 8, 256, 0, s>>>(x.class5, kP5Keys, b5, x.prefix5);
+  const uint32_t nsub = kP5Classes << kP5Low;
+  k_sub_canon<<<(nsub + 255) / 256, 256, 0, s>>>(x.sub, x.masks5, x.bitmap, nsteps6);
+  e = launch_rank(x.bitmap, x.ngroups, x.tiles, x.prefix, s);
+  if (e != cudaSuccess) return e;
+  k_assign<<<sms * 16, 256, 0, s>>>(x.sub, nsub, b6, x.prefix);
+  k_bit_list<<<sms * 8, 256, 0, s>>>(b6, x.ngroups, x.prefix, class_masks, kNumClasses[6]);
+  return cudaGetLastError();
+}
+
+// Number of set bits of a ranked bitmap, read back to `out[0..4]` (prefix of
+// the last group, then its words).
+static cudaError_t read_total(const uint32_t* bitmap, const int32_t* prefix, size_t ngroups,
+                              uint32_t* out, cudaStream_t s) {
+  cudaError_t e = cudaMemcpyAsync(out, prefix + ngroups - 1, 4, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(out + 1, bitmap + 4 * (ngroups - 1), 16, cudaMemcpyDeviceToHost, s);
+  return e;
+}
+static uint32_t total_of(const uint32_t* r) {
+  uint32_t t = r[0];
+  for (int i = 1; i < 5; ++i) t += (uint32_t)__builtin_popcount(r[i]);
+  return t;
+}
+
+static void table_drop(mt_table* t) {
+  if (t->table) cudaFree(t->table);
+  if (t->class_masks) cudaFree(t->class_masks);
+  if (t->xclass) cudaFree(t->xclass);
+  if (t->xmap) cudaFree(t->xmap);
+  delete t;
 }
 
 static mt_status build_table(int k, cudaStream_t s, mt_table** out) {
   const uint64_t nkeys = 1ull << (k * (k - 1));
-  const size_t nwords = (size_t)std::max<uint64_t>(nkeys / 32, 1);
-  std::vector<uint8_t> seq = sjt_sequence(k);
-  {  // the walk must visit every ordering exactly once
-    std::vector<int> p(k);
-    std::iota(p.begin(), p.end(), 0);
-    std::vector<std::vector<int>> seen{p};
-    for (uint8_t q : seq) {
-      std::swap(p[q], p[q + 1]);
-      seen.push_back(p);
-    }
-    std::sort(seen.begin(), seen.end());
-    size_t fact = 1;
-    for (int i = 2; i <= k; ++i) fact *= i;
-    if (seq.size() + 1 != fact || std::unique(seen.begin(), seen.end()) != seen.end())
-      return MT_ECUDA;
-  }
-  MT_CUDA_TRY(cudaMemcpyToSymbolAsync(c_sjt, seq.data(), seq.size(), 0, cudaMemcpyHostToDevice, s));
-
+  int nsteps = 0, nsteps5 = 0;
+  MT_TRY(upload_sjt(k, s, &nsteps));
+  if (k == 6) MT_TRY(upload_sjt(5, s, &nsteps5));
   mt_table* t = new mt_table();
   t->k = k;
   t->nkeys = nkeys;
   t->classes = kNumClasses[k];
-  uint32_t* bitmap = nullptr;
-  int32_t* prefix = nullptr;
-  int32_t* tiles = nullptr;
-  const size_t ntiles = (nwords + kScanTile - 1) / kScanTile;
+  TableScratch x;
   cudaError_t e = cudaMalloc(&t->table, nkeys * 4);
   if (e == cudaSuccess) e = cudaMalloc(&t->class_masks, (size_t)t->classes * 4);
-  if (e == cudaSuccess) e = cudaMallocAsync(&bitmap, nwords * 4, s);
-  if (e == cudaSuccess) e = cudaMallocAsync(&prefix, nwords * 4, s);
-  if (e == cudaSuccess) e = cudaMallocAsync(&tiles, ntiles * 4, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(bitmap, 0, nwords * 4, s);
+  if (e == cudaSuccess) e = scratch_alloc(&x, k, s);
   if (e == cudaSuccess) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sm_count();
     const int grid = (int)std::min<uint64_t>((nkeys + 255) / 256, (uint64_t)sms * 16);
-    const int nsteps = (int)seq.size();
-    switch (k) {
-      case 3: k_canon<3><<<grid, 256, 0, s>>>(t->table, bitmap, nkeys, nsteps); break;
-      case 4: k_canon<4><<<grid, 256, 0, s>>>(t->table, bitmap, nkeys, nsteps); break;
-      case 5: k_canon<5><<<grid, 256, 0, s>>>(t->table, bitmap, nkeys, nsteps); break;
-      default: k_canon<6><<<grid, 256, 0, s>>>(t->table, bitmap, nkeys, nsteps); break;
+    if (k == 6) {
+      e = launch_sub6(x, t->class_masks, nsteps5, nsteps, sms, s);
+      if (e == cudaSuccess)
+        k_expand<<<sms * 8, 256, 0, s>>>(t->table, x.sub, x.class5, x.sigma, nullptr, kP5Keys);
+    } else {
+      switch (k) {
+        case 3: k_canon<3><<<grid, 256, 0, s>>>(t->table, x.bitmap, nkeys, nsteps); break;
+        case 4: k_canon<4><<<grid, 256, 0, s>>>(t->table, x.bitmap, nkeys, nsteps); break;
+        default: k_canon<5><<<grid, 256, 0, s>>>(t->table, x.bitmap, nkeys, nsteps); break;
+      }
+      e = launch_rank(x.bitmap, x.ngroups, x.tiles, x.prefix, s);
+      const uint4* bits = (const uint4*)x.bitmap;
+      k_assign<<<grid, 256, 0, s>>>(t->table, nkeys, bits, x.prefix);
+      k_bit_list<<<(unsigned)((x.ngroups + 255) / 256), 256, 0, s>>>(
+          bits, x.ngroups, x.prefix, t->class_masks, t->classes);
     }
-    e = cudaGetLastError();
-    if (e == cudaSuccess) {
-      k_tile_popc<<<(unsigned)ntiles, kScanThreads, 0, s>>>(bitmap, nwords, tiles);
-      k_scan_single<<<1, 1024, 0, s>>>(tiles, (int)ntiles);
-      k_tile_prefix<<<(unsigned)ntiles, kScanThreads, 0, s>>>(bitmap, nwords, tiles, prefix);
-      k_assign<<<grid, 256, 0, s>>>(t->table, nkeys, bitmap, prefix);
-      const int g2 = (int)std::min<size_t>((nwords + 255) / 256, (size_t)sms * 8);
-      k_class_list<<<g2, 256, 0, s>>>(bitmap, nwords, prefix, t->class_masks, t->classes);
-      e = cudaGetLastError();
-    }
+    if (e == cudaSuccess) e = cudaGetLastError();
   }
-  // the number of connected canonical masks must equal the closed-form count
-  int32_t last_prefix = 0;
-  uint32_t last_word = 0;
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&last_prefix, prefix + nwords - 1, 4, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&last_word, bitmap + nwords - 1, 4, cudaMemcpyDeviceToHost, s);
-  if (bitmap) cudaFreeAsync(bitmap, s);
-  if (prefix) cudaFreeAsync(prefix, s);
-  if (tiles) cudaFreeAsync(tiles, s);
+  // the numbers of canonical masks must equal the closed-form counts
+  uint32_t got[5] = {0}, got5[5] = {0};
+  if (e == cudaSuccess) e = read_total(x.bitmap, x.prefix, x.ngroups, got, s);
+  if (e == cudaSuccess && k == 6) e = read_total(x.bitmap5, x.prefix5, x.ngroups5, got5, s);
+  if (x.mem) cudaFreeAsync(x.mem, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
     set_last_error(cudaGetErrorString(e));
-    if (t->table) cudaFree(t->table);
-    if (t->class_masks) cudaFree(t->class_masks);
-    delete t;
+    table_drop(t);
     return e == cudaErrorMemoryAllocation ? MT_ENOMEM : MT_ECUDA;
   }
-  const uint32_t found = (uint32_t)last_prefix + (uint32_t)__builtin_popcount(last_word);
-  if (found != t->classes) {
-    set_last_error("table builder found " + std::to_string(found) + " classes");
-    cudaFree(t->table);
-    cudaFree(t->class_masks);
-    delete t;
+  if (total_of(got) != t->classes || (k == 6 && total_of(got5) != kP5Classes)) {
+    set_last_error("table builder found " + std::to_string(total_of(got)) + " classes");
+    table_drop(t);
     return MT_ECUDA;
   }
   *out = t;
@@ -390,70 +621,67 @@ __global__ void k_xreps(const uint32_t* xbits, const int32_t* xrep, int32_t* rep
     if ((xbits[c >> 5] >> (c & 31u)) & 1u) reps[r++] = xrep[c];
 }
 
-// compact[c << 18 | low] = full[rep(c) << 18 | low]
-__global__ void k_xgather(const uint32_t* full, const int32_t* reps, uint32_t* compact) {
-  const uint64_t n = (uint64_t)kXClasses << kXLow;
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint32_t c = (uint32_t)(i >> kXLow), low = (uint32_t)(i & ((1u << kXLow) - 1u));
-    compact[i] = full[((uint64_t)reps[c] << kXLow) | low];
-  }
-}
-
 static mt_status build_compact6(cudaStream_t s, mt_table** out) {
-  mt_table* full = nullptr;
-  MT_TRY(build_table(6, s, &full));
+  int nsteps = 0, nsteps5 = 0;
+  MT_TRY(upload_sjt(6, s, &nsteps));
+  MT_TRY(upload_sjt(5, s, &nsteps5));
   mt_table* t = new mt_table();
   t->k = 6;
-  t->classes = full->classes;
-  t->class_masks = full->class_masks;
-  full->class_masks = nullptr;
+  t->classes = kNumClasses[6];
   t->compact = true;
   t->nkeys = (uint64_t)kXClasses << kXLow;
+  TableScratch x;
   uint16_t* xcanon = nullptr;
   uint8_t* xsigma = nullptr;
   uint32_t* xbits = nullptr;
-  int32_t *xrep = nullptr, *reps = nullptr;
+  int32_t* xrep = nullptr;
   cudaError_t e = cudaMalloc(&t->table, t->nkeys * 4);
+  if (e == cudaSuccess) e = cudaMalloc(&t->class_masks, (size_t)t->classes * 4);
   if (e == cudaSuccess) e = cudaMalloc(&t->xclass, kXKeys * 2);
   if (e == cudaSuccess) e = cudaMalloc(&t->xmap, kXKeys * 256);
+  if (e == cudaSuccess) e = scratch_alloc(&x, 6, s);
   if (e == cudaSuccess) e = cudaMallocAsync(&xcanon, kXKeys * 2, s);
   if (e == cudaSuccess) e = cudaMallocAsync(&xsigma, kXKeys, s);
   if (e == cudaSuccess) e = cudaMallocAsync(&xbits, kXKeys / 8, s);
   if (e == cudaSuccess) e = cudaMallocAsync(&xrep, kXKeys * 4, s);
-  if (e == cudaSuccess) e = cudaMallocAsync(&reps, kXClasses * 4, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(xbits, 0, kXKeys / 8, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(reps, 0, kXClasses * 4, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(x.reps, 0, kXClasses * 4, s);
   int32_t nreps = 0;
   if (e == cudaSuccess) {
+    const int sms = sm_count();
+    e = launch_sub6(x, t->class_masks, nsteps5, nsteps, sms, s);
     k_xprefix<<<kXKeys / 256, 256, 0, s>>>(xcanon, xsigma, xbits, xrep);
     k_xtables<<<kXKeys, 256, 0, s>>>(xcanon, xsigma, xbits, t->xclass, t->xmap);
-    k_xreps<<<1, 32, 0, s>>>(xbits, xrep, reps);
-    k_xgather<<<1024, 256, 0, s>>>(full->table, reps, t->table);
-    e = cudaGetLastError();
+    k_xreps<<<1, 32, 0, s>>>(xbits, xrep, x.reps);
+    if (e == cudaSuccess)
+      k_expand<<<sms * 8, 256, 0, s>>>(t->table, x.sub, x.class5, x.sigma, x.reps,
+                                       (uint32_t)kXClasses << (kXLow - kP5Low));
+    if (e == cudaSuccess) e = cudaGetLastError();
   }
-  // the number of connected 4-vertex classes must be 199
+  // the numbers of classes: connected 4-vertex, all 5-vertex, connected 6-vertex
+  uint32_t got[5] = {0}, got5[5] = {0};
   std::vector<uint32_t> hb(kXKeys / 32);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(hb.data(), xbits, kXKeys / 8, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = read_total(x.bitmap, x.prefix, x.ngroups, got, s);
+  if (e == cudaSuccess) e = read_total(x.bitmap5, x.prefix5, x.ngroups5, got5, s);
   if (xcanon) cudaFreeAsync(xcanon, s);
   if (xsigma) cudaFreeAsync(xsigma, s);
   if (xbits) cudaFreeAsync(xbits, s);
   if (xrep) cudaFreeAsync(xrep, s);
-  if (reps) cudaFreeAsync(reps, s);
+  if (x.mem) cudaFreeAsync(x.mem, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   for (uint32_t w : hb) nreps += __builtin_popcount(w);
-  cudaFree(full->table);
-  delete full;
-  if (e != cudaSuccess || nreps != kXClasses) {
-    if (e != cudaSuccess) set_last_error(cudaGetErrorString(e));
-    else set_last_error("compact table: " + std::to_string(nreps) + " prefix classes");
-    cudaFree(t->table);
-    cudaFree(t->class_masks);
-    cudaFree(t->xclass);
-    cudaFree(t->xmap);
-    delete t;
+  if (e != cudaSuccess) {
+    set_last_error(cudaGetErrorString(e));
+    table_drop(t);
     return e == cudaErrorMemoryAllocation ? MT_ENOMEM : MT_ECUDA;
+  }
+  if (nreps != kXClasses || total_of(got) != t->classes || total_of(got5) != kP5Classes) {
+    set_last_error("compact table: " + std::to_string(nreps) + " prefix classes, " +
+                   std::to_string(total_of(got)) + " classes");
+    table_drop(t);
+    return MT_ECUDA;
   }
   *out = t;
   return MT_OK;

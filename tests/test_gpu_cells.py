@@ -1,0 +1,50 @@
+"""The cell method where its branches change: more distinct cells than it
+numbers, rows longer than a lane's segments, hubs, lists that fill batches
+exactly, against per-subgraph classification of the same graph (itself checked
+against the oracle elsewhere).  GPU only."""
+import numpy as np
+import pytest
+
+import synthetic as syn
+
+pytestmark = pytest.mark.gpu
+
+
+def _hub(n, d, m, seed):
+    """A vertex adjacent to d others (ids on both sides of it) in a sparse background."""
+    rng = np.random.default_rng(seed)
+    hub = n // 3
+    others = rng.choice(np.delete(np.arange(n), hub), d, replace=False)
+    key = {(hub, int(o)) if i % 3 else (int(o), hub) for i, o in enumerate(others)}
+    while len(key) < d + m:
+        a, b = (int(x) for x in rng.integers(0, n, 2))
+        if a != b and a != hub and b != hub:
+            key.add((a, b))
+    a = np.array(sorted(key))
+    return syn.csr_from_arcs(n, a[:, 0], a[:, 1])
+
+
+GRAPHS = {
+    "dense100": lambda: syn.random_small_digraph(100, 0.35, 0.4, 3),   # > 64 cells at k = 6
+    "dense64": lambda: syn.random_small_digraph(64, 0.5, 0.2, 4),
+    "complete33": lambda: syn.complete_digraph(33),                    # lists of 32 and fewer
+    "hub": lambda: _hub(700, 260, 900, 5),
+    "hub_rows": lambda: _hub(400, 97, 1500, 6),
+    "power": lambda: syn.chung_lu_digraph(500, 2200, 2.1, None, 0.2, 7),
+}
+
+
+@pytest.mark.parametrize("k,name", [(k, g) for g in GRAPHS for k in (3, 4, 5, 6)
+                                    if not (k == 6 and g in ("hub", "power"))])
+def test_cells_equal_per_subgraph_counts(lib, k, name):
+    lib.load_library()
+    t = lib.table_build(k)
+    dg = lib.graph_from(GRAPHS[name]())
+    want = lib.to_numpy_u64(lib.count_tuned(dg, t, method=lib.METHOD_ENUMERATE))
+    assert lib.count_stats(dg)[1] == 0
+    for wpb in (0, 3):
+        got = lib.to_numpy_u64(lib.count_tuned(dg, t, warps_per_block=wpb,
+                                               method=lib.METHOD_CELLS))
+        assert lib.count_stats(dg)[1] == 0
+        np.testing.assert_array_equal(got, want)
+    t.free()

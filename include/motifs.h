@@ -140,10 +140,9 @@ mt_status mt_table_build(int k, void* stream, mt_table** out);
  * fifth is not), which leaves the class of the whole unchanged.  Slot
  * (class of X) << 18 | relabelled fifth word << 10 | relabelled sixth word
  * holds the dense id.  Scratch while it builds: about 220 MB, freed before
- * return.  Class ids and class masks are the
- * full table's.  Counting with a compact table supports the per-subgraph
- * method only (MT_METHOD_CELLS gives MT_EUNSUPPORTED); mt_table_entries reads
- * compact slots.  Synchronises `stream`.
+ * return.  Class ids and class masks are the full table's.  With a compact
+ * table an explicit MT_METHOD_CELLS gives MT_EUNSUPPORTED; mt_table_entries
+ * reads compact slots.  Synchronises `stream`.
  * Errors: MT_EUNSUPPORTED (k != 6), MT_ENOMEM, MT_ECUDA. */
 mt_status mt_table_build_compact(int k, void* stream, mt_table** out);
 
@@ -174,7 +173,10 @@ mt_status mt_table_entries(const mt_table* t, uint64_t first, uint64_t count, ui
  * connected set is produced exactly once by the extension enumerator (root =
  * smallest vertex, extension by exclusive neighbours), its adjacency bits are
  * gathered from the labelled neighbour rows (the row-scan strategy of Sec. 3.1)
- * and classified by one table read (Sec. 3.2).  n < k gives all zeros.
+ * and classified by one table read (Sec. 3.2); at k = 5 and 6, and at k = 4 on
+ * large graphs, the last two vertices are counted per pair of cells instead
+ * (Algorithm 1 of Sec. 3; see mt_method), with the same result.  n < k gives
+ * all zeros.
  * The call may grow device scratch memory held by the graph handle.  At k = 6
  * that scratch includes 7 extra copies of the histogram (12 MB each): the
  * count spreads its thread blocks over 8 copies, so that fewer blocks add into
@@ -200,7 +202,10 @@ mt_status mt_count_roots(const mt_graph* g, const mt_table* t, int32_t root_begi
                          int32_t root_end, uint64_t* hist, void* stream);
 
 /* Counting method.
- * MT_METHOD_ENUMERATE (default): every connected k-set is produced and its class
+ * Calls without an mt_tuning (or with a null one) and servers whose method was
+ * not set use the faster of the two for k and the graph's size; the value of
+ * mt_tuning.method is always followed.
+ * MT_METHOD_ENUMERATE (0): every connected k-set is produced and its class
  *   read from the table (per-subgraph classification, Sec. 3.2).
  * MT_METHOD_CELLS: the enumeration stops at (k-2)-sets X; the k-sets X + {y, z}
  *   are counted per pair of cells of Part(adj(X)) (Sec. 2) with one table read
@@ -452,7 +457,8 @@ mt_status mt_server_result(mt_server* s, uint64_t id, int32_t* state, uint64_t* 
                            double* latency_ms);
 
 /* Counting method of the rounds launched from now on (an mt_method; the
- * default is MT_METHOD_ENUMERATE).  Results do not depend on it. */
+ * default is the faster one for each k and size, see mt_method).  Results do
+ * not depend on it. */
 mt_status mt_server_set_method(mt_server* s, int method);
 
 /* Device bytes currently charged against the budget by active requests. */

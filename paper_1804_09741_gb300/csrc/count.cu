@@ -36,8 +36,9 @@
 //    three choices at a time instead (see kWideTailBlocksPerGraph); at k = 6,
 //    short candidate lists let several choices share one pass, a (choice,
 //    candidate) pair per lane;
-//  * MT_METHOD_CELLS stops one level earlier and counts the last two vertices
-//    per pair of cells (Algorithm 1 of Sec. 3; see pair_level below);
+//  * MT_METHOD_CELLS, the automatic choice at k = 5 and 6, stops one level
+//    earlier and counts the last two vertices per pair of cells (Algorithm 1 of
+//    Sec. 3; see pair_level below);
 //  * histograms: per-block shared-memory 32-bit counters for k <= 5 (13 / 199
 //    / 9,364 classes), the graph's 64-bit global counters for k = 6 (a
 //    one-graph count spreads its blocks over kHistCopies copies of them and
@@ -1346,24 +1347,12 @@ static const void* pick_kernel(int K, bool gc, bool ls, bool cb, bool sg) {
   }
 }
 
-mt_status count_configure(CountPlan* p, int K, int G, int nmax, int dmax, int64_t fwd_bound,
-                          int64_t entry_stride, uint32_t classes, double split_cost,
-                          int warps_per_block, bool compact) {
-  mt_tuning t;
-  t.split_cost = split_cost;
-  t.split_scale = 0.0;
-  t.warps_per_block = warps_per_block;
-  t.stack_cap = 0;
-  t.method = MT_METHOD_ENUMERATE;
-  const bool plain = split_cost == 0.0;
-  MT_TRY(count_configure_tuned(p, K, G, nmax, dmax, fwd_bound, entry_stride, classes,
-                               plain && warps_per_block == 0 ? nullptr : &t, compact));
-  return MT_OK;
-}
+constexpr int kCellsAboveK4 = 4096;  // k = 4: vertices above which cells are faster
 
 mt_status count_configure_tuned(CountPlan* p, int K, int G, int nmax, int dmax, int64_t fwd_bound,
                                 int64_t entry_stride, uint32_t classes, const mt_tuning* tuning,
-                                bool compact) {
+                                bool compact, int method) {
+  if (tuning) method = tuning->method;
   if (K < 3 || K > 6 || G < 1 || nmax < 1) return MT_EINVAL;
   const double split_cost = tuning ? tuning->split_cost : 0.0;
   const int warps_per_block = tuning ? tuning->warps_per_block : 0;
@@ -1384,9 +1373,20 @@ mt_status count_configure_tuned(CountPlan* p, int K, int G, int nmax, int dmax, 
                                              : std::max(K - 2, 1) * std::max(dmax, 1) + 32;
   if (p->cap > 65535) return MT_EUNSUPPORTED;
   p->nu_cap = (int)p->entry_stride;
-  p->comb = tuning && tuning->method == MT_METHOD_CELLS;
+  // The library's own choice: the cell method where it is the faster one (it
+  // counts the same histogram from the (k-2)-sets instead of from every k-set).
+  // Measured on a GB300, per-subgraph against cells: one k = 6 graph (n = 800)
+  // 4.6 : 1.6 ms and 65 of them 135 : 71 ms, one k = 5 graph (n = 1,500) 2.7 :
+  // 1.3 ms and 257 of them 526 : 187 ms, small graphs at k = 5 (n = 112 to 310)
+  // 1.1 to 1.2 times faster; k = 4 at n = 6,437 0.94 : 0.69 ms but at n = 3,646
+  // 0.64 : 0.68 and at n = 2,000 0.39 : 0.45 ms; at k = 3 a few per cent slower.
+  if (method == kAutoMethod)
+    method = K >= 5 || (K == 4 && nmax > kCellsAboveK4) ? MT_METHOD_CELLS : MT_METHOD_ENUMERATE;
+  else if (compact && method == MT_METHOD_CELLS)
+    return MT_EUNSUPPORTED;
+  p->comb = method == MT_METHOD_CELLS;
   p->compact = compact;
-  if (compact && (K != 6 || p->comb)) return MT_EUNSUPPORTED;
+  if (compact && K != 6) return MT_EUNSUPPORTED;
   p->map_bytes = compact ? 256 : 0;
   const size_t lab_elem = (K <= 4 || (p->comb && K <= 5)) ? 1 : ((K == 5 || p->comb) ? 2 : 4);
   const size_t lab_bytes = round16((size_t)nmax * lab_elem);

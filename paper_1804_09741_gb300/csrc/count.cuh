@@ -44,16 +44,14 @@ struct CountPlan {
 
 // Fill in the launch shape and the workspace size.  `fwd_bound` is a bound on
 // the total number of forward entries (sum of undirected edges) of the G graphs.
-mt_status count_configure(CountPlan* p, int K, int G, int nmax, int dmax, int64_t fwd_bound,
-                          int64_t entry_stride, uint32_t classes, double split_cost,
-                          int warps_per_block, bool compact = false);
-
-// Same, with the tuning of include/motifs.h (nullptr = automatic).
-// `compact`: the table is the compact k = 6 form (per-subgraph method only;
-// MT_EUNSUPPORTED otherwise).
+// `tuning` as in include/motifs.h (nullptr = automatic, with the
+// counting method `method`: an mt_method, or kAutoMethod for the library's
+// choice).  `compact`: the table is the compact k = 6 form (an explicit
+// MT_METHOD_CELLS is then MT_EUNSUPPORTED).
+constexpr int kAutoMethod = -1;
 mt_status count_configure_tuned(CountPlan* p, int K, int G, int nmax, int dmax, int64_t fwd_bound,
                                 int64_t entry_stride, uint32_t classes, const mt_tuning* tuning,
-                                bool compact = false);
+                                bool compact = false, int method = kAutoMethod);
 
 // Enqueue planner + enumerator.  `graphs` is a device array of G DevGraph whose
 // hist pointers are already zeroed (the launch adds into them).  Roots in

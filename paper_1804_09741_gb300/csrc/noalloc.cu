@@ -78,11 +78,16 @@ static mt_status count_noalloc(const mt_graph* g, const mt_table* t, uint64_t* h
   MT_TRY(scratch_address(&scratch));
   const int K = table_k(t);
   const uint32_t C = table_classes(t);
+  // the automatic launch, or per-subgraph classification where only that fits
   CountPlan p;
-  MT_TRY(count_configure(&p, K, 1, g->n, g->dmax, g->nu / 2 + 1, g->nu > 0 ? g->nu : 1, C, 0.0, 0,
-                         table_compact(t)));
-  const size_t desc_off = (p.ws_bytes + 255) & ~(size_t)255;
-  const size_t need = desc_off + 256;
+  size_t desc_off = 0, need = 0;
+  for (const int method : {kAutoMethod, (int)MT_METHOD_ENUMERATE}) {
+    MT_TRY(count_configure_tuned(&p, K, 1, g->n, g->dmax, g->nu / 2 + 1, g->nu > 0 ? g->nu : 1, C,
+                                 nullptr, table_compact(t), method));
+    desc_off = (p.ws_bytes + 255) & ~(size_t)255;
+    need = desc_off + 256;
+    if (need <= kNoAllocScratchBytes) break;
+  }
   if (need > kNoAllocScratchBytes) {
     set_last_error("mt_count_noalloc: this graph needs " + std::to_string(need) +
                    " bytes of scratch; the fixed scratch holds " +

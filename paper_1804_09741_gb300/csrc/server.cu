@@ -92,7 +92,7 @@ struct mt_server {
   size_t reserved[4] = {0, 0, 0, 0};  // round scratch charged to the budget, per k
   std::vector<uint64_t*> pinned_free[4];  // result buffers by k
   std::chrono::steady_clock::time_point t0;
-  int method = MT_METHOD_ENUMERATE;
+  int method = mt::kAutoMethod;
 };
 
 namespace mt {
@@ -155,16 +155,9 @@ static mt_status plan_for(const mt_server* s, int ki, const SrvRequest* extra, C
   if (extra) add(extra);
   *G = g;
   if (g == 0) return MT_OK;
-  mt_tuning tun;
-  tun.split_cost = 0.0;
-  tun.split_scale = 0.0;
-  tun.warps_per_block = 0;
-  tun.stack_cap = 0;
-  tun.method = s->method;
   return count_configure_tuned(p, ki + 3, g, nmax, dmax, fwd, numax,
-                               table_classes(s->tables[ki]),
-                               s->method == MT_METHOD_ENUMERATE ? nullptr : &tun,
-                               table_compact(s->tables[ki]));
+                               table_classes(s->tables[ki]), nullptr,
+                               table_compact(s->tables[ki]), s->method);
 }
 
 // Round scratch of k's launch (planner and work queue, graph descriptors) for
@@ -417,15 +410,8 @@ static mt_status step(mt_server* s, int32_t* completed) {
         fwd += c.r->g->nu / 2 + 1;
       }
       CountPlan p;
-      mt_tuning tun;
-      tun.split_cost = 0.0;
-      tun.split_scale = 0.0;
-      tun.warps_per_block = 0;
-      tun.stack_cap = 0;
-      tun.method = s->method;
-      mt_status cst =
-          count_configure_tuned(&p, K, (int)chunks.size(), nmax, dmax, fwd, numax, C,
-                                s->method == MT_METHOD_ENUMERATE ? nullptr : &tun, table_compact(t));
+      mt_status cst = count_configure_tuned(&p, K, (int)chunks.size(), nmax, dmax, fwd, numax, C,
+                                            nullptr, table_compact(t), s->method);
       if (cst == MT_OK) cst = ensure_capacity(s, ki, p.ws_bytes, chunks.size());
       if (cst == MT_OK)  // charge what is held, should the plan outgrow the reservation
         s->reserved[ki] = std::max(s->reserved[ki],

@@ -5,7 +5,9 @@ against the oracle elsewhere).  GPU only."""
 import numpy as np
 import pytest
 
+import oracle
 import synthetic as syn
+from gpu_helpers import oracle_dense
 
 pytestmark = pytest.mark.gpu
 
@@ -47,4 +49,30 @@ def test_cells_equal_per_subgraph_counts(lib, k, name):
                                                method=lib.METHOD_CELLS))
         assert lib.count_stats(dg)[1] == 0
         np.testing.assert_array_equal(got, want)
+    t.free()
+
+
+@pytest.mark.parametrize("k", [3, 4, 5, 6])
+def test_per_subgraph_counts_equal_oracle(lib, k):
+    """The per-subgraph method asked for by name (calls without a tuning take
+    the faster method for their k and size)."""
+    lib.load_library()
+    t = lib.table_build(k)
+    for g in (syn.random_small_digraph(24, 0.18, 0.3, k),
+              syn.chung_lu_digraph(150, 500, 2.2, None, 0.15, k)):
+        dg = lib.graph_from(g)
+        h = lib.to_numpy_u64(lib.count_tuned(dg, t, method=lib.METHOD_ENUMERATE))
+        assert lib.count_stats(dg)[1] == 0
+        np.testing.assert_array_equal(h, oracle_dense(oracle.count(g, k)[0], t.class_masks()))
+    t.free()
+
+
+@pytest.mark.parametrize("n", [4096, 4097])
+def test_automatic_method_around_its_line(lib, n):
+    """k = 4 changes method above 4,096 vertices: both sides equal the oracle."""
+    lib.load_library()
+    t = lib.table_build(4)
+    g = syn.chung_lu_digraph(n, 2 * n, 2.4, 60, 0.1, 9)
+    want = oracle_dense(oracle.count(g, 4)[0], t.class_masks())
+    np.testing.assert_array_equal(lib.count_host(lib.graph_from(g), t), want)
     t.free()

@@ -16,15 +16,13 @@
 namespace mt {
 cudaError_t launch_randomize(int32_t n, int32_t m, int G, const int32_t* row_ptr,
                              const int32_t* col0, const uint64_t* seeds, uint64_t swaps,
-                             int32_t* col_out, uint32_t* gscratch, int64_t* accepted,
-                             cudaStream_t s);
+                             int32_t* col_out, uint32_t* gscratch, cudaStream_t s);
 size_t rand_gscratch_words(int32_t m, int G);
 cudaError_t launch_randomize_dyads(int32_t n, int32_t m, int G, const int32_t* row_ptr,
                                    const int32_t* col0, const uint64_t* seeds, uint64_t attempts,
                                    int32_t* col_out, int32_t* scratch, uint32_t* gscratch,
-                                   int64_t* accepted, cudaStream_t s);
+                                   cudaStream_t s);
 size_t dyad_scratch_ints(int32_t n, int32_t m);
-size_t rand_smem_bytes(int32_t m);
 }  // namespace mt
 
 struct mt_batch {
@@ -218,10 +216,10 @@ static mt_status batch_enqueue(mt_batch* b, cudaStream_t s) {
   MT_CUDA_TRY(cudaEventRecordWithFlags(b->ev[0], s, cudaEventRecordExternal));
   if (b->null_model == MT_NULL_DYAD_SWAP)
     MT_CUDA_TRY(launch_randomize_dyads(n, m, R, b->g0->row_ptr, b->g0->col, b->d_seeds, b->swaps,
-                                       b->col_rand, b->dyad_scratch, b->rand_scratch, nullptr, s));
+                                       b->col_rand, b->dyad_scratch, b->rand_scratch, s));
   else
     MT_CUDA_TRY(launch_randomize(n, m, R, b->g0->row_ptr, b->g0->col, b->d_seeds, b->swaps,
-                                 b->col_rand, b->rand_scratch, nullptr, s));
+                                 b->col_rand, b->rand_scratch, s));
   BuildArgs a;
   a.n = n; a.m = m; a.G = R;
   a.row_ptr = b->g0->row_ptr; a.row_stride = 0;

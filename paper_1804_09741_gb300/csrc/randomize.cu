@@ -9,35 +9,36 @@
 // only the destinations move, and the builder re-sorts the rows afterwards.
 //
 // GPU mapping: one thread block per graph.  The arc array (src<<16 | dst) and a
-// bucketed hash set of the present arcs sit in shared memory (global memory
-// for graphs too large for it); the block fills them in parallel.  Then warp
-// 0 runs the attempts 32 at a time, lane j taking attempt t0 + j:
-//  * speculation: every lane evaluates its attempt against the state at the
-//    start of the batch (the two arcs at its positions, the checks, whether
-//    the two new arcs are present, where the two old ones and free slots for
-//    the new ones are);
+// hash set of the present arcs sit in shared memory (global memory for graphs
+// too large for it); the block fills them in parallel.  Then 256 threads run
+// the attempts in windows of 64, four threads per attempt (one per arc that it
+// looks up or replaces), while two warps draw the next attempts' positions,
+// which do not depend on the graph:
+//  * speculation: every attempt is evaluated against the state at the start of
+//    the window (the two arcs at its positions, the checks, whether the two new
+//    arcs are present);
 //  * resolution: an attempt's speculative outcome is its sequential outcome
-//    unless an earlier attempt of the batch that the speculation accepted
-//    wrote one of its two positions, inserted or erased one of the two arcs it
-//    looks up, or would fill the same free slot (a new key takes the first free
-//    slot of its bucket at or after one picked by the key's low bits, so
-//    attempts sharing a bucket rarely pick the same).  Every lane checks this
-//    against all earlier lanes at once; the attempts before the first unsafe
-//    one are applied together (their writes are disjoint), the unsafe one is
-//    evaluated on the current state by the whole warp, which looks up its four
-//    arcs in one round of shared-memory loads (eight lanes per arc read its
-//    32-slot bucket, a ballot finds the key or a free slot), and the next
-//    batch starts after it.  The outcome is that of the attempts run one after
-//    another.
+//    unless an earlier attempt of the window that the speculation accepted wrote
+//    one of its two positions, or inserted or erased one of the two arcs it
+//    looks up.  Accepted attempts set their bit in two small tables hashed by
+//    position and by arc; an attempt reads the bits of its own four entries and
+//    compares itself with the earlier attempts it finds there, so hash
+//    collisions cost a comparison and no lost attempt;
+//  * the attempts before the first unsafe one are applied together (their
+//    positions and arcs are disjoint), and the next window starts at it.
+// The outcome is that of the attempts run one after another.  What bounds it is
+// the latency of one window after another: at m = 6,000 a window passes 44.5
+// attempts (two attempts of a window overlap with probability about 4 / m; 128
+// wide it would pass 50) and takes 1.5 us.  One graph of m = 6,000, 60,000
+// attempts: 7.2 ms with one warp, 32 attempts and bucket scans by every lane,
+// 2.3 ms now; 511 graphs of m = 1,500: 6.0 -> 1.5 ms.
 //
-// Bucketed set: 2^bb buckets of 32 slots (at least 2 slots per stored key,
-// so a bucket holds 16 on average); a key lives in the first bucket of its
-// probe sequence (home bucket, then the next ones) that had a free slot when it
-// was inserted, and a bucket that was ever found full keeps a sticky
-// "overflowed" flag, so a lookup moves on to the next bucket only past flagged
-// ones.  Erasing empties the slot; flags stay.  Only membership matters to the
-// attempts, not where a key is stored, so the results are those of the
-// sequential definition.
+// Set: 2^bb buckets of 8 slots (two 16-byte reads), 2 to 4 keys per bucket on
+// average; a key lives in the first bucket of its probe sequence (home bucket,
+// then the next ones) that had a free slot when it was inserted, and every
+// bucket counts the keys that passed over it, so a lookup moves on only past
+// buckets with a count.  Only membership matters to the attempts, not where a
+// key is stored, so the results are those of the sequential definition.
 //
 // SplitMix64 (Steele, Lea and Flood, OOPSLA 2014, public-domain reference
 // generator): state advances by the golden gamma 0x9E3779B97F4A7C15, output =
@@ -57,276 +58,276 @@ __device__ __forceinline__ uint64_t sm64_mix(uint64_t z) {
 }
 
 // Layout of one graph's randomiser state (in 32-bit words): the entry array
-// (arcs, or the dyad lists) padded to 4 words, the buckets, the overflow flags.
+// (arcs, or the dyad lists) padded to 4 words, the buckets, their counts (16
+// bits each).
 struct RandLayout {
   int bb;          // log2 of the number of buckets (>= 1)
   size_t t_off;    // first slot
-  size_t f_off;    // first flag word
+  size_t c_off;    // first count word
   size_t words;    // total
 };
 
 __host__ __device__ inline RandLayout rand_layout(int32_t m) {
   RandLayout L;
   int bb = 1;
-  while ((32ll << bb) < 2ll * (m > 0 ? m : 1)) ++bb;  // >= 2 slots per stored key
+  while ((4ll << bb) < (m > 0 ? m : 1)) ++bb;  // at most 4 keys per bucket on average
   L.bb = bb;
   L.t_off = ((size_t)(m > 0 ? m : 1) + 3) & ~(size_t)3;
-  L.f_off = L.t_off + ((size_t)32 << bb);
-  const size_t nflag = ((size_t)1 << bb) > 32 ? ((size_t)1 << bb) / 32 : 1;
-  L.words = (L.f_off + nflag + 3) & ~(size_t)3;
+  L.c_off = L.t_off + ((size_t)8 << bb);
+  L.words = (L.c_off + ((size_t)1 << bb) / 2 + 3) & ~(size_t)3;
   return L;
 }
 
-// The free slot of `free_mask` at or after slot r (cyclically), or -1.
-__device__ __forceinline__ int free_slot_from(unsigned free_mask, int r) {
-  if (!free_mask) return -1;
-  const unsigned rot = r ? (free_mask >> r) | (free_mask << (32 - r)) : free_mask;
-  return (__ffs(rot) - 1 + r) & 31;
+// Reads of the state: another thread of the block may have written it, and the
+// set's global-memory form is updated by atomics, so that form reads past L1.
+template <bool GM, typename T>
+__device__ __forceinline__ T state_read(const T* p) {
+  return GM ? __ldcg(p) : *p;
 }
 
+// A bucket's 8 slots.
+struct BucketRow {
+  uint4 a, b;
+  __device__ __forceinline__ bool has(uint32_t key) const {
+    return a.x == key || a.y == key || a.z == key || a.w == key || b.x == key || b.y == key ||
+           b.z == key || b.w == key;
+  }
+  // bits of the slots holding `key`
+  __device__ __forceinline__ unsigned mask(uint32_t key) const {
+    return (a.x == key ? 1u : 0u) | (a.y == key ? 2u : 0u) | (a.z == key ? 4u : 0u) |
+           (a.w == key ? 8u : 0u) | (b.x == key ? 16u : 0u) | (b.y == key ? 32u : 0u) |
+           (b.z == key ? 64u : 0u) | (b.w == key ? 128u : 0u);
+  }
+  // index of the first slot holding `key`, or -1
+  __device__ __forceinline__ int find(uint32_t key) const {
+    int at = -1;
+    if (b.w == key) at = 7;
+    if (b.z == key) at = 6;
+    if (b.y == key) at = 5;
+    if (b.x == key) at = 4;
+    if (a.w == key) at = 3;
+    if (a.z == key) at = 2;
+    if (a.y == key) at = 1;
+    if (a.x == key) at = 0;
+    return at;
+  }
+};
+
+template <bool GM>
 struct BucketSet {
-  uint32_t* t;     // (1 << bb) x 32 slots
-  uint32_t* flag;  // overflow bits, one per bucket
+  uint32_t* t;     // (1 << bb) x 8 slots
+  uint32_t* cnt;   // keys that passed over each bucket, two 16-bit counts per word
   int bb;
   uint32_t bmask;
-  __device__ uint32_t home(uint32_t key) const { return (key * 0x9E3779B1u) >> (32 - bb); }
-  __device__ bool overflowed(uint32_t b) const { return (flag[b >> 5] >> (b & 31)) & 1u; }
-  __device__ void mark(uint32_t b) const { atomicOr(&flag[b >> 5], 1u << (b & 31)); }
+  __device__ __forceinline__ uint32_t home(uint32_t key) const {
+    return (key * 0x9E3779B1u) >> (32 - bb);
+  }
+  __device__ __forceinline__ BucketRow row(uint32_t b) const {
+    const uint4* r = (const uint4*)t + 2 * b;
+    return BucketRow{state_read<GM>(r), state_read<GM>(r + 1)};
+  }
+  __device__ __forceinline__ bool passed(uint32_t b) const {
+    return ((state_read<GM>(cnt + (b >> 1)) >> (16 * (b & 1u))) & 0xFFFFu) != 0;
+  }
 
-  // Thread-level insert (the parallel fill): a free slot of the key's bucket,
-  // else the next bucket, flagging the full one.
-  __device__ void insert_thread(uint32_t key) const {
+  // Whether `key` is in a bucket after b (called when b has a count).
+  __device__ __noinline__ bool contains_after(uint32_t key, uint32_t b) const {
+    for (uint32_t i = 0; i < bmask; ++i) {
+      b = (b + 1) & bmask;
+      if (row(b).find(key) >= 0) return true;
+      if (!passed(b)) break;
+    }
+    return false;
+  }
+
+  // Insert a key known to be absent (several threads at once).
+  __device__ __noinline__ void insert(uint32_t key) const {
     uint32_t b = home(key);
     for (uint32_t i = 0; i <= bmask; ++i) {
-      for (int s = 0; s < 32; ++s) {
-        const int slot = (s + (int)(key & 31u)) & 31;
-        if (atomicCAS(&t[b * 32 + slot], kEmpty, key) == kEmpty) return;
-      }
-      mark(b);
+      for (int at = row(b).find(kEmpty); at >= 0; at = row(b).find(kEmpty))
+        if (atomicCAS(&t[8 * b + at], kEmpty, key) == kEmpty) return;
+      atomicAdd(&cnt[b >> 1], 1u << (16 * (b & 1u)));
       b = (b + 1) & bmask;
     }
   }
 
-  // Warp-level lookup of one key (all lanes, same key): bucket index and slot,
-  // or bucket -1 when absent.
-  __device__ int2 find_warp(uint32_t key, int lane) const {
-    uint32_t b = home(key);
-    for (uint32_t i = 0; i <= bmask; ++i) {
-      const unsigned hit = __ballot_sync(kWarp, t[b * 32 + lane] == key);
-      if (hit) return make_int2((int)b, __ffs(hit) - 1);
-      if (!overflowed(b)) break;
+  // Erase a key that is present but not in its home bucket b (several threads
+  // at once, insertions too: keys do not move).
+  __device__ __noinline__ void erase_after(uint32_t key, uint32_t b) const {
+    for (uint32_t i = 0; i < bmask; ++i) {
+      atomicSub(&cnt[b >> 1], 1u << (16 * (b & 1u)));
       b = (b + 1) & bmask;
-    }
-    return make_int2(-1, -1);
-  }
-
-  // Warp-level insert of a key known to be absent; returns its bucket.
-  __device__ uint32_t insert_warp(uint32_t key, int lane) const {
-    uint32_t b = home(key);
-    for (uint32_t i = 0; i <= bmask; ++i) {
-      const unsigned emp = __ballot_sync(kWarp, t[b * 32 + lane] == kEmpty);
-      if (emp) {
-        if (lane == 0) t[b * 32 + __ffs(emp) - 1] = key;
-        __syncwarp();
-        return b;
-      }
-      if (lane == 0) mark(b);
-      __syncwarp();
-      b = (b + 1) & bmask;
-    }
-    return b;
-  }
-
-  // Thread-level scan of one bucket (the lanes of a warp scan different
-  // buckets, each starting at another quarter-row to spread the banks): the
-  // slot holding `key` (-1 if none) and the mask of free slots.
-  __device__ void scan(uint32_t b, uint32_t key, int lane, int& at, unsigned& free_mask) const {
-    at = -1;
-    free_mask = 0;
-    const uint4* row = (const uint4*)(t + (size_t)b * 32);
-#pragma unroll 4
-    for (int c = 0; c < 8; ++c) {
-      const int q = (c + lane) & 7;
-      const uint4 v = row[q];
-      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (w[i] == key) at = 4 * q + i;
-        if (w[i] == kEmpty) free_mask |= 1u << (4 * q + i);
+      const int at = row(b).find(key);
+      if (at >= 0) {
+        t[8 * b + at] = kEmpty;
+        return;
       }
     }
   }
 };
 
-// One attempt's four set operations, by the whole warp: keys q[0], q[1] (the
-// new arcs or pairs: looked up, must be absent) and q[2], q[3] (the old ones:
-// present, erased on acceptance).  Lanes 8g..8g+7 read key g's home bucket as
-// four slots each.  Returns whether the attempt is accepted (neither new key
-// present) and, if so, has replaced the old keys by the new ones.
-__device__ __forceinline__ bool swap_keys(const BucketSet& S, uint32_t n1, uint32_t n2,
-                                          uint32_t o1, uint32_t o2, int lane, uint32_t& ib1,
-                                          uint32_t& ib2) {
-  const int grp = lane >> 3, sub = lane & 7;
-  const uint32_t key = grp == 0 ? n1 : grp == 1 ? n2 : grp == 2 ? o1 : o2;
-  const uint32_t b = S.home(key);
-  const uint4 v = ((const uint4*)(S.t + (size_t)b * 32))[sub];
-  const unsigned hit4 = (v.x == key ? 1u : 0u) | (v.y == key ? 2u : 0u) | (v.z == key ? 4u : 0u) |
-                        (v.w == key ? 8u : 0u);
-  const unsigned emp4 = (v.x == kEmpty ? 1u : 0u) | (v.y == kEmpty ? 2u : 0u) |
-                        (v.z == kEmpty ? 4u : 0u) | (v.w == kEmpty ? 8u : 0u);
-  const unsigned hm = __ballot_sync(kWarp, hit4 != 0);
-  const unsigned em = __ballot_sync(kWarp, emp4 != 0);
-  const bool miss = ((hm >> (8 * grp)) & 0xFFu) == 0;
-  // a key not in its home bucket may sit in a later one only past a flagged bucket
-  const unsigned deeper = __ballot_sync(kWarp, sub == 0 && miss && S.overflowed(b));
-  bool present1, present2;
-  if (deeper & 0x0101u) {  // a new key needs the slow lookup
-    present1 = S.find_warp(n1, lane).x >= 0;
-    present2 = S.find_warp(n2, lane).x >= 0;
-  } else {
-    present1 = (hm & 0xFFu) != 0;
-    present2 = (hm & 0xFF00u) != 0;
-  }
-  if (present1 || present2) return false;
-  // locations: slot = 4 * (first lane of the group with a match) + its first bit
-  const int hl1 = __ffs((hm >> 16) & 0xFFu) - 1, hl2 = __ffs((hm >> 24) & 0xFFu) - 1;
-  const unsigned h1 = __shfl_sync(kWarp, hit4, 16 + (hl1 < 0 ? 0 : hl1));
-  const unsigned h2 = __shfl_sync(kWarp, hit4, 24 + (hl2 < 0 ? 0 : hl2));
-  const int el1 = __ffs(em & 0xFFu) - 1, el2 = __ffs((em >> 8) & 0xFFu) - 1;
-  const unsigned f1 = __shfl_sync(kWarp, emp4, el1 < 0 ? 0 : el1);
-  const unsigned f2 = __shfl_sync(kWarp, emp4, 8 + (el2 < 0 ? 0 : el2));
-  const uint32_t b1 = __shfl_sync(kWarp, b, 0), b2 = __shfl_sync(kWarp, b, 8);
-  const uint32_t b3 = __shfl_sync(kWarp, b, 16), b4 = __shfl_sync(kWarp, b, 24);
-  // erase the old keys (at home, else by the slow lookup)
-  int2 p3 = make_int2((int)b3, hl1 < 0 ? -1 : 4 * hl1 + __ffs(h1) - 1);
-  int2 p4 = make_int2((int)b4, hl2 < 0 ? -1 : 4 * hl2 + __ffs(h2) - 1);
-  if (p3.y < 0) p3 = S.find_warp(o1, lane);
-  if (p4.y < 0) p4 = S.find_warp(o2, lane);
-  // insert the new keys into free slots of their home buckets; the slow insert
-  // for a full home bucket, or for the second key when both share one
-  const bool fast1 = el1 >= 0;
-  const bool fast2 = el2 >= 0 && b2 != b1;
-  if (lane == 0) {
-    if (p3.x >= 0) S.t[(size_t)p3.x * 32 + p3.y] = kEmpty;
-    if (p4.x >= 0) S.t[(size_t)p4.x * 32 + p4.y] = kEmpty;
-    if (fast1) S.t[(size_t)b1 * 32 + 4 * el1 + __ffs(f1) - 1] = n1;
-    if (fast2) S.t[(size_t)b2 * 32 + 4 * el2 + __ffs(f2) - 1] = n2;
-  }
-  __syncwarp();
-  ib1 = fast1 ? b1 : S.insert_warp(n1, lane);
-  ib2 = fast2 ? b2 : S.insert_warp(n2, lane);
-  return true;
+// Shared-memory working set of the windows.
+constexpr int kWindow = 64;      // attempts per window, four threads each
+constexpr int kRunners = 4 * kWindow;
+constexpr int kRandThreads = kRunners + 64;  // two warps draw
+constexpr int kDraws = 256;      // attempts per buffer of drawn positions
+constexpr int kKeyTab = 512, kPosTab = 512;
+struct RandWindow {
+  uint4 keys[kWindow];           // of an accepted attempt: new arcs, old arcs
+  uint2 pos[kWindow];            //   and its positions
+  uint2 ktab[kKeyTab];           // bits of the accepted attempts by arc (hashed)
+  uint2 ptab[kPosTab];           //   and by position
+  uint2 draws[2][kDraws];
+  int first_bad[2];              // first unsafe attempt; windows alternate
+};
+
+__device__ __forceinline__ uint32_t key_slot(uint32_t key) {
+  return (key * 0x85EBCA6Bu) >> 23;  // 32 - log2(kKeyTab)
 }
 
-// The attempts of one graph: `ent` is the entry array (arcs, or the dyad
-// lists), `Pol` draws an attempt's two positions and derives from the two
-// entries there its validity, the two new keys (to be absent), the two old
-// keys (to be erased) and the two new entries.  See the file comment for the
-// speculation and resolution of a batch of 32 attempts.
-template <class Pol>
-__device__ void run_attempts(const Pol& pol, uint32_t* ent, const BucketSet& S, uint64_t attempts,
-                             int lane, int64_t* accepted_out) {
-  int64_t acc = 0;
-  for (uint64_t t0 = 0; t0 < attempts;) {
-    const int cnt = (int)((attempts - t0) < 32 ? (attempts - t0) : 32);
-    // speculation; mode: 0 never valid (same position twice or past the
-    // end), 1 rejected (a new key present), 2 accepted with the recorded
-    // locations, 3 to be evaluated on the current state, 4 invalid entries
-    uint32_t e1 = 0, e2 = 0;
-    const bool drawn = pol.draw(t0 + lane, e1, e2) && lane < cnt;
-    int mode = 0;
-    uint32_t k1 = 0, k2 = 0, o1 = 0, o2 = 0, w1 = 0, w2 = 0, hb1 = 0xFFFFFFFFu, hb2 = 0xFFFFFFFFu;
-    int l1 = -1, l2 = -1, f1 = -1, f2 = -1;
-    if (drawn) {
-      mode = 4;
-      if (pol.make(ent[e1], ent[e2], k1, k2, o1, o2, w1, w2)) {
-        hb1 = S.home(k1);
-        hb2 = S.home(k2);
-        int at1, at2;
-        unsigned fm1, fm2, dummy;
-        S.scan(hb1, k1, lane, at1, fm1);
-        S.scan(hb2, k2, lane, at2, fm2);
-        S.scan(S.home(o1), o1, lane, l1, dummy);
-        S.scan(S.home(o2), o2, lane, l2, dummy);
-        if (l1 >= 0) l1 += (int)S.home(o1) * 32;
-        if (l2 >= 0) l2 += (int)S.home(o2) * 32;
-        if (at1 >= 0 || at2 >= 0) {
-          mode = 1;
-        } else if (S.overflowed(hb1) || S.overflowed(hb2) || l1 < 0 || l2 < 0) {
-          mode = 3;  // a key may lie past its home bucket
+// Barrier of the threads that run the attempts.
+__device__ __forceinline__ void run_sync() {
+  asm volatile("bar.sync 1, %0;" ::"n"(kRunners) : "memory");
+}
+
+// Threads 0 .. kRunners-1: the attempts whose positions are draws[0..n), in
+// order, thread 4j + q holding key q of the window's attempt j (0, 1: the new
+// keys, to be absent; 2, 3: the old ones).  `Pol::make` derives from the two
+// entries an attempt's validity, its keys and the two new entries.
+template <class Pol, bool GM>
+__device__ __forceinline__ void run_draws(const Pol& pol, uint32_t* ent, const BucketSet<GM>& S,
+                                          RandWindow& W, const uint2* draws, int n) {
+  const int j = threadIdx.x >> 2, q = threadIdx.x & 3, quad = threadIdx.x & 28;
+  const bool fresh = q < 2;
+  const int half = j >> 5;
+  const unsigned bit = 1u << (j & 31);
+  for (int t = 0, w = 0; t < n; w ^= 1) {
+    const int cnt = min(kWindow, n - t);
+    // speculation; `valid`: the outcome depends on the graph, `tried`: its keys
+    // are looked up, `acc`: accepted
+    uint2 e = make_uint2(0, 0);
+    if (j < cnt) e = draws[t + j];
+    const bool valid = e.x != e.y;
+    uint32_t k1 = 0, k2 = 0, o1 = 0, o2 = 0, w1 = 0, w2 = 0;
+    bool tried = false;
+    if (valid)
+      tried = pol.make(state_read<GM>(ent + e.x), state_read<GM>(ent + e.y), k1, k2, o1, o2, w1,
+                       w2);
+    const uint32_t key = fresh ? (q == 0 ? k1 : k2) : (q == 2 ? o1 : o2);
+    const uint32_t pos = q == 2 ? e.x : e.y;
+    // A new key: is it there, and a free slot of its home bucket.  An old one:
+    // its slot (only this attempt may erase it, so the slot stays valid).
+    const uint32_t h = S.home(key);
+    const BucketRow r = S.row(h);
+    // (New keys of one window prefer different slots of a bucket.)
+    const unsigned slots = r.mask(fresh ? kEmpty : key);
+    const unsigned turned = fresh ? (slots | slots << 8) >> (j & 7) : slots;
+    const int at = slots ? (__ffs(turned) - 1 + (fresh ? j : 0)) & 7 : -1;
+    bool there = r.has(key);
+    if (tried && fresh && !there && S.passed(h)) there = S.contains_after(key, h);
+    const unsigned hit = __ballot_sync(kWarp, fresh && there) >> quad;
+    const bool acc = tried && (hit & 3u) == 0;
+    const uint32_t ks = key_slot(key), ps = pos & (kPosTab - 1);
+    if (acc) {
+      if (q == 0) W.keys[j] = make_uint4(k1, k2, o1, o2);
+      if (q == 1) W.pos[j] = e;
+      atomicOr((uint32_t*)&W.ktab[ks] + half, bit);
+      if (!fresh) atomicOr((uint32_t*)&W.ptab[ps] + half, bit);
+    }
+    run_sync();
+    // earlier accepted attempts that may overlap: by arc for the new keys, by
+    // position for the old ones
+    bool unsafe = false;
+    if (fresh ? tried : valid) {
+      const uint2 c = fresh ? W.ktab[ks] : W.ptab[ps];
+      uint32_t lo = c.x, hi = c.y;
+      if (half == 0) {
+        lo &= bit - 1u;
+        hi = 0;
+      } else {
+        hi &= bit - 1u;
+      }
+      while (lo | hi) {
+        const int i = lo ? __ffs(lo) - 1 : 31 + __ffs(hi);
+        if (lo) lo &= lo - 1;
+        else hi &= hi - 1;
+        bool same;
+        if (fresh) {
+          const uint4 k = W.keys[i];
+          same = key == k.x || key == k.y || key == k.z || key == k.w;
         } else {
-          f1 = free_slot_from(fm1, (int)(k1 & 31u));
-          if (hb1 == hb2 && f1 >= 0) fm2 = fm1 & ~(1u << f1);
-          f2 = free_slot_from(fm2, (int)(k2 & 31u));
-          mode = (f1 >= 0 && f2 >= 0) ? 2 : 3;
+          const uint2 p = W.pos[i];
+          same = pos == p.x || pos == p.y;
+        }
+        if (same) {
+          unsafe = true;
+          break;
         }
       }
     }
-    // the slots this attempt would fill (bucket * 32 + slot)
-    const uint32_t s1 = mode == 2 ? hb1 * 32 + (uint32_t)f1 : 0xFFFFFFFFu;
-    const uint32_t s2 = mode == 2 ? hb2 * 32 + (uint32_t)f2 : 0xFFFFFFFFu;
-    // An attempt is unsafe when an earlier attempt of the batch that the
-    // speculation accepted wrote one of its positions, inserted or erased a
-    // key it looks up, or fills a slot it would fill.  Before the first unsafe
-    // attempt every speculative outcome is the sequential one, and the
-    // accepted attempts there touch disjoint entries and slots.
-    bool unsafe = mode == 3;
-#pragma unroll 4
-    for (int i = 0; i < 31; ++i) {
-      const int im = __shfl_sync(kWarp, mode, i);
-      const uint32_t ie1 = __shfl_sync(kWarp, e1, i), ie2 = __shfl_sync(kWarp, e2, i);
-      const uint32_t ik1 = __shfl_sync(kWarp, k1, i), ik2 = __shfl_sync(kWarp, k2, i);
-      const uint32_t io1 = __shfl_sync(kWarp, o1, i), io2 = __shfl_sync(kWarp, o2, i);
-      const uint32_t is1 = __shfl_sync(kWarp, s1, i), is2 = __shfl_sync(kWarp, s2, i);
-      const bool pos = e1 == ie1 || e1 == ie2 || e2 == ie1 || e2 == ie2;
-      const bool key = k1 == ik1 || k1 == ik2 || k2 == ik1 || k2 == ik2 || k1 == io1 ||
-                       k1 == io2 || k2 == io1 || k2 == io2;
-      const bool slot = s1 == is1 || s1 == is2 || s2 == is1 || s2 == is2;
-      unsafe |= im == 2 && lane > i &&
-                (pos || (key && (mode == 1 || mode == 2)) || (slot && mode == 2));
-    }
-    const unsigned bad = __ballot_sync(kWarp, unsafe && mode != 0 && lane < cnt);
-    const int p = bad ? __ffs(bad) - 1 : cnt;
-    if (lane < p && mode == 2) {
-      S.t[l1] = kEmpty;
-      S.t[l2] = kEmpty;
-      S.t[s1] = k1;
-      S.t[s2] = k2;
-      ent[e1] = w1;
-      ent[e2] = w2;
-    }
-    acc += __popc(__ballot_sync(kWarp, lane < p && mode == 2));
-    __syncwarp();
-    if (p < cnt) {
-      // the first unsafe attempt, on the current state, by the whole warp
-      const uint32_t je1 = __shfl_sync(kWarp, e1, p), je2 = __shfl_sync(kWarp, e2, p);
-      uint32_t nk1, nk2, no1, no2, nw1, nw2, nb1, nb2;
-      if (pol.make(ent[je1], ent[je2], nk1, nk2, no1, no2, nw1, nw2) &&
-          swap_keys(S, nk1, nk2, no1, no2, lane, nb1, nb2)) {
-        if (lane == 0) {
-          ent[je1] = nw1;
-          ent[je2] = nw2;
+    const unsigned bad = __ballot_sync(kWarp, unsafe);
+    if (bad && (threadIdx.x & 31) == 0)
+      atomicMin(&W.first_bad[w], (int)(threadIdx.x >> 2) + ((__ffs(bad) - 1) >> 2));
+    run_sync();
+    // attempts before the first unsafe one (the first of a window is never
+    // unsafe) are applied, and the marks go.  A free slot that another key took,
+    // or a bucket without one, sends a key the slow way.
+    const int p = min(W.first_bad[w], cnt);
+    if (threadIdx.x == 0) W.first_bad[w ^ 1] = kWindow;
+    if (acc) {
+      W.ktab[ks] = make_uint2(0, 0);
+      if (!fresh) W.ptab[ps] = make_uint2(0, 0);
+      if (j < p) {
+        if (!fresh) {
+          ent[pos] = q == 2 ? w1 : w2;
+          if (at >= 0) S.t[8 * h + at] = kEmpty;
+          else S.erase_after(key, h);
+        } else if (at < 0 || atomicCAS(&S.t[8 * h + at], kEmpty, key) != kEmpty) {
+          S.insert(key);
         }
-        ++acc;
       }
-      __syncwarp();
-      t0 += (uint64_t)p + 1;
-    } else {
-      t0 += (uint64_t)cnt;
     }
+    run_sync();
+    t += p;
   }
-  if (lane == 0 && accepted_out) *accepted_out = acc;
+}
+
+// The attempts of one graph, by the whole block: kRunners threads run the drawn
+// attempts of one buffer while the others draw the next buffer's positions.
+template <class Pol, bool GM>
+__device__ void run_attempts(const Pol& pol, uint32_t* ent, const BucketSet<GM>& S, RandWindow& W,
+                             uint64_t attempts) {
+  const int tid = threadIdx.x;
+  for (int i = tid; i < kKeyTab; i += blockDim.x) W.ktab[i] = make_uint2(0, 0);
+  for (int i = tid; i < kPosTab; i += blockDim.x) W.ptab[i] = make_uint2(0, 0);
+  if (tid < 2) W.first_bad[tid] = kWindow;
+  auto draw = [&](uint64_t t0, int buf, int first, int step) {
+    for (int j = first; j < kDraws && t0 + j < attempts; j += step)
+      pol.draw(t0 + j, W.draws[buf][j].x, W.draws[buf][j].y);
+  };
+  draw(0, 0, tid, blockDim.x);
+  __syncthreads();
+  int buf = 0;
+  for (uint64_t t0 = 0; t0 < attempts; t0 += kDraws, buf ^= 1) {
+    if (tid < kRunners) {
+      const int n = (int)(attempts - t0 < (uint64_t)kDraws ? attempts - t0 : kDraws);
+      run_draws(pol, ent, S, W, W.draws[buf], n);
+      if (tid == 0) W.first_bad[0] = kWindow;
+    } else {
+      draw(t0 + kDraws, buf ^ 1, tid - kRunners, blockDim.x - kRunners);
+    }
+    __syncthreads();
+  }
 }
 
 // Degree-preserving arc swaps: attempt t's positions are SplitMix64 outputs
 // 2t and 2t+1 scaled to [0, m); entries and keys are arcs (src << 16 | dst).
 struct ArcSwap {
   uint64_t seed, m;
-  __device__ bool draw(uint64_t t, uint32_t& e1, uint32_t& e2) const {
+  __device__ void draw(uint64_t t, uint32_t& e1, uint32_t& e2) const {
     const uint64_t gamma = 0x9E3779B97F4A7C15ull;
     e1 = (uint32_t)__umul64hi(sm64_mix(seed + (2 * t + 1) * gamma), m);
     e2 = (uint32_t)__umul64hi(sm64_mix(seed + (2 * t + 2) * gamma), m);
-    return e1 != e2;
   }
   __device__ bool make(uint32_t A, uint32_t B, uint32_t& k1, uint32_t& k2, uint32_t& o1,
                        uint32_t& o2, uint32_t& w1, uint32_t& w2) const {
@@ -348,8 +349,6 @@ struct RandArgs {
   uint64_t swaps;
   int32_t* col_out;        // G x m destinations after the swaps (rows unsorted)
   uint32_t* gscratch;      // per-graph state when it does not fit shared memory
-  int use_smem;
-  int64_t* accepted;       // G counters (may be null)
 };
 
 __device__ __forceinline__ int row_of(const int32_t* row_ptr, int n, int e) {
@@ -361,31 +360,29 @@ __device__ __forceinline__ int row_of(const int32_t* row_ptr, int n, int e) {
   return lo;
 }
 
-__global__ void __launch_bounds__(512, 2) k_randomize(RandArgs a) {
+template <bool GM>
+__global__ void __launch_bounds__(kRandThreads) k_randomize(RandArgs a) {
   extern __shared__ __align__(16) uint32_t rsm[];
+  __shared__ RandWindow W;
   const int g = blockIdx.x;
   const int m = a.m, n = a.n;
   const RandLayout L = rand_layout(m);
-  uint32_t* base = a.use_smem ? rsm : a.gscratch + (size_t)g * L.words;
-  uint32_t* arcs = base;
-  BucketSet S{base + L.t_off, base + L.f_off, L.bb, (1u << L.bb) - 1u};
-  for (size_t i = threadIdx.x; i < ((size_t)32 << L.bb); i += blockDim.x) S.t[i] = kEmpty;
-  for (size_t i = threadIdx.x; i < L.words - L.f_off; i += blockDim.x) S.flag[i] = 0;
+  uint32_t* arcs = GM ? a.gscratch + (size_t)g * L.words : rsm;
+  const BucketSet<GM> S{arcs + L.t_off, arcs + L.c_off, L.bb, (1u << L.bb) - 1u};
+  for (size_t i = threadIdx.x; i < L.c_off - L.t_off; i += blockDim.x) S.t[i] = kEmpty;
+  for (size_t i = threadIdx.x; i < L.words - L.c_off; i += blockDim.x) S.cnt[i] = 0;
   for (int e = threadIdx.x; e < m; e += blockDim.x)
     arcs[e] = ((uint32_t)row_of(a.row_ptr, n, e) << 16) | (uint32_t)a.col0[e];
   __syncthreads();
-  for (int e = threadIdx.x; e < m; e += blockDim.x) S.insert_thread(arcs[e]);
+  for (int e = threadIdx.x; e < m; e += blockDim.x) S.insert(arcs[e]);
   __syncthreads();
-  // Warp 0: the lanes draw the arc positions of 32 attempts at a time (the
-  // SplitMix64 outputs do not depend on the graph), then the warp applies the
-  // attempts one after another.
-  if (threadIdx.x < 32 && m > 0) {
+  if (m > 0) {
     const ArcSwap pol{a.seeds[g], (uint64_t)m};
-    run_attempts(pol, arcs, S, a.swaps, threadIdx.x, a.accepted ? a.accepted + g : nullptr);
+    run_attempts(pol, arcs, S, W, a.swaps);
   }
   __syncthreads();
   for (int e = threadIdx.x; e < m; e += blockDim.x)
-    a.col_out[(size_t)g * m + e] = (int32_t)(arcs[e] & 0xFFFFu);
+    a.col_out[(size_t)g * m + e] = (int32_t)(state_read<GM>(arcs + e) & 0xFFFFu);
 }
 
 // Dyad-preserving variant (swap mutual pairs and one-way arcs separately; the
@@ -405,8 +402,6 @@ struct DyadArgs {
   int32_t* col_out;        // G x m destinations, rows unsorted
   int32_t* scratch;        // G x (2m + n + 2) ints
   uint32_t* gscratch;      // per-graph state when it does not fit shared memory
-  int use_smem;
-  int64_t* accepted;
 };
 
 __device__ __forceinline__ bool has_arc(const int32_t* row_ptr, const int32_t* col, int a, int b) {
@@ -429,7 +424,7 @@ __device__ __forceinline__ uint32_t pair_key(uint32_t u, uint32_t v) {
 // [0, S) and the mutual dyads [S, S + D), keys the unordered adjacent pairs.
 struct DyadSwap {
   uint64_t seed, S, D;
-  __device__ bool draw(uint64_t t, uint32_t& e1, uint32_t& e2) const {
+  __device__ void draw(uint64_t t, uint32_t& e1, uint32_t& e2) const {
     const uint64_t gamma = 0x9E3779B97F4A7C15ull;
     const uint64_t r0 = sm64_mix(seed + (3 * t + 1) * gamma);
     const uint64_t r1 = sm64_mix(seed + (3 * t + 2) * gamma);
@@ -439,7 +434,6 @@ struct DyadSwap {
     const uint32_t base_l = single ? 0u : (uint32_t)S;
     e1 = base_l + (uint32_t)__umul64hi(r1, len);
     e2 = base_l + (uint32_t)__umul64hi(r2, len);
-    return e1 != e2;
   }
   __device__ bool make(uint32_t A, uint32_t B, uint32_t& k1, uint32_t& k2, uint32_t& o1,
                        uint32_t& o2, uint32_t& w1, uint32_t& w2) const {
@@ -455,20 +449,22 @@ struct DyadSwap {
   }
 };
 
-__global__ void __launch_bounds__(512, 2) k_randomize_dyads(DyadArgs a) {
+template <bool GM>
+__global__ void __launch_bounds__(kRandThreads) k_randomize_dyads(DyadArgs a) {
   extern __shared__ __align__(16) uint32_t dsm[];
+  __shared__ RandWindow W;
   __shared__ int scan_tmp[33];
   const int g = blockIdx.x;
   const int m = a.m, n = a.n;
   const RandLayout L = rand_layout(m);
-  uint32_t* base = a.use_smem ? dsm : a.gscratch + (size_t)g * L.words;
-  uint32_t* lists = base;  // singles [0, S), dyads [S, S + D)
-  BucketSet Sset{base + L.t_off, base + L.f_off, L.bb, (1u << L.bb) - 1u};
+  // singles [0, S), dyads [S, S + D)
+  uint32_t* lists = GM ? a.gscratch + (size_t)g * L.words : dsm;
+  const BucketSet<GM> Sset{lists + L.t_off, lists + L.c_off, L.bb, (1u << L.bb) - 1u};
   int32_t* fs = a.scratch + (size_t)g * (2 * (size_t)m + n + 2);
   int32_t* fd = fs + m + 1;
   int32_t* cur = fd + m + 1;
-  for (size_t i = threadIdx.x; i < ((size_t)32 << L.bb); i += blockDim.x) Sset.t[i] = kEmpty;
-  for (size_t i = threadIdx.x; i < L.words - L.f_off; i += blockDim.x) Sset.flag[i] = 0;
+  for (size_t i = threadIdx.x; i < L.c_off - L.t_off; i += blockDim.x) Sset.t[i] = kEmpty;
+  for (size_t i = threadIdx.x; i < L.words - L.c_off; i += blockDim.x) Sset.cnt[i] = 0;
   for (int v = threadIdx.x; v < n; v += blockDim.x) cur[v] = 0;
   // kinds of the arcs, in CSR order
   for (int e = threadIdx.x; e < m; e += blockDim.x) {
@@ -495,19 +491,18 @@ __global__ void __launch_bounds__(512, 2) k_randomize_dyads(DyadArgs a) {
   }
   __syncthreads();
   for (int i = threadIdx.x; i < S + D; i += blockDim.x)
-    Sset.insert_thread(pair_key(lists[i] >> 16, lists[i] & 0xFFFFu));
+    Sset.insert(pair_key(lists[i] >> 16, lists[i] & 0xFFFFu));
   __syncthreads();
-  if (threadIdx.x < 32 && S + D > 0) {
+  if (S + D > 0) {
     const DyadSwap pol{a.seeds[g], (uint64_t)S, (uint64_t)D};
-    run_attempts(pol, lists, Sset, a.attempts, threadIdx.x,
-                 a.accepted ? a.accepted + g : nullptr);
+    run_attempts(pol, lists, Sset, W, a.attempts);
   }
   __syncthreads();
   // arcs back into the rows of the fixed out-CSR shape (order inside a row is
   // arbitrary; the builder sorts)
   int32_t* out = a.col_out + (size_t)g * m;
   for (int i = threadIdx.x; i < S + D; i += blockDim.x) {
-    const uint32_t x = lists[i];
+    const uint32_t x = state_read<GM>(lists + i);
     const int u = (int)(x >> 16), v = (int)(x & 0xFFFFu);
     out[a.row_ptr[u] + atomicAdd(&cur[u], 1)] = v;
     if (i >= S) out[a.row_ptr[v] + atomicAdd(&cur[v], 1)] = u;
@@ -523,7 +518,7 @@ static bool rand_fits_smem(int32_t m) {
   int dev = 0, max_smem = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  return rand_smem_bytes(m) <= (size_t)max_smem - 2048;
+  return rand_smem_bytes(m) <= (size_t)max_smem - sizeof(RandWindow) - 2048;
 }
 
 // Scratch (uint32 words) that G randomisations need when their state does not
@@ -532,42 +527,50 @@ size_t rand_gscratch_words(int32_t m, int G) {
   return rand_fits_smem(m) ? 0 : (size_t)G * rand_layout(m).words;
 }
 
-template <typename Kern, typename Args>
-static cudaError_t launch_rand(Kern kern, Args& a, int32_t m, int G, uint32_t* gscratch,
-                               cudaStream_t s) {
-  a.use_smem = rand_fits_smem(m) ? 1 : 0;
+template <typename Args>
+static cudaError_t launch_rand(void (*in_smem)(Args), void (*in_global)(Args), Args& a, int32_t m,
+                               int G, uint32_t* gscratch, cudaStream_t s) {
   a.gscratch = gscratch;
-  if (!a.use_smem && !gscratch) return cudaErrorInvalidValue;
-  const size_t smem = a.use_smem ? rand_smem_bytes(m) : 0;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+  if (!rand_fits_smem(m)) {
+    if (!gscratch) return cudaErrorInvalidValue;
+    in_global<<<G, kRandThreads, 0, s>>>(a);
+    return cudaGetLastError();
   }
-  kern<<<G, 512, smem, s>>>(a);
+  const size_t smem = rand_smem_bytes(m);
+  // the limit is the function's, shared by launches of other sizes: always the
+  // largest this rule lets through
+  int dev = 0, max_smem = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute((const void*)in_smem, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             max_smem - (int)sizeof(RandWindow) - 2048);
+  if (e != cudaSuccess) return e;
+  in_smem<<<G, kRandThreads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
 cudaError_t launch_randomize_dyads(int32_t n, int32_t m, int G, const int32_t* row_ptr,
                                    const int32_t* col0, const uint64_t* seeds, uint64_t attempts,
                                    int32_t* col_out, int32_t* scratch, uint32_t* gscratch,
-                                   int64_t* accepted, cudaStream_t s) {
+                                   cudaStream_t s) {
   DyadArgs a;
   a.n = n; a.m = m; a.G = G;
   a.row_ptr = row_ptr; a.col0 = col0; a.seeds = seeds; a.attempts = attempts;
-  a.col_out = col_out; a.scratch = scratch; a.accepted = accepted;
-  return launch_rand(k_randomize_dyads, a, m, G, gscratch, s);
+  a.col_out = col_out; a.scratch = scratch;
+  return launch_rand(k_randomize_dyads<false>, k_randomize_dyads<true>, a, m, G, gscratch, s);
 }
 
 // Enqueue G randomisations of the graph (row_ptr, col0) into col_out.
 cudaError_t launch_randomize(int32_t n, int32_t m, int G, const int32_t* row_ptr,
                              const int32_t* col0, const uint64_t* seeds, uint64_t swaps,
-                             int32_t* col_out, uint32_t* gscratch, int64_t* accepted,
-                             cudaStream_t s) {
+                             int32_t* col_out, uint32_t* gscratch, cudaStream_t s) {
   RandArgs a;
   a.n = n; a.m = m; a.G = G;
   a.row_ptr = row_ptr; a.col0 = col0; a.seeds = seeds; a.swaps = swaps;
-  a.col_out = col_out; a.accepted = accepted;
-  return launch_rand(k_randomize, a, m, G, gscratch, s);
+  a.col_out = col_out;
+  return launch_rand(k_randomize<false>, k_randomize<true>, a, m, G, gscratch, s);
 }
 
 mt_status graph_alloc(int32_t n, int32_t m, mt_graph** out);
@@ -598,8 +601,7 @@ mt_status mt_randomize(const mt_graph* src, uint64_t seed, uint64_t swaps, void*
   uint32_t* gscr = gwords ? (uint32_t*)((char*)d_seed + 16) : nullptr;
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_seed, &seed, 8, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
-    e = launch_randomize(src->n, src->m, 1, src->row_ptr, src->col, d_seed, swaps, col_tmp, gscr,
-                         nullptr, s);
+    e = launch_randomize(src->n, src->m, 1, src->row_ptr, src->col, d_seed, swaps, col_tmp, gscr, s);
   if (e != cudaSuccess) {
     set_last_error(cudaGetErrorString(e));
     if (scratch) cudaFreeAsync(scratch, s);
@@ -638,7 +640,7 @@ mt_status mt_randomize_dyads(const mt_graph* src, uint64_t seed, uint64_t attemp
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_seed, &seed, 8, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
     e = launch_randomize_dyads(src->n, src->m, 1, src->row_ptr, src->col, d_seed, attempts,
-                               col_tmp, dsc, gscr, nullptr, s);
+                               col_tmp, dsc, gscr, s);
   if (e != cudaSuccess) {
     set_last_error(cudaGetErrorString(e));
     if (scratch) cudaFreeAsync(scratch, s);

@@ -173,8 +173,8 @@ mt_status mt_table_entries(const mt_table* t, uint64_t first, uint64_t count, ui
  * connected set is produced exactly once by the extension enumerator (root =
  * smallest vertex, extension by exclusive neighbours), its adjacency bits are
  * gathered from the labelled neighbour rows (the row-scan strategy of Sec. 3.1)
- * and classified by one table read (Sec. 3.2); at k = 5 and 6, and at k = 4 on
- * large graphs, the last two vertices are counted per pair of cells instead
+ * and classified by one table read (Sec. 3.2) under MT_METHOD_ENUMERATE; calls
+ * without a tuning count the last two vertices per pair of cells instead
  * (Algorithm 1 of Sec. 3; see mt_method), with the same result.  n < k gives
  * all zeros.
  * The call may grow device scratch memory held by the graph handle.  At k = 6
@@ -203,8 +203,8 @@ mt_status mt_count_roots(const mt_graph* g, const mt_table* t, int32_t root_begi
 
 /* Counting method.
  * Calls without an mt_tuning (or with a null one) and servers whose method was
- * not set use the faster of the two for k and the graph's size; the value of
- * mt_tuning.method is always followed.
+ * not set use the faster one (cells); the value of mt_tuning.method is always
+ * followed.
  * MT_METHOD_ENUMERATE (0): every connected k-set is produced and its class
  *   read from the table (per-subgraph classification, Sec. 3.2).
  * MT_METHOD_CELLS: the enumeration stops at (k-2)-sets X; the k-sets X + {y, z}
@@ -216,7 +216,8 @@ mt_status mt_count_roots(const mt_graph* g, const mt_table* t, int32_t root_begi
 typedef enum { MT_METHOD_ENUMERATE = 0, MT_METHOD_CELLS = 1 } mt_method;
 
 /* Launch tuning of the enumerator (all fields 0 = automatic).
- * - split_cost: estimated work (classified subgraphs) above which a first-level
+ * - split_cost: estimated work (classified subgraphs, or list entries of the
+ *   cell method) above which a first-level
  *   extension branch of a root is split into second-level work items, and the
  *   target size of first-level items; the root-split threshold.
  * - split_scale: when split_cost is 0, a multiplier of the automatic threshold
@@ -457,8 +458,7 @@ mt_status mt_server_result(mt_server* s, uint64_t id, int32_t* state, uint64_t* 
                            double* latency_ms);
 
 /* Counting method of the rounds launched from now on (an mt_method; the
- * default is the faster one for each k and size, see mt_method).  Results do
- * not depend on it. */
+ * default is the faster one, see mt_method).  Results do not depend on it. */
 mt_status mt_server_set_method(mt_server* s, int method);
 
 /* Device bytes currently charged against the budget by active requests. */

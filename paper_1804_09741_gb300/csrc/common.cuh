@@ -43,14 +43,15 @@ struct DevGraph {
   unsigned long long* hist; // histogram this graph's subgraphs are added to
 };
 
-// Work item of the enumerator: root `root` of graph `g`, first-level branches
-// [j1a, j1b) of the root's forward neighbour list; when j1b == j1a + 1 the
-// second-level choices may be limited to [a2, b2) (b2 == 0xFFFF: no limit).
+// Work item of the enumerator: root `root` of the queue's graph, first-level
+// branches [j1a, j1b) of the root's forward neighbour list; when j1b == j1a + 1
+// the second-level choices may be limited to [a2, b2) (b2 == 0xFFFF: no limit),
+// and when b2 == a2 + 1 the third-level ones to [a3, b3) likewise (k = 6).
 struct Item {
-  uint32_t g;
   uint32_t root;
   uint16_t j1a, j1b;
   uint16_t a2, b2;
+  uint16_t a3, b3;
 };
 static_assert(sizeof(Item) == 16, "Item is 16 bytes");
 

@@ -64,12 +64,25 @@ struct Hdr {
   uint32_t head;
   uint32_t err;
   uint32_t pad0, pad1;
-  double total_est;
-  double pad2;
+};
+
+// The planner's result for one graph: its estimated work, and its items
+// [base, base + count) of the launch's array with the queue's head.
+struct GraphPlan {
+  double est;
+  uint32_t count, base;
+  uint32_t qhead, pad;
 };
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr int kTargetItemsPerWarp = 64;
+// Cell method: an item's least estimated work, below which fetching it and
+// marking its root's neighbours costs more than the warps it feeds give.  One
+// graph on a GB300: k = 4 (n = 2,000 / 3,646 / 6,437) 119 / 163 / 180 us at 128
+// against 147 / 199 / 203 at 512 and 195 / 432 / 627 near 10; k = 5 (n = 1,500)
+// 884 at 512, 1,044 near 50; k = 3 (n = 20,000) 149 at 1,024, 176 at 256.
+template <int K>
+constexpr double kCellsItemFloor = K == 3 ? 1024.0 : K == 4 ? 128.0 : 512.0;
 // Adds one warp may make to a shared 32-bit histogram between two flushes of
 // it by exchange (enumeration path, k <= 5; see `ladd` in k_count).
 constexpr int kLeafBudget = 1 << 25;
@@ -120,11 +133,21 @@ __device__ __forceinline__ float choose_f(int x, int r) {
 }
 
 // Estimated work of a first-level branch whose second-level candidate list has
-// x1 entries: about C(x1, k-2) sets of k-1 vertices, each touching its
-// candidates once.
-template <int K>
-__device__ __forceinline__ float branch_cost(int x1) {
-  return 1.f + (float)x1 + choose_f(x1, K - 2) * (K >= 4 ? 2.f : 1.f);
+// x1 entries, whose degrees add up to w1.  Per-subgraph method: about
+// C(x1, k-2) sets of k-1 vertices, each touching its candidates once.  Cell
+// method: a fixed cost (64) for each (k-2)-set, and its list; the third-level
+// lists (x1^2 / 2 + w1 entries together) are the k = 5 sets' lists and the number
+// of k = 6 sets.  With x1 alone a k = 6 branch that reaches a hub was estimated
+// 160 times too low, and its block ran on after the others (SMs active 2.2 to
+// 4.1 million cycles on one graph of n = 800).
+template <int K, bool CB>
+__device__ __forceinline__ float branch_cost(int x1, float w1) {
+  const float x = (float)x1;
+  if (!CB) return 1.f + x + choose_f(x1, K - 2) * (K >= 4 ? 2.f : 1.f);
+  if (K == 3) return 8.f + x;
+  if (K == 4) return 72.f + 2.f * x;
+  const float l2 = 0.5f * x * x + w1;
+  return K == 5 ? 8.f + 65.f * x + l2 : 8.f + x + l2 * (64.f + x);
 }
 
 // Offset of position p's 2p bits in an extension-order key of k vertices:
@@ -143,158 +166,215 @@ __device__ __forceinline__ void red_add_shared(int* p, int v) {
                : "memory");
 }
 
-// Whether vertex x is in sorted packed entries [lo, hi).
-__device__ __forceinline__ bool contains(const uint32_t* __restrict__ ucol, int lo, int hi, int x) {
+// First index in sorted packed entries [lo, hi) whose vertex is > x.
+__device__ __forceinline__ int first_above(const uint32_t* __restrict__ ucol, int lo, int hi,
+                                           int x) {
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
-    const int y = (int)(__ldg(&ucol[mid]) & kVertexMask);
-    if (y == x) return true;
-    if (y < x) lo = mid + 1; else hi = mid;
+    if ((int)(__ldg(&ucol[mid]) & kVertexMask) > x) hi = mid; else lo = mid + 1;
   }
-  return false;
+  return lo;
 }
 
 // ------------------------------------------------------------------ planner
+//
+// Two launches: the graphs' estimated work, then their items.  A branch's
+// estimate takes the neighbours of its vertex above the root as its new
+// candidates, common neighbours counted twice: that bounds the second-level list
+// (ranges past its end are empty items) and needs one binary search where exact
+// counts took a search per neighbour.  Measured on a GB300, one k = 5 graph
+// (n = 1,500): 400 us before, 40 now;
+// 512 graphs of n = 300 at k = 3: 590 us before, 130 now.
 
-template <int K>
-__global__ void __launch_bounds__(256) k_plan_est(const DevGraph* __restrict__ graphs,
-                                                  int64_t stride, float* est, int32_t* x1s,
-                                                  Hdr* hdr, int root_begin, int root_end) {
-  __shared__ float red[8];
-  const int g = blockIdx.y;
-  const DevGraph G = graphs[g];
-  float local = 0.f;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < G.nu; e += gridDim.x * blockDim.x) {
-    const int v = G.usrc[e];
-    const int u = (int)(G.ucol[e] & kVertexMask);
-    float c = 0.f;
-    int x1 = 0;
-    if (u > v && v >= root_begin && v < root_end && v >= G.root_begin && v < G.root_end) {
-      const int re = G.urow[v + 1];
-      const int f = G.urow[v] + G.ufwd[v];
-      const int j1 = e - f;
-      int ex = 0;
-      for (int i = G.urow[u]; i < G.urow[u + 1]; ++i) {
-        const int x = (int)(G.ucol[i] & kVertexMask);
-        if (x > v && !contains(G.ucol, f, re, x)) ++ex;
-      }
-      x1 = (re - f) - j1 - 1 + ex;
-      c = branch_cost<K>(x1);
+// Sum of the neighbours' degrees of every vertex (the cell method at k >= 5).
+__global__ void __launch_bounds__(256) k_plan_degsum(const DevGraph* __restrict__ graphs, int nmax,
+                                                     int32_t* dsum) {
+  const DevGraph G = graphs[blockIdx.y];
+  const int lane = threadIdx.x & 31;
+  const int nwarps = (int)(gridDim.x * (blockDim.x >> 5));
+  for (int v = blockIdx.x * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5); v < G.n;
+       v += nwarps) {
+    int sum = 0;
+    for (int i = G.urow[v] + lane; i < G.urow[v + 1]; i += 32) {
+      const int u = (int)(G.ucol[i] & kVertexMask);
+      sum += G.urow[u + 1] - G.urow[u];
     }
-    est[g * stride + e] = c;
-    x1s[g * stride + e] = x1;
-    local += c;
+    for (int d = 16; d; d >>= 1) sum += __shfl_xor_sync(kFull, sum, d);
+    if (lane == 0) dsum[(int64_t)blockIdx.y * nmax + v] = sum;
+  }
+}
+
+// Branch of entry e (a forward entry of root v, whose row is [rs, re)): its
+// cost, and x = the bound of its second-level list.  dsum: this graph's sums of
+// the neighbours' degrees; the degrees of the root's later neighbours are taken
+// as the row's mean.
+template <int K, bool CB>
+__device__ __forceinline__ float entry_cost(const DevGraph& G, const int32_t* __restrict__ dsum,
+                                            int v, int rs, int re, int e, int& x) {
+  const int u = (int)(__ldg(&G.ucol[e]) & kVertexMask);
+  const int ue = __ldg(&G.urow[u + 1]);
+  x = (re - e - 1) + (ue - first_above(G.ucol, __ldg(&G.urow[u]), ue, v));
+  float w = 0.f;
+  if (CB && K >= 5)
+    w = (float)__ldg(&dsum[u]) + (float)(re - e - 1) * ((float)__ldg(&dsum[v]) / (float)(re - rs));
+  return branch_cost<K, CB>(x, w);
+}
+
+template <int K, bool CB>
+__global__ void __launch_bounds__(256) k_plan_total(const DevGraph* __restrict__ graphs,
+                                                    GraphPlan* gp,
+                                                    const int32_t* __restrict__ dsum_all, int nmax,
+                                                    int root_begin, int root_end) {
+  __shared__ double red[8];
+  const DevGraph G = graphs[blockIdx.y];
+  const int32_t* dsum = dsum_all + (int64_t)blockIdx.y * nmax;
+  const int r0 = max(root_begin, G.root_begin), r1 = min(root_end, G.root_end);
+  double local = 0.0;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < G.nu; e += gridDim.x * blockDim.x) {
+    const int v = __ldg(&G.usrc[e]);
+    if (v < r0 || v >= r1) continue;
+    const int rs = __ldg(&G.urow[v]);
+    int x;
+    if (e >= rs + __ldg(&G.ufwd[v]))
+      local += entry_cost<K, CB>(G, dsum, v, rs, __ldg(&G.urow[v + 1]), e, x);
   }
   for (int d = 16; d; d >>= 1) local += __shfl_xor_sync(kFull, local, d);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = local;
   __syncthreads();
   if (threadIdx.x == 0) {
-    float s = 0.f;
+    double s = 0.0;
     for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += red[i];
-    if (s > 0.f) atomicAdd(&hdr->total_est, (double)s);
+    if (s > 0.0) atomicAdd(&gp[blockIdx.y].est, s);
   }
 }
 
-// Walk one root's forward branches and cut them into items (count or write).
-// One warp per root: the lanes load 32 entries at a time, every lane walks them
-// in order with the same (warp-uniform) packing state, and the many level-2
-// ranges of a split branch are written by all lanes at once, so a hub root's
-// thousands of items cost a few stores per lane instead of a serial loop.
-template <int K, bool WRITE>
-__global__ void __launch_bounds__(256) k_plan_items(const DevGraph* __restrict__ graphs,
-                                                    int64_t stride, const float* est,
-                                                    const int32_t* x1s, int nmax, int32_t* cnt,
-                                                    Item* items, uint64_t items_max, Hdr* hdr,
-                                                    double split_cost, double split_scale,
-                                                    double target_items, double items_factor,
-                                                    int root_begin, int root_end) {
+// How the roots are cut into items.
+struct SplitArgs {
+  double split_cost, split_scale, target_items, items_factor, floor;
+  uint64_t items_max;
+  int root_begin, root_end;
+};
+
+// A warp takes 32 branches of a root at a time, a lane each (hub roots have more
+// and are spread over the grid's z).  Branches above twice the threshold T are
+// cut into second-level ranges; the others form first-level ranges, a new one
+// wherever the running cost passes a multiple of T, next to a cut branch and
+// every 32 branches.  A graph's items start at the sum of the
+// bounds of the graphs before it (every block adds them up: G is at most some
+// hundreds) and are handed out by an atomic counter.
+template <int K, bool CB>
+__global__ void __launch_bounds__(256) k_plan_items(const DevGraph* __restrict__ graphs, int ng,
+                                                    GraphPlan* gp,
+                                                    const int32_t* __restrict__ dsum_all, int nmax,
+                                                    Item* items, Hdr* hdr, SplitArgs a) {
+  __shared__ double red[8];
+  __shared__ unsigned long long redb[8];
+  __shared__ float s_T;
+  __shared__ uint32_t s_base;
   const int g = blockIdx.y;
-  const int lane = threadIdx.x & 31;
-  const int v = blockIdx.x * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5);
-  if (!WRITE && g == 0 && v == 0 && lane == 0) cnt[(int64_t)gridDim.y * nmax] = 0;
-  if (v >= nmax) return;
-  const int64_t slot = (int64_t)g * nmax + v;
-  const DevGraph G = graphs[g];
-  if (v >= G.n || v < root_begin || v >= root_end || v < G.root_begin || v >= G.root_end) {
-    if (!WRITE && lane == 0) cnt[slot] = 0;
-    return;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double local = 0.0;
+  for (int h = threadIdx.x; h < ng; h += blockDim.x) local += gp[h].est;
+  for (int d = 16; d; d >>= 1) local += __shfl_xor_sync(kFull, local, d);
+  if (lane == 0) red[wid] = local;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double total = 0.0;
+    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) total += red[i];
+    // root-split threshold: explicit, or the automatic one scaled; never so small
+    // that the items exceed their budget
+    const double t_auto = fmax(total / a.target_items, a.floor);
+    double T = a.split_cost > 0.0 ? a.split_cost : t_auto * a.split_scale;
+    T = fmax(fmax(T, total / (a.items_factor * a.target_items)), 1.0);
+    s_T = (float)T;
   }
-  // root-split threshold: explicit, or the automatic one scaled; never so small
-  // that the items exceed their budget
-  const double t_auto = hdr->total_est / target_items;
-  double T = split_cost > 0.0 ? split_cost : t_auto * split_scale;
-  const double t_min = hdr->total_est / (items_factor * target_items);
-  if (T < t_min) T = t_min;
-  if (T < 1.0) T = 1.0;
-  const float Tf = (float)T;
-  const int re = G.urow[v + 1];
-  const int f = G.urow[v] + G.ufwd[v];
-  const int dplus = re - f;
-  int64_t pos = WRITE ? cnt[slot] : 0;
-  int count = 0;
-  auto put = [&](int64_t at, int j1a, int j1b, int a2, int b2) {
-    if ((uint64_t)at < items_max) {
-      Item it;
-      it.g = (uint32_t)g;
-      it.root = (uint32_t)v;
-      it.j1a = (uint16_t)j1a;
-      it.j1b = (uint16_t)j1b;
-      it.a2 = (uint16_t)a2;
-      it.b2 = (uint16_t)b2;
-      items[at] = it;
-    } else {
-      atomicOr(&hdr->err, kErrStackOverflow);
-    }
-  };
-  auto emit = [&](int j1a, int j1b) {  // one whole-range item, written by lane 0
-    if (WRITE && lane == 0) put(pos, j1a, j1b, 0, 0xFFFF);
-    ++pos;
-    ++count;
-  };
-  float acc = 0.f;
-  int start = 0;
-  for (int base = 0; base < dplus; base += 32) {
-    float c_l = 0.f;
-    int x_l = 0;
-    if (base + lane < dplus) {
-      const int64_t e = (int64_t)g * stride + f + base + lane;
-      c_l = est[e];
-      x_l = x1s[e];
-    }
-    const int n = min(32, dplus - base);
-    for (int i = 0; i < n; ++i) {
-      const float c = __shfl_sync(kFull, c_l, i);
-      const int x = __shfl_sync(kFull, x_l, i);
-      const int j = base + i;
-      if (K >= 4 && c > 2.f * Tf && x >= 2) {
-        if (j > start) emit(start, j);
-        int nch = (int)ceilf(c / Tf);
-        if (nch > x) nch = x;
-        const int r2 = (x + nch - 1) / nch;
-        const int ns = (x + r2 - 1) / r2;
-        if (WRITE)
-          for (int t = lane; t < ns; t += 32) put(pos + t, j, j + 1, t * r2, min(t * r2 + r2, x));
-        pos += ns;
-        count += ns;
-        start = j + 1;
-        acc = 0.f;
+  __syncthreads();
+  const float T = s_T, inv_T = 1.f / T;
+  unsigned long long before = 0;
+  for (int h = threadIdx.x; h < g; h += blockDim.x)
+    before += (unsigned long long)(gp[h].est / (double)T * 1.001) +
+              2ull * (unsigned)(graphs[h].nu / 2) + 16ull;
+  for (int d = 16; d; d >>= 1) before += __shfl_xor_sync(kFull, before, d);
+  if (lane == 0) redb[wid] = before;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long b = 0;
+    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) b += redb[i];
+    s_base = (uint32_t)min(b, (unsigned long long)a.items_max);
+    if (blockIdx.x == 0 && blockIdx.z == 0) gp[g].base = s_base;
+  }
+  __syncthreads();
+  const uint32_t base = s_base;
+  const DevGraph G = graphs[g];
+  const int32_t* dsum = dsum_all + (int64_t)g * nmax;
+  const int r0 = max(max(a.root_begin, G.root_begin), 0);
+  const int r1 = min(min(a.root_end, G.root_end), G.n);
+  const int nwarps = (int)(gridDim.x * (blockDim.x >> 5));
+  for (int v = r0 + (int)(blockIdx.x * (blockDim.x >> 5)) + wid; v < r1; v += nwarps) {
+    const int rs = __ldg(&G.urow[v]), re = __ldg(&G.urow[v + 1]);
+    const int f = rs + __ldg(&G.ufwd[v]);
+    const int dplus = re - f;
+    auto put = [&](uint32_t at, int j1a, int j1b, int a2, int b2) {
+      const uint64_t pos = (uint64_t)base + at;
+      if (pos < a.items_max) {
+        Item it;
+        it.root = (uint32_t)v;
+        it.j1a = (uint16_t)j1a;
+        it.j1b = (uint16_t)j1b;
+        it.a2 = (uint16_t)a2;
+        it.b2 = (uint16_t)b2;
+        it.a3 = 0;
+        it.b3 = 0xFFFF;
+        items[pos] = it;
       } else {
-        acc += c;
-        if (acc >= Tf) {
-          emit(start, j + 1);
-          start = j + 1;
-          acc = 0.f;
-        }
+        atomicOr(&hdr->err, kErrStackOverflow);
+      }
+    };
+    for (int jb = 32 * (int)blockIdx.z; jb < dplus; jb += 32 * (int)gridDim.z) {
+      const int n = min(32, dplus - jb);
+      const int j = jb + lane;
+      float c = 0.f;
+      int x = 0;
+      if (lane < n) c = entry_cost<K, CB>(G, dsum, v, rs, re, f + j, x);
+      const bool cut = K >= 4 && lane < n && c > 2.f * T && x >= 2;
+      int r2 = 0, ns = 0;
+      if (cut) {
+        const int nch = min((int)ceilf(fminf(c * inv_T, 65536.f)), x);
+        r2 = (x + nch - 1) / nch;
+        ns = (x + r2 - 1) / r2;
+      }
+      float sum = cut ? 0.f : c;
+      for (int d = 1; d < 32; d <<= 1) {
+        const float y = __shfl_up_sync(kFull, sum, d);
+        if (lane >= d) sum += y;
+      }
+      const int step = (int)fminf((sum - (cut ? 0.f : c)) * inv_T, 1e9f);
+      const int step_before = __shfl_up_sync(kFull, step, 1);
+      const unsigned cuts = __ballot_sync(kFull, cut);
+      const bool start = lane < n && !cut &&
+                         (lane == 0 || (cuts >> (lane - 1) & 1u) || step != step_before);
+      const unsigned ends = cuts | __ballot_sync(kFull, start);
+      const int mine = start ? 1 : ns;
+      const int incl = warp_incl_scan(mine);
+      uint32_t at = 0;
+      const int all = __shfl_sync(kFull, incl, 31);
+      if (lane == 0 && all) at = atomicAdd(&gp[g].count, (uint32_t)all);
+      at = __shfl_sync(kFull, at, 0);
+      if (start) {
+        const unsigned later = lane == 31 ? 0u : ends >> (lane + 1);
+        const int end = later ? lane + __ffs(later) : n;
+        put(at + incl - 1, j, jb + end, 0, 0xFFFF);
+      }
+      for (unsigned q = cuts; q; q &= q - 1) {
+        const int l = __ffs(q) - 1;
+        const int ns_l = __shfl_sync(kFull, ns, l), r_l = __shfl_sync(kFull, r2, l);
+        const int x_l = __shfl_sync(kFull, x, l);
+        const uint32_t at_l = at + (uint32_t)(__shfl_sync(kFull, incl, l) - ns_l);
+        for (int t = lane; t < ns_l; t += 32)
+          put(at_l + t, jb + l, jb + l + 1, t * r_l, min(t * r_l + r_l, x_l));
       }
     }
   }
-  if (start < dplus) emit(start, dplus);
-  if (!WRITE && lane == 0) cnt[slot] = count;
-}
-
-__global__ void __launch_bounds__(1024) k_scan_counts(int32_t* data, int count) {
-  __shared__ int tmp[33];
-  block_exclusive_scan(data, count, tmp);
 }
 
 // ------------------------------------------------------------------ enumerator
@@ -428,8 +508,7 @@ __global__ void __launch_bounds__(256) k_fold_copies(unsigned long long* __restr
 struct CountArgs {
   const DevGraph* graphs;
   const Item* items;
-  const int32_t* item_off;   // scanned item counts: graph g owns [item_off[g*nmax], item_off[(g+1)*nmax])
-  uint32_t* qhead;           // per-graph queue heads
+  GraphPlan* gp;             // per graph: its items and its queue's head
   Hdr* hdr;
   const uint32_t* table;
   const uint16_t* xclass;    // compact k = 6 table: prefix key -> class of the first 4 vertices
@@ -594,8 +673,8 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
       if (cp) ghist = a.hist_copies + (size_t)(cp - 1) * a.copy_stride;
     }
     const int32_t* ufwd = Gp->ufwd;
-    const int ib = a.item_off[(int64_t)g * a.nmax];
-    const int ie = a.item_off[(int64_t)(g + 1) * a.nmax];
+    const uint32_t nitems = a.gp[g].count;
+    const Item* my_items = a.items + a.gp[g].base;
 
     // Adds of the cell method, which may be negative (corrections).  For k <= 5
     // the shared 32-bit counters take deltas below 2^20 under the add budget
@@ -919,11 +998,10 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
     // The warp's next item: the graph's queue, then donated items.
     auto next_item = [&](Item& out) -> bool {
       uint32_t idx = 0;
-      if (lane == 0) idx = atomicAdd(&a.qhead[g], 1u);
+      if (lane == 0) idx = atomicAdd(&a.gp[g].qhead, 1u);
       idx = __shfl_sync(kFull, idx, 0);
-      const int64_t pos = (int64_t)ib + idx;
-      if (pos < ie) {
-        out = a.items[pos];
+      if (idx < nitems) {
+        out = my_items[idx];
         return true;
       }
       uint4 raw = make_uint4(0, 0, 0, 0);
@@ -977,7 +1055,7 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
       int cur_e = min(dplus - j1a, w.cap);
       int cur_c = 0, cur_ce = min(j1b - j1a, cur_e);
       uint32_t cur_key = 0;
-      const bool has2 = it.b2 != 0xFFFF;
+      const bool has2 = it.b2 != 0xFFFF, has3 = it.b3 != 0xFFFF;
       // The enumerator's slot codes (bits of positions k-2 and up) are not
       // cleared by row scans: the tail pass writes each candidate back
       // without them, and a candidate list is cleaned once when its level
@@ -1206,10 +1284,11 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
         if (c < ce) {
           // work donation: with an idle warp in the block, hand the second
           // half of this level's remaining choices over as a new item (a
-          // first-level range, or a second-level range under the current
-          // first-level choice)
+          // range of this level under the current choices of the levels above).
+          // At k = 6 that includes the third level: one second-level choice that
+          // reaches a hub can hold more work than a warp's share of a launch.
           int cee = ce;
-          if (L <= 2 && L < K - 2 && ce - c >= 2) {
+          if (L <= 3 && L < K - 2 && ce - c >= 2) {
             int hungry = 0;
             if (lane == 0) hungry = *v_idle > 0 && *v_ndon < kDonSlots;
             hungry = __shfl_sync(kFull, hungry, 0);
@@ -1218,19 +1297,26 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
               int ok = 0;
               if (lane == 0) {
                 Item d;
-                d.g = (uint32_t)g;
                 d.root = (uint32_t)v;
+                d.a2 = d.a3 = 0;
+                d.b2 = d.b3 = 0xFFFF;
                 if (L == 1) {
                   d.j1a = (uint16_t)(j1a + mid);
                   d.j1b = (uint16_t)(j1a + ce);
-                  d.a2 = 0;
-                  d.b2 = 0xFFFF;
                 } else {
                   const int c1 = lvs[5] - 1;  // index of the first-level choice
                   d.j1a = (uint16_t)(j1a + c1);
                   d.j1b = (uint16_t)(j1a + c1 + 1);
-                  d.a2 = (uint16_t)(mid - (c1 + 1));
-                  d.b2 = (uint16_t)(ce - (c1 + 1));
+                  if (L == 2) {
+                    d.a2 = (uint16_t)(mid - (c1 + 1));
+                    d.b2 = (uint16_t)(ce - (c1 + 1));
+                  } else {
+                    const int c2 = lvs[10] - 1;  // and of the second-level choice
+                    d.a2 = (uint16_t)(c2 - (c1 + 1));
+                    d.b2 = (uint16_t)(c2 - c1);
+                    d.a3 = (uint16_t)(mid - (c2 + 1));
+                    d.b3 = (uint16_t)(ce - (c2 + 1));
+                  }
                 }
                 if (block_lock()) {
                   const int nd = *v_ndon;
@@ -1271,6 +1357,10 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
             cur_c = c + 1 + it.a2;
             cur_ce = min(c + 1 + (int)it.b2, ne);
           }
+          if (K == 6 && L == 2 && has3) {
+            cur_c = c + 1 + it.a3;
+            cur_ce = min(c + 1 + (int)it.b3, ne);
+          }
           L += 1;
           if (L == K - 2) fresh = true;
         } else {
@@ -1307,8 +1397,7 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
       int next = -1;
       for (int t = 1; t <= a.G; ++t) {
         const int g2 = (g + t) % a.G;
-        const int n2 = a.item_off[(int64_t)(g2 + 1) * a.nmax] - a.item_off[(int64_t)g2 * a.nmax];
-        if ((int)*(volatile uint32_t*)&a.qhead[g2] < n2) {
+        if (*(volatile uint32_t*)&a.gp[g2].qhead < a.gp[g2].count) {
           next = g2;
           break;
         }
@@ -1347,8 +1436,6 @@ static const void* pick_kernel(int K, bool gc, bool ls, bool cb, bool sg) {
   }
 }
 
-constexpr int kCellsAboveK4 = 4096;  // k = 4: vertices above which cells are faster
-
 mt_status count_configure_tuned(CountPlan* p, int K, int G, int nmax, int dmax, int64_t fwd_bound,
                                 int64_t entry_stride, uint32_t classes, const mt_tuning* tuning,
                                 bool compact, int method) {
@@ -1373,15 +1460,13 @@ mt_status count_configure_tuned(CountPlan* p, int K, int G, int nmax, int dmax, 
                                              : std::max(K - 2, 1) * std::max(dmax, 1) + 32;
   if (p->cap > 65535) return MT_EUNSUPPORTED;
   p->nu_cap = (int)p->entry_stride;
-  // The library's own choice: the cell method where it is the faster one (it
-  // counts the same histogram from the (k-2)-sets instead of from every k-set).
-  // Measured on a GB300, per-subgraph against cells: one k = 6 graph (n = 800)
-  // 4.6 : 1.6 ms and 65 of them 135 : 71 ms, one k = 5 graph (n = 1,500) 2.7 :
-  // 1.3 ms and 257 of them 526 : 187 ms, small graphs at k = 5 (n = 112 to 310)
-  // 1.1 to 1.2 times faster; k = 4 at n = 6,437 0.94 : 0.69 ms but at n = 3,646
-  // 0.64 : 0.68 and at n = 2,000 0.39 : 0.45 ms; at k = 3 a few per cent slower.
-  if (method == kAutoMethod)
-    method = K >= 5 || (K == 4 && nmax > kCellsAboveK4) ? MT_METHOD_CELLS : MT_METHOD_ENUMERATE;
+  // The library's own choice counts the same histogram from the (k-2)-sets
+  // instead of from every k-set.  Measured on a GB300, per-subgraph against
+  // cells: k = 6 one graph (n = 800) 2.3 : 1.2 ms, 65 of them 135 : 71 ms; k = 5
+  // one graph (n = 1,500) 2.4 : 0.88 ms, 257 of them 526 : 187 ms; k = 4 n = 239 /
+  // 2,000 / 3,646 59 : 59, 235 : 119, 455 : 163 us; k = 3 n = 122 / 300 / 20,000
+  // 57 : 58, 58 : 60, 289 : 144 us.
+  if (method == kAutoMethod) method = MT_METHOD_CELLS;
   else if (compact && method == MT_METHOD_CELLS)
     return MT_EUNSUPPORTED;
   p->comb = method == MT_METHOD_CELLS;
@@ -1478,13 +1563,13 @@ mt_status count_configure_tuned(CountPlan* p, int K, int G, int nmax, int dmax, 
   if (occ < 1) return MT_EUNSUPPORTED;
   p->blocks = sms * occ;
   const double target = (double)p->blocks * p->warps_per_block * kTargetItemsPerWarp;
-  p->items_max = (uint64_t)(target * p->items_factor) + (uint64_t)G * nmax +
+  p->items_max = (uint64_t)(target * p->items_factor * 1.01) + 16 * (uint64_t)G +
                  2 * (uint64_t)fwd_bound + 4096;
   size_t off = 0;
   p->off_hdr = off; off += 256;
-  p->off_qhead = off; off += round16((size_t)G * 4);
-  p->off_est = off; off += round16((size_t)G * p->entry_stride * 4) * 2;
-  p->off_cnt = off; off += round16(((size_t)G * nmax + 1) * 4);
+  p->off_gp = off; off += round16((size_t)G * sizeof(GraphPlan));
+  p->off_dsum = off;
+  if (p->comb && K >= 5) off += round16((size_t)G * nmax * 4);
   p->off_items = off; off += round16(p->items_max * sizeof(Item));
   p->off_lab = off;
   if (!p->lab_smem) off += (size_t)p->blocks * p->warps_per_block * lab_bytes;
@@ -1498,7 +1583,7 @@ uint32_t* count_err_ptr(const CountPlan& p, void* ws) {
   return &((Hdr*)((char*)ws + p.off_hdr))->err;
 }
 uint32_t* count_nitems_ptr(const CountPlan& p, void* ws) {
-  return (uint32_t*)((char*)ws + p.off_cnt) + (size_t)p.G * p.nmax;
+  return &((GraphPlan*)((char*)ws + p.off_gp))->count;
 }
 
 template <int K, bool CB>
@@ -1521,28 +1606,37 @@ static cudaError_t enqueue_k(const CountPlan& p, void* ws, const DevGraph* graph
                              unsigned long long* copies_base, int copies, uint32_t copy_stride) {
   char* base = (char*)ws;
   Hdr* hdr = (Hdr*)(base + p.off_hdr);
-  uint32_t* qhead = (uint32_t*)(base + p.off_qhead);
-  float* est = (float*)(base + p.off_est);
-  int32_t* x1s = (int32_t*)(base + p.off_est + round16((size_t)p.G * p.entry_stride * 4));
-  int32_t* cnt = (int32_t*)(base + p.off_cnt);
+  GraphPlan* gp = (GraphPlan*)(base + p.off_gp);
   Item* items = (Item*)(base + p.off_items);
   void* lab = base + p.off_lab;
-  cudaError_t e = cudaMemsetAsync(hdr, 0, sizeof(Hdr), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(qhead, 0, (size_t)p.G * 4, s);
+  // header and graph plans are neighbours
+  cudaError_t e = cudaMemsetAsync(base + p.off_hdr, 0,
+                                  p.off_gp - p.off_hdr + (size_t)p.G * sizeof(GraphPlan), s);
   if (e != cudaSuccess) return e;
+  SplitArgs sa;
+  sa.split_cost = p.split_cost;
+  sa.split_scale = p.split_scale;
+  sa.target_items = (double)p.blocks * p.warps_per_block * kTargetItemsPerWarp;
+  sa.items_factor = p.items_factor;
+  sa.floor = p.comb ? kCellsItemFloor<K> : 1.0;
+  sa.items_max = p.items_max;
+  sa.root_begin = rb;
+  sa.root_end = re;
   const int ex = (int)std::min<int64_t>((p.entry_stride + 255) / 256, 4096);
-  k_plan_est<K><<<dim3(ex, p.G), 256, 0, s>>>(graphs, p.entry_stride, est, x1s, hdr, rb, re);
-  const int rx = (p.nmax + 7) / 8;  // one warp per root, 8 per block
-  const double target = (double)p.blocks * p.warps_per_block * kTargetItemsPerWarp;
-  k_plan_items<K, false><<<dim3(rx, p.G), 256, 0, s>>>(graphs, p.entry_stride, est, x1s, p.nmax,
-                                                       cnt, items, p.items_max, hdr, p.split_cost,
-                                                       p.split_scale, target, p.items_factor, rb,
-                                                       re);
-  k_scan_counts<<<1, 1024, 0, s>>>(cnt, p.G * p.nmax + 1);
-  k_plan_items<K, true><<<dim3(rx, p.G), 256, 0, s>>>(graphs, p.entry_stride, est, x1s, p.nmax,
-                                                      cnt, items, p.items_max, hdr, p.split_cost,
-                                                      p.split_scale, target, p.items_factor, rb,
-                                                      re);
+  // one warp per root, until the grid holds some thousands of blocks
+  const int rx = std::max(1, std::min((p.nmax + 7) / 8, std::max(4096 / p.G, 4)));
+  const int rz = std::max(1, std::min(8, std::min((p.dmax + 31) / 32, 64 / p.G)));
+  int32_t* dsum = (int32_t*)(base + p.off_dsum);
+  if (p.comb) {
+    if (K >= 5) k_plan_degsum<<<dim3(rx, p.G), 256, 0, s>>>(graphs, p.nmax, dsum);
+    k_plan_total<K, true><<<dim3(ex, p.G), 256, 0, s>>>(graphs, gp, dsum, p.nmax, rb, re);
+    k_plan_items<K, true><<<dim3(rx, p.G, rz), 256, 0, s>>>(graphs, p.G, gp, dsum, p.nmax, items, hdr,
+                                                        sa);
+  } else {
+    k_plan_total<K, false><<<dim3(ex, p.G), 256, 0, s>>>(graphs, gp, dsum, p.nmax, rb, re);
+    k_plan_items<K, false><<<dim3(rx, p.G, rz), 256, 0, s>>>(graphs, p.G, gp, dsum, p.nmax, items, hdr,
+                                                         sa);
+  }
   if (!p.lab_smem) {
     e = cudaMemsetAsync(lab, 0, (size_t)p.blocks * p.warps_per_block * p.lab_bytes, s);
     if (e != cudaSuccess) return e;
@@ -1550,8 +1644,7 @@ static cudaError_t enqueue_k(const CountPlan& p, void* ws, const DevGraph* graph
   CountArgs a;
   a.graphs = graphs;
   a.items = items;
-  a.item_off = cnt;
-  a.qhead = qhead;
+  a.gp = gp;
   a.hdr = hdr;
   a.table = table.slots;
   a.xclass = p.compact ? table.xclass : nullptr;

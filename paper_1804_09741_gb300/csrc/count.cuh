@@ -38,7 +38,7 @@ struct CountPlan {
   uint32_t classes = 0;
   size_t ws_bytes = 0;
   // workspace offsets
-  size_t off_hdr = 0, off_qhead = 0, off_est = 0, off_cnt = 0, off_items = 0, off_lab = 0;
+  size_t off_hdr = 0, off_gp = 0, off_dsum = 0, off_items = 0, off_lab = 0;
   size_t off_stack = 0;
 };
 

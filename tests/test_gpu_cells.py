@@ -67,12 +67,30 @@ def test_per_subgraph_counts_equal_oracle(lib, k):
     t.free()
 
 
-@pytest.mark.parametrize("n", [4096, 4097])
-def test_automatic_method_around_its_line(lib, n):
-    """k = 4 changes method above 4,096 vertices: both sides equal the oracle."""
+@pytest.mark.parametrize("n", [4096, 16383, 16384, 16385])
+def test_large_graphs_equal_oracle(lib, n):
+    """Sizes around the 16-bit graph copy's limit (2^14 vertices)."""
     lib.load_library()
     t = lib.table_build(4)
     g = syn.chung_lu_digraph(n, 2 * n, 2.4, 60, 0.1, 9)
     want = oracle_dense(oracle.count(g, 4)[0], t.class_masks())
     np.testing.assert_array_equal(lib.count_host(lib.graph_from(g), t), want)
+    t.free()
+
+
+@pytest.mark.parametrize("k", [4, 5, 6])
+def test_one_branch_holds_the_work(lib, k):
+    """A path into a hub: one branch, and one of its choices, hold nearly all of
+    the work, so it is cut and handed over at every level (third at k = 6)."""
+    lib.load_library()
+    t = lib.table_build(k)
+    leaves = {4: 400, 5: 120, 6: 60}[k]
+    src = [0, 1, 2] + [3] * leaves
+    dst = [1, 2, 3] + list(range(4, 4 + leaves))
+    g = syn.csr_from_arcs(4 + leaves, src, dst)
+    want = oracle_dense(oracle.count(g, k)[0], t.class_masks())
+    for perm in (np.arange(g.n), np.arange(g.n)[::-1]):
+        dg = lib.graph_from(syn.relabel(g, perm))
+        for _ in range(3):
+            np.testing.assert_array_equal(lib.count_host(dg, t), want)
     t.free()

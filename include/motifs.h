@@ -13,13 +13,15 @@
  * Conventions shared by every entry point
  * ---------------------------------------
  * - Every function returns an mt_status and never aborts; no C++ exception
- *   crosses this boundary.  Input errors are reported as MT_EINVAL before any
- *   device work starts.
+ *   crosses this boundary.  Input errors are reported as MT_EINVAL, before any
+ *   device work starts except where a function says that the device finds them.
  * - `stream` is a cudaStream_t passed as void* (NULL = the legacy default
  *   stream).  Work is enqueued on it; unless a function says it synchronises,
  *   results are valid after the stream is synchronised.
  * - Handles (mt_graph, mt_table, mt_batch) own device memory the library
- *   allocated; the caller frees them with the matching *_free.  Buffers passed
+ *   allocated; the caller frees them with the matching *_free.  Graphs and
+ *   scratch come from a memory pool per device, which keeps up to 128 MiB of
+ *   freed memory for the next ones while any graph or table is alive.  Buffers passed
  *   in by the caller stay the caller's.  Pointers documented as "device or host"
  *   are inspected with cudaPointerGetAttributes: a device pointer keeps the call
  *   asynchronous, a host pointer makes the call copy and synchronise the stream.
@@ -87,7 +89,8 @@ const char* mt_last_error(void);
  * copies them into device memory it owns, then builds on the device the sorted
  * directed CSR and the undirected neighbour CSR in which every entry carries
  * the 2-bit relation of Sec. 2 (A: both arcs, B: v->u only, C: u->v only).
- * Synchronises `stream` (a duplicate arc is detected on the device).
+ * Synchronises `stream` (self-loops and duplicate arcs are detected on the
+ * device).
  * Errors: MT_EINVAL (null pointers, n < 1, m < 0, row_ptr[0] != 0,
  * row_ptr[n] != m, decreasing row_ptr, id out of range, self-loop, duplicate
  * arc), MT_EUNSUPPORTED (n > 65535), MT_ENOMEM, MT_ECUDA.  *out is set only on

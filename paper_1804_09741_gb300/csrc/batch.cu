@@ -3,7 +3,7 @@
 // per-class z-scores.
 //
 // One step is:  randomise R graphs (K3, one block per graph) -> rebuild their
-// sorted and undirected CSRs (K4, one block per graph) -> zero the R+1
+// undirected CSRs (K4, all graphs together) -> zero the R+1
 // histograms -> plan work items over all R+1 graphs -> one persistent
 // enumerate-and-classify launch over all items of all graphs (K2) -> z-scores
 // (K5).  The step is captured once into a CUDA graph and replayed.
@@ -36,10 +36,9 @@ struct mt_batch {
   void* mem = nullptr;
   size_t mem_bytes = 0;
   // views into mem
-  int32_t *col_rand = nullptr, *col_sorted = nullptr, *urow = nullptr, *usrc = nullptr,
-          *ufwd = nullptr;
-  uint32_t* ucol = nullptr;
-  int32_t *in_ptr = nullptr, *in_tmp = nullptr, *in_col = nullptr, *cursor = nullptr;
+  int32_t *col_rand = nullptr, *urow = nullptr, *usrc = nullptr, *ufwd = nullptr;
+  uint32_t *ucol = nullptr, *tmp = nullptr;
+  int32_t* cursor = nullptr;
   mt::BuildStats* stats = nullptr;
   uint32_t* rand_scratch = nullptr;
   int null_model = MT_NULL_ARC_SWAP;
@@ -126,14 +125,11 @@ static mt_status batch_create(const mt_graph* g0, const mt_table* t, int R, uint
     return o;
   };
   const size_t o_col_rand = take((size_t)R * m1 * 4);
-  const size_t o_col_sorted = take((size_t)R * m1 * 4);
   const size_t o_urow = take((size_t)R * (n + 1) * 4);
   const size_t o_ucol = take((size_t)R * 2 * m1 * 4);
   const size_t o_usrc = take((size_t)R * 2 * m1 * 4);
   const size_t o_ufwd = take((size_t)R * n * 4);
-  const size_t o_in_ptr = take((size_t)R * (n + 1) * 4);
-  const size_t o_in_tmp = take((size_t)R * m1 * 4);
-  const size_t o_in_col = take((size_t)R * m1 * 4);
+  const size_t o_tmp = take((size_t)R * 2 * m1 * 4);
   const size_t o_cursor = take((size_t)R * n * 4);
   const size_t o_stats = take((size_t)R * sizeof(BuildStats));
   const size_t o_rs = take(rs_words * 4);
@@ -153,14 +149,11 @@ static mt_status batch_create(const mt_graph* g0, const mt_table* t, int R, uint
   }
   char* base = (char*)b->mem;
   b->col_rand = (int32_t*)(base + o_col_rand);
-  b->col_sorted = (int32_t*)(base + o_col_sorted);
   b->urow = (int32_t*)(base + o_urow);
   b->ucol = (uint32_t*)(base + o_ucol);
   b->usrc = (int32_t*)(base + o_usrc);
   b->ufwd = (int32_t*)(base + o_ufwd);
-  b->in_ptr = (int32_t*)(base + o_in_ptr);
-  b->in_tmp = (int32_t*)(base + o_in_tmp);
-  b->in_col = (int32_t*)(base + o_in_col);
+  b->tmp = (uint32_t*)(base + o_tmp);
   b->cursor = (int32_t*)(base + o_cursor);
   b->stats = (BuildStats*)(base + o_stats);
   b->rand_scratch = rs_words ? (uint32_t*)(base + o_rs) : nullptr;
@@ -188,7 +181,7 @@ static mt_status batch_create(const mt_graph* g0, const mt_table* t, int R, uint
     d.root_end = n;
     d.pad = 0;
     d.row_ptr = g0->row_ptr;
-    d.col = b->col_sorted + (size_t)r * m1;
+    d.col = b->col_rand + (size_t)r * m1;  // rows in any order
     d.urow = b->urow + (size_t)r * (n + 1);
     d.ucol = b->ucol + (size_t)r * 2 * m1;
     d.usrc = b->usrc + (size_t)r * 2 * m1;
@@ -211,7 +204,6 @@ static mt_status batch_create(const mt_graph* g0, const mt_table* t, int R, uint
 static mt_status batch_enqueue(mt_batch* b, cudaStream_t s) {
   const int R = b->R;
   const int32_t n = b->n, m = b->m;
-  const size_t m1 = (size_t)std::max(m, 1);
   MT_CUDA_TRY(cudaMemcpyAsync(b->d_seeds, b->h_seeds, (size_t)R * 8, cudaMemcpyHostToDevice, s));
   MT_CUDA_TRY(cudaEventRecordWithFlags(b->ev[0], s, cudaEventRecordExternal));
   if (b->null_model == MT_NULL_DYAD_SWAP)
@@ -222,17 +214,18 @@ static mt_status batch_enqueue(mt_batch* b, cudaStream_t s) {
                                  b->col_rand, b->rand_scratch, s));
   BuildArgs a;
   a.n = n; a.m = m; a.G = R;
-  a.row_ptr = b->g0->row_ptr; a.row_stride = 0;
-  a.col_in = b->col_rand; a.col_out = b->col_sorted;
-  a.in_ptr = b->in_ptr; a.in_tmp = b->in_tmp; a.in_col = b->in_col; a.cursor = b->cursor;
+  a.row_ptr = b->g0->row_ptr;
+  a.col_in = b->col_rand;
+  a.rank = b->g0->rank; a.off = b->g0->off;  // the null graphs keep the degrees
+  a.tmp = b->tmp; a.cursor = b->cursor;
   a.urow = b->urow; a.ucol = b->ucol; a.usrc = b->usrc; a.ufwd = b->ufwd; a.stats = b->stats;
-  (void)m1;
   MT_CUDA_TRY(launch_build(a, s));
   k_fill_nu<<<(R + 255) / 256, 256, 0, s>>>(b->d_graphs + 1, b->stats, R);
   MT_CUDA_TRY(cudaGetLastError());
   MT_CUDA_TRY(cudaEventRecordWithFlags(b->ev[1], s, cudaEventRecordExternal));
   MT_CUDA_TRY(cudaMemsetAsync(b->d_hists, 0, (size_t)(R + 1) * b->C * 8, s));
   if (n >= b->K) MT_TRY(count_enqueue(b->plan, b->ws, b->d_graphs, table_view(b->t), 0, n, s));
+  else MT_CUDA_TRY(cudaMemsetAsync(count_err_ptr(b->plan, b->ws), 0, 4, s));  // no launch sets it
   MT_CUDA_TRY(cudaEventRecordWithFlags(b->ev[2], s, cudaEventRecordExternal));
   k_zscore<<<(b->C + 255) / 256, 256, 0, s>>>(b->d_hists, R, b->C, b->d_z);
   MT_CUDA_TRY(cudaGetLastError());

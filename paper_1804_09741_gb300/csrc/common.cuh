@@ -19,6 +19,7 @@ constexpr uint32_t kNumClasses[7] = {0, 1, 2, 13, 199, 9364, 1530843};
 // Error bits written by kernels into a device status word.
 constexpr uint32_t kErrStackOverflow = 1u;
 constexpr uint32_t kErrDuplicateArc = 2u;
+constexpr uint32_t kErrSelfLoop = 8u;
 constexpr uint32_t kErrWaitLimit = 4u;  // a bounded device wait gave up
 
 // Undirected neighbour entry: vertex id in bits 0..29, bit 30 set iff the arc
@@ -96,16 +97,27 @@ __device__ __forceinline__ int warp_incl_scan(int x) {
 
 // Exclusive prefix sum of data[0..count) in place, by one thread block (any
 // blockDim multiple of 32, <= 1024); returns the total to every thread.  `tmp`
-// is shared scratch of 33 ints.  All threads of the block must call it.
+// is shared scratch of 33 ints.  All threads of the block must call it.  A
+// thread takes kPer values of a tile, its reads in flight together: with one
+// value per thread and tile 20,000 values took 19 us.
 __device__ inline long long block_exclusive_scan(int32_t* data, int count, int* tmp) {
+  constexpr int kPer = 8;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int nw = blockDim.x >> 5;
   long long carry = 0;
-  for (int base = 0; base < count; base += blockDim.x) {
-    int i = base + tid;
-    int x = i < count ? data[i] : 0;
-    int inc = warp_incl_scan(x);
-    if (lane == 31) tmp[wid] = inc;
+  for (int base = 0; base < count; base += kPer * (int)blockDim.x) {
+    // warp-contiguous: value j of a lane is at its warp's first + 32 j + lane
+    const int at = base + wid * 32 * kPer + lane;
+    int x[kPer], sum = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) x[j] = at + 32 * j < count ? data[at + 32 * j] : 0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+      const int inc = warp_incl_scan(x[j]);
+      x[j] = sum + inc - x[j];
+      sum += __shfl_sync(0xFFFFFFFFu, inc, 31);
+    }
+    if (lane == 0) tmp[wid] = sum;
     __syncthreads();
     if (wid == 0) {
       int s = lane < nw ? tmp[lane] : 0;
@@ -114,7 +126,9 @@ __device__ inline long long block_exclusive_scan(int32_t* data, int count, int* 
       if (lane == nw - 1) tmp[32] = si;
     }
     __syncthreads();
-    if (i < count) data[i] = (int32_t)(carry + tmp[wid] + inc - x);
+#pragma unroll
+    for (int j = 0; j < kPer; ++j)
+      if (at + 32 * j < count) data[at + 32 * j] = (int32_t)(carry + tmp[wid] + x[j]);
     carry += tmp[32];
     __syncthreads();
   }

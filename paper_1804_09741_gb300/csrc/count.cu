@@ -641,21 +641,25 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
       const int32_t* grow = Gp->urow;
       const uint32_t* gcol = Gp->ucol;
       if (COMB) {
-        // rows start at multiples of kSeg entries, padded with zeros
+        // rows start at multiples of kSeg entries, padded with zeros; an entry
+        // per thread, so that the loads of a whole copy are in flight together
+        const int32_t* gsrc = Gp->usrc;
+        uint4* words = (uint4*)s_ucol;
+        const int nwords = (int)((unsigned char*)s_hist - (unsigned char*)s_ucol) / 16;
+        for (int i = tid; i < nwords; i += blockDim.x) words[i] = make_uint4(0, 0, 0, 0);
         for (int i = tid; i <= n; i += blockDim.x)
           s_urow[i] = i < n ? (grow[i + 1] - grow[i] + kSeg - 1) / kSeg : 0;
         __syncthreads();
         block_exclusive_scan(s_urow, n + 1, s_scan);
-        for (int x = wid; x < n; x += nwarps) {
-          const int at = s_urow[x], g0 = grow[x], len = grow[x + 1] - g0;
-          const int pad = (len + kSeg - 1) / kSeg * kSeg;
-          for (int i = lane; i < pad; i += 32) {
-            const uint32_t ent = i < len ? gcol[g0 + i] : 0u;
-            s_ucol[at * kSeg + i] = (ET)(ent_vertex(ent) | (ent_code(ent) << 14));
-          }
-          __syncwarp();
-          if (lane == 0) s_urow[x] = (int32_t)(((uint32_t)at << 16) | (uint32_t)len);
+        for (int i = tid; i < nu; i += blockDim.x) {
+          const int x = gsrc[i];
+          const uint32_t ent = gcol[i];
+          s_ucol[s_urow[x] * kSeg + (i - grow[x])] =
+              (ET)(ent_vertex(ent) | (ent_code(ent) << 14));
         }
+        __syncthreads();
+        for (int i = tid; i < n; i += blockDim.x)
+          s_urow[i] = (int32_t)(((uint32_t)s_urow[i] << 16) | (uint32_t)(grow[i + 1] - grow[i]));
       } else {
         for (int i = tid; i <= n; i += blockDim.x) s_urow[i] = grow[i];
         for (int i = tid; i < nu; i += blockDim.x) s_ucol[i] = (ET)gcol[i];
@@ -1624,12 +1628,17 @@ static cudaError_t enqueue_k(const CountPlan& p, void* ws, const DevGraph* graph
   sa.root_end = re;
   const int ex = (int)std::min<int64_t>((p.entry_stride + 255) / 256, 4096);
   // one warp per root, until the grid holds some thousands of blocks
-  const int rx = std::max(1, std::min((p.nmax + 7) / 8, std::max(4096 / p.G, 4)));
-  const int rz = std::max(1, std::min(8, std::min((p.dmax + 31) / 32, 64 / p.G)));
+  const int rx = std::max(1, std::min((p.nmax + 7) / 8, std::max(2048 / p.G, 4)));
+  const int rz = std::max(1, std::min(8, std::min((p.dmax + 31) / 32, 2048 / (rx * p.G))));
   int32_t* dsum = (int32_t*)(base + p.off_dsum);
   if (p.comb) {
     if (K >= 5) k_plan_degsum<<<dim3(rx, p.G), 256, 0, s>>>(graphs, p.nmax, dsum);
-    k_plan_total<K, true><<<dim3(ex, p.G), 256, 0, s>>>(graphs, gp, dsum, p.nmax, rb, re);
+    // One graph whose whole work is below the items' floor whatever its rows are:
+    // the threshold is the floor (an upper bound of the total stands for it).
+    const double most = (double)(p.entry_stride / 2 + 1) * (72.0 + 4.0 * p.dmax);
+    const bool known = K <= 4 && p.G == 1 && p.split_cost == 0.0 && p.split_scale == 1.0 &&
+                       most <= sa.floor * sa.target_items;
+    if (!known) k_plan_total<K, true><<<dim3(ex, p.G), 256, 0, s>>>(graphs, gp, dsum, p.nmax, rb, re);
     k_plan_items<K, true><<<dim3(rx, p.G, rz), 256, 0, s>>>(graphs, p.G, gp, dsum, p.nmax, items, hdr,
                                                         sa);
   } else {
@@ -1720,14 +1729,21 @@ static mt_status count_one(const mt_graph* gc, const mt_table* t, uint64_t* hist
     return MT_EINVAL;
   }
   if (g->ws_bytes < need) {
+    // scratch outlives a captured launch, so it is not allocated by one
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    MT_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
+    if (cap != cudaStreamCaptureStatusNone) {
+      set_last_error("the first count of a graph allocates scratch: not under stream capture");
+      return MT_ECUDA;
+    }
     if (g->ws) {
       // an earlier count may still use the old scratch, on any stream
       MT_CUDA_TRY(cudaDeviceSynchronize());
-      cudaFree(g->ws);
+      pool_free(g->ws, s);
       g->ws = nullptr;
       g->ws_bytes = 0;
     }
-    MT_CUDA_TRY(cudaMalloc(&g->ws, need));
+    MT_CUDA_TRY(pool_alloc(&g->ws, need, s));
     g->ws_bytes = need;
   }
   if (!g->ev0) {
@@ -1751,7 +1767,13 @@ static mt_status count_one(const mt_graph* gc, const mt_table* t, uint64_t* hist
   }
   unsigned long long* dh =
       dev_hist ? (unsigned long long*)hist : (unsigned long long*)(base + p.ws_bytes + 256);
-  DevGraph hg = dev_view(g, dh);
+  // a part of the roots: sets belong to their smallest original vertex
+  const bool part = rb > 0 || re < g->n;
+  if (part && g->n >= K && rb < re) {
+    if (original_scratch_bytes(g) > p.ws_bytes - p.off_items) return MT_EOVERFLOW;
+    MT_TRY(graph_build_original(g, base + p.off_items, s));  // before the items are written
+  }
+  DevGraph hg = dev_view(g, dh, part);
   MT_CUDA_TRY(cudaMemcpyAsync(dg, &hg, sizeof(DevGraph), cudaMemcpyHostToDevice, s));
   MT_CUDA_TRY(cudaMemsetAsync(dh, 0, (size_t)C * 8, s));
   if (g->n >= K && rb < re) {
@@ -1769,6 +1791,8 @@ static mt_status count_one(const mt_graph* gc, const mt_table* t, uint64_t* hist
     }
     MT_CUDA_TRY(cudaEventRecord(g->ev1, s));
   } else {
+    // no launch: the status word and the item count are read all the same
+    MT_CUDA_TRY(cudaMemsetAsync(base + p.off_hdr, 0, p.off_gp - p.off_hdr + sizeof(GraphPlan), s));
     MT_CUDA_TRY(cudaEventRecord(g->ev0, s));
     MT_CUDA_TRY(cudaEventRecord(g->ev1, s));
   }
@@ -1861,7 +1885,7 @@ mt_status mt_set_workspace(mt_graph* g, void* ws, size_t bytes) {
   }
   // an earlier count may still use the current scratch, on any stream
   MT_CUDA_TRY(cudaDeviceSynchronize());
-  if (g->ws && g->ws_owned) cudaFree(g->ws);
+  if (g->ws && g->ws_owned) pool_free(g->ws, nullptr);
   g->ws = ws;
   g->ws_bytes = ws ? bytes : 0;
   g->ws_owned = ws == nullptr;

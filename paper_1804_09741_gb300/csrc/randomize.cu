@@ -573,9 +573,6 @@ cudaError_t launch_randomize(int32_t n, int32_t m, int G, const int32_t* row_ptr
   return launch_rand(k_randomize<false>, k_randomize<true>, a, m, G, gscratch, s);
 }
 
-mt_status graph_alloc(int32_t n, int32_t m, mt_graph** out);
-mt_status graph_build_sync(mt_graph* g, const int32_t* col_in, cudaStream_t s);
-
 }  // namespace mt
 
 using namespace mt;
@@ -588,14 +585,14 @@ mt_status mt_randomize(const mt_graph* src, uint64_t seed, uint64_t swaps, void*
   TraceRange tr("mt_randomize");
   cudaStream_t s = (cudaStream_t)stream;
   mt_graph* g = nullptr;
-  MT_TRY(graph_alloc(src->n, src->m, &g));
+  MT_TRY(graph_alloc(src->n, src->m, s, &g));
   const size_t m1 = (size_t)(src->m > 0 ? src->m : 1);
   const size_t gwords = rand_gscratch_words(src->m, 1);
   char* scratch = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&scratch, m1 * 4 + 16 + gwords * 4 + 16, s);
+  cudaError_t e = pool_alloc((void**)&scratch, m1 * 4 + 16 + gwords * 4 + 16, s);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(g->row_ptr, src->row_ptr, (size_t)(src->n + 1) * 4,
-                        cudaMemcpyDeviceToDevice, s);
+    e = cudaMemcpyAsync(g->row_ptr, src->row_ptr, (3 * (size_t)src->n + 2) * 4,
+                        cudaMemcpyDeviceToDevice, s);  // row_ptr, rank, off
   int32_t* col_tmp = (int32_t*)scratch;
   uint64_t* d_seed = (uint64_t*)(scratch + ((m1 * 4 + 15) & ~(size_t)15));
   uint32_t* gscr = gwords ? (uint32_t*)((char*)d_seed + 16) : nullptr;
@@ -604,14 +601,14 @@ mt_status mt_randomize(const mt_graph* src, uint64_t seed, uint64_t swaps, void*
     e = launch_randomize(src->n, src->m, 1, src->row_ptr, src->col, d_seed, swaps, col_tmp, gscr, s);
   if (e != cudaSuccess) {
     set_last_error(cudaGetErrorString(e));
-    if (scratch) cudaFreeAsync(scratch, s);
-    mt_graph_free(g);
+    pool_free(scratch, s);
+    graph_release(g, s);
     return MT_ECUDA;
   }
-  mt_status st = graph_build_sync(g, col_tmp, s);
-  cudaFreeAsync(scratch, s);
+  mt_status st = graph_build_sync(g, col_tmp, true, s);
+  pool_free(scratch, s);
   if (st != MT_OK) {
-    mt_graph_free(g);
+    graph_release(g, s);
     return st;
   }
   *out = g;
@@ -624,33 +621,33 @@ mt_status mt_randomize_dyads(const mt_graph* src, uint64_t seed, uint64_t attemp
   TraceRange tr("mt_randomize_dyads");
   cudaStream_t s = (cudaStream_t)stream;
   mt_graph* g = nullptr;
-  MT_TRY(graph_alloc(src->n, src->m, &g));
+  MT_TRY(graph_alloc(src->n, src->m, s, &g));
   const size_t m1 = (size_t)(src->m > 0 ? src->m : 1);
   const size_t sc = dyad_scratch_ints(src->n, src->m);
   const size_t gwords = rand_gscratch_words(src->m, 1);
   char* scratch = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&scratch, (m1 + sc) * 4 + 64 + gwords * 4 + 16, s);
+  cudaError_t e = pool_alloc((void**)&scratch, (m1 + sc) * 4 + 64 + gwords * 4 + 16, s);
   int32_t* col_tmp = (int32_t*)scratch;
   int32_t* dsc = col_tmp + m1;
   uint64_t* d_seed = (uint64_t*)(((uintptr_t)(dsc + sc) + 15) & ~(uintptr_t)15);
   uint32_t* gscr = gwords ? (uint32_t*)((char*)d_seed + 16) : nullptr;
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(g->row_ptr, src->row_ptr, (size_t)(src->n + 1) * 4,
-                        cudaMemcpyDeviceToDevice, s);
+    e = cudaMemcpyAsync(g->row_ptr, src->row_ptr, (3 * (size_t)src->n + 2) * 4,
+                        cudaMemcpyDeviceToDevice, s);  // row_ptr, rank, off
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_seed, &seed, 8, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
     e = launch_randomize_dyads(src->n, src->m, 1, src->row_ptr, src->col, d_seed, attempts,
                                col_tmp, dsc, gscr, s);
   if (e != cudaSuccess) {
     set_last_error(cudaGetErrorString(e));
-    if (scratch) cudaFreeAsync(scratch, s);
-    mt_graph_free(g);
+    pool_free(scratch, s);
+    graph_release(g, s);
     return MT_ECUDA;
   }
-  mt_status st = graph_build_sync(g, col_tmp, s);
-  cudaFreeAsync(scratch, s);
+  mt_status st = graph_build_sync(g, col_tmp, true, s);
+  pool_free(scratch, s);
   if (st != MT_OK) {
-    mt_graph_free(g);
+    graph_release(g, s);
     return st;
   }
   *out = g;

@@ -76,7 +76,7 @@ struct mt_server {
   int max_slots = 0;
   double round_cost = 0;
   cudaStream_t stream = nullptr, load_stream = nullptr;
-  cudaEvent_t load_ev = nullptr;
+  mt::BuildStats* h_stats = nullptr;  // pinned: what the loads of an admission found
   cudaStream_t kstream[4] = {nullptr, nullptr, nullptr, nullptr};  // a round's launch per k
   cudaEvent_t fork_ev = nullptr, kdone_ev[4] = {nullptr, nullptr, nullptr, nullptr};
   std::deque<mt::SrvRequest*> pending;
@@ -110,7 +110,8 @@ static double choose_d(double x, int r) {
 }
 
 // Per-root cost estimate from degrees: every arc (a,b) adds C(d_a + d_b, k-2)
-// to its smaller end, the root that owns the sets grown through it.
+// (from a table of the sums) to its smaller end, the root that owns the sets
+// grown through it.
 static void root_costs(SrvRequest* r) {
   const int n = r->n;
   std::vector<int32_t> deg(n, 0);
@@ -119,12 +120,14 @@ static void root_costs(SrvRequest* r) {
   r->dmax_b = 1;
   for (int v = 0; v < n; ++v) r->dmax_b = std::max(r->dmax_b, deg[v]);
   r->nu_b = std::max(2 * r->m, 1);
+  std::vector<double> of_sum(2 * (size_t)r->dmax_b + 1);
+  for (size_t d = 0; d < of_sum.size(); ++d) of_sum[d] = 1.0 + choose_d((double)d, r->k - 2);
   std::vector<double> cost(n, 1.0);
   for (int v = 0; v < n; ++v)
     for (int32_t e = r->rp[v]; e < r->rp[v + 1]; ++e) {
       const int u = r->col[e];
       const int lo = std::min(v, u), hi = std::max(v, u);
-      cost[lo] += 1.0 + choose_d((double)deg[lo] + deg[hi], r->k - 2);
+      cost[lo] += of_sum[deg[lo] + deg[hi]];
     }
   r->cum.assign(n + 1, 0.0);
   for (int v = 0; v < n; ++v) r->cum[v + 1] = r->cum[v] + cost[v];
@@ -190,7 +193,7 @@ static mt_status acquire_pinned(mt_server* s, int k, uint32_t C, uint64_t** out)
 static void release_request(mt_server* s, SrvRequest* r) {
   if (r->g) graph_release(r->g, s->stream);
   r->g = nullptr;
-  if (r->d_hist) cudaFreeAsync(r->d_hist, s->stream);
+  pool_free(r->d_hist, s->stream);
   r->d_hist = nullptr;
   if (r->state == 1 || r->state == 2) s->used -= std::min(s->used, r->bytes);
 }
@@ -209,8 +212,23 @@ static void fail_request(mt_server* s, RoundBuf& R, SrvRequest* r, mt_status st)
   if (f != R.finishing.end()) R.finishing.erase(f);
 }
 
+// A request whose load failed.
+static void drop_load(mt_server* s, SrvRequest* r, mt_status st) {
+  graph_release(r->g, s->load_stream);
+  r->g = nullptr;
+  pool_free(r->d_hist, s->load_stream);
+  r->d_hist = nullptr;
+  if (r->h_result) s->pinned_free[r->k - 3].push_back(r->h_result);
+  r->h_result = nullptr;
+  r->state = 3;
+  r->status = st;
+  r->t_done = now_ms(s);
+}
+
+// The loads of a round's admissions are enqueued one after another and waited
+// for once.
 static void admit(mt_server* s) {
-  bool loaded = false;
+  std::vector<SrvRequest*> loading;
   while (!s->pending.empty() && (int)s->active.size() < s->max_slots) {
     SrvRequest* r = s->pending.front();
     const uint32_t C = table_classes(s->tables[r->k - 3]);
@@ -234,10 +252,11 @@ static void admit(mt_server* s) {
     }
     if (s->used + r->bytes + reserved_total(s) - s->reserved[ki] + need_k > s->budget) break;
     s->pending.pop_front();
-    mt_status st = graph_load_on(r->n, r->m, r->rp.data(), r->col.data(), s->load_stream, &r->g);
+    mt_status st = graph_load_begin(r->n, r->m, r->rp.data(), r->col.data(), s->load_stream,
+                                    s->h_stats + loading.size(), &r->g);
     if (st == MT_OK) st = acquire_pinned(s, r->k, C, &r->h_result);
     if (st == MT_OK) {
-      cudaError_t e = cudaMallocAsync((void**)&r->d_hist, (size_t)C * 8, s->load_stream);
+      cudaError_t e = pool_alloc((void**)&r->d_hist, (size_t)C * 8, s->load_stream);
       if (e == cudaSuccess) e = cudaMemsetAsync(r->d_hist, 0, (size_t)C * 8, s->load_stream);
       if (e != cudaSuccess) {
         set_last_error(cudaGetErrorString(e));
@@ -245,28 +264,29 @@ static void admit(mt_server* s) {
       }
     }
     if (st != MT_OK) {
-      if (r->g) graph_release(r->g, s->load_stream);
-      r->g = nullptr;
-      if (r->h_result) s->pinned_free[r->k - 3].push_back(r->h_result);
-      r->h_result = nullptr;
-      r->state = 3;
-      r->status = st;
-      r->t_done = now_ms(s);
+      drop_load(s, r, st);
       continue;
     }
-    std::vector<int32_t>().swap(r->rp);
-    std::vector<int32_t>().swap(r->col);
     s->used += r->bytes;
     s->reserved[ki] = need_k;
     r->state = 1;
     r->t_admit = now_ms(s);
     r->next_root = 0;
     s->active.push_back(r);
-    loaded = true;
+    loading.push_back(r);
   }
-  if (loaded) {
-    cudaEventRecord(s->load_ev, s->load_stream);
-    cudaStreamWaitEvent(s->stream, s->load_ev, 0);
+  if (loading.empty()) return;
+  const cudaError_t e = cudaStreamSynchronize(s->load_stream);
+  for (size_t i = 0; i < loading.size(); ++i) {
+    SrvRequest* r = loading[i];
+    std::vector<int32_t>().swap(r->rp);
+    std::vector<int32_t>().swap(r->col);
+    const mt_status st = e != cudaSuccess ? MT_ECUDA : graph_take_stats(r->g, s->h_stats[i]);
+    if (st != MT_OK) {
+      s->active.erase(std::find(s->active.begin(), s->active.end(), r));
+      s->used -= std::min(s->used, r->bytes);
+      drop_load(s, r, st);
+    }
   }
 }
 
@@ -275,16 +295,16 @@ static void admit(mt_server* s) {
 // budget.
 static mt_status ensure_capacity(mt_server* s, int ki, size_t ws_need, size_t graphs) {
   if (s->ws_bytes[ki] < ws_need) {
-    if (s->ws[ki]) MT_CUDA_TRY(cudaFreeAsync(s->ws[ki], s->stream));
+    pool_free(s->ws[ki], s->stream);
     s->ws[ki] = nullptr;
     s->ws_bytes[ki] = 0;
-    MT_CUDA_TRY(cudaMallocAsync(&s->ws[ki], ws_need, s->stream));
+    MT_CUDA_TRY(pool_alloc(&s->ws[ki], ws_need, s->stream));
     s->ws_bytes[ki] = ws_need;
   }
   if (s->d_graphs_cap[ki] < graphs) {
-    if (s->d_graphs[ki]) MT_CUDA_TRY(cudaFreeAsync(s->d_graphs[ki], s->stream));
+    pool_free(s->d_graphs[ki], s->stream);
     const size_t cap = graphs;
-    MT_CUDA_TRY(cudaMallocAsync((void**)&s->d_graphs[ki], cap * sizeof(DevGraph), s->stream));
+    MT_CUDA_TRY(pool_alloc((void**)&s->d_graphs[ki], cap * sizeof(DevGraph), s->stream));
     s->d_graphs_cap[ki] = cap;
   }
   return MT_OK;
@@ -297,8 +317,8 @@ static void release_idle_scratch(mt_server* s) {
     bool any = false;
     for (const SrvRequest* r : s->active) any |= r->k == ki + 3;
     if (any) continue;
-    if (s->ws[ki]) cudaFreeAsync(s->ws[ki], s->stream);
-    if (s->d_graphs[ki]) cudaFreeAsync(s->d_graphs[ki], s->stream);
+    pool_free(s->ws[ki], s->stream);
+    pool_free(s->d_graphs[ki], s->stream);
     s->ws[ki] = nullptr;
     s->ws_bytes[ki] = 0;
     s->d_graphs[ki] = nullptr;
@@ -490,7 +510,8 @@ mt_status mt_server_create(const mt_table* t3, const mt_table* t4, const mt_tabl
   s->t0 = std::chrono::steady_clock::now();
   cudaError_t e = cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->load_stream, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->load_ev, cudaEventDisableTiming);
+  if (e == cudaSuccess)
+    e = cudaMallocHost((void**)&s->h_stats, (size_t)max_slots * sizeof(BuildStats));
   for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
     e = cudaEventCreateWithFlags(&s->rb[i].ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&s->rb[i].h_err, 4 * sizeof(uint32_t));
@@ -585,13 +606,13 @@ mt_status mt_server_free(mt_server* s) {
   for (auto& kv : s->all) {
     SrvRequest* r = kv.second;
     if (r->g) graph_release(r->g, s->stream);
-    if (r->d_hist) cudaFreeAsync(r->d_hist, s->stream);
+    pool_free(r->d_hist, s->stream);
     if (r->h_result) cudaFreeHost(r->h_result);
     delete r;
   }
   for (int i = 0; i < 4; ++i) {
-    if (s->ws[i]) cudaFreeAsync(s->ws[i], s->stream);
-    if (s->d_graphs[i]) cudaFreeAsync(s->d_graphs[i], s->stream);
+    pool_free(s->ws[i], s->stream);
+    pool_free(s->d_graphs[i], s->stream);
     for (uint64_t* p : s->pinned_free[i]) cudaFreeHost(p);
   }
   if (s->stream) cudaStreamSynchronize(s->stream);
@@ -600,7 +621,7 @@ mt_status mt_server_free(mt_server* s) {
     if (b.h_graphs) cudaFreeHost(b.h_graphs);
     if (b.h_err) cudaFreeHost(b.h_err);
   }
-  if (s->load_ev) cudaEventDestroy(s->load_ev);
+  if (s->h_stats) cudaFreeHost(s->h_stats);
   if (s->fork_ev) cudaEventDestroy(s->fork_ev);
   for (int i = 0; i < 4; ++i) {
     if (s->kstream[i]) {

@@ -23,7 +23,7 @@
 #include <numeric>
 #include <vector>
 
-#include "common.cuh"
+#include "graph.cuh"
 #include "trace.cuh"
 
 struct mt_table {
@@ -424,7 +424,7 @@ static cudaError_t scratch_alloc(TableScratch* x, int k, cudaStream_t s) {
   const size_t o_m = take(k == 6 ? (size_t)kP5Classes * 4 : 0);
   const size_t o_g = take(k == 6 ? (size_t)kP5Keys * 2 : 0);
   const size_t o_r = take(k == 6 ? 256 * 4 : 0);
-  cudaError_t e = cudaMallocAsync((void**)&x->mem, off, s);
+  cudaError_t e = pool_alloc((void**)&x->mem, off, s);
   if (e != cudaSuccess) return e;
   x->bitmap = (uint32_t*)(x->mem + o_b);
   x->bitmap5 = (uint32_t*)(x->mem + o_b5);
@@ -482,6 +482,12 @@ static void table_drop(mt_table* t) {
   delete t;
 }
 
+static mt_status table_done(mt_table* t, mt_table** out) {
+  handle_born();
+  *out = t;
+  return MT_OK;
+}
+
 static mt_status build_table(int k, cudaStream_t s, mt_table** out) {
   const uint64_t nkeys = 1ull << (k * (k - 1));
   int nsteps = 0, nsteps5 = 0;
@@ -520,7 +526,7 @@ static mt_status build_table(int k, cudaStream_t s, mt_table** out) {
   uint32_t got[5] = {0}, got5[5] = {0};
   if (e == cudaSuccess) e = read_total(x.bitmap, x.prefix, x.ngroups, got, s);
   if (e == cudaSuccess && k == 6) e = read_total(x.bitmap5, x.prefix5, x.ngroups5, got5, s);
-  if (x.mem) cudaFreeAsync(x.mem, s);
+  pool_free(x.mem, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
     set_last_error(cudaGetErrorString(e));
@@ -532,8 +538,7 @@ static mt_status build_table(int k, cudaStream_t s, mt_table** out) {
     table_drop(t);
     return MT_ECUDA;
   }
-  *out = t;
-  return MT_OK;
+  return table_done(t, out);
 }
 
 // ---------------------------------------------------------- compact k = 6 form
@@ -669,7 +674,7 @@ static mt_status build_compact6(cudaStream_t s, mt_table** out) {
   if (xsigma) cudaFreeAsync(xsigma, s);
   if (xbits) cudaFreeAsync(xbits, s);
   if (xrep) cudaFreeAsync(xrep, s);
-  if (x.mem) cudaFreeAsync(x.mem, s);
+  pool_free(x.mem, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   for (uint32_t w : hb) nreps += __builtin_popcount(w);
   if (e != cudaSuccess) {
@@ -683,8 +688,7 @@ static mt_status build_compact6(cudaStream_t s, mt_table** out) {
     table_drop(t);
     return MT_ECUDA;
   }
-  *out = t;
-  return MT_OK;
+  return table_done(t, out);
 }
 
 TableView table_view(const mt_table* t) {
@@ -729,11 +733,8 @@ mt_status mt_table_is_compact(const mt_table* t, int* compact) {
 mt_status mt_table_free(mt_table* t) {
   if (!t) return MT_OK;
   cudaDeviceSynchronize();
-  cudaFree(t->table);
-  cudaFree(t->class_masks);
-  if (t->xclass) cudaFree(t->xclass);
-  if (t->xmap) cudaFree(t->xmap);
-  delete t;
+  table_drop(t);
+  handle_died();
   return MT_OK;
 }
 

@@ -78,11 +78,12 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr int kTargetItemsPerWarp = 64;
 // Cell method: an item's least estimated work, below which fetching it and
 // marking its root's neighbours costs more than the warps it feeds give.  One
-// graph on a GB300: k = 4 (n = 2,000 / 3,646 / 6,437) 119 / 163 / 180 us at 128
-// against 147 / 199 / 203 at 512 and 195 / 432 / 627 near 10; k = 5 (n = 1,500)
-// 884 at 512, 1,044 near 50; k = 3 (n = 20,000) 149 at 1,024, 176 at 256.
+// graph on a GB300: k = 4 (n = 2,000) 97 us at 128 against 113 at 32 and 140 at
+// 512; k = 5 (n = 112 / 310 / 343) 127 / 177 / 115 us at 128, 151 / 225 / 138 at
+// 512, 114 / 173 / 115 near 10, n = 1,500 indifferent; k = 3 (n = 20,000) 131 us at
+// 1,024, 151 at 512.
 template <int K>
-constexpr double kCellsItemFloor = K == 3 ? 1024.0 : K == 4 ? 128.0 : 512.0;
+constexpr double kCellsItemFloor = K == 3 ? 1024.0 : 128.0;
 // Adds one warp may make to a shared 32-bit histogram between two flushes of
 // it by exchange (enumeration path, k <= 5; see `ladd` in k_count).
 constexpr int kLeafBudget = 1 << 25;

@@ -122,12 +122,17 @@ static void root_costs(SrvRequest* r) {
   r->nu_b = std::max(2 * r->m, 1);
   std::vector<double> of_sum(2 * (size_t)r->dmax_b + 1);
   for (size_t d = 0; d < of_sum.size(); ++d) of_sum[d] = 1.0 + choose_d((double)d, r->k - 2);
+  // the numbering of the roots: by descending degree, as the device build's (the
+  // order of equal degrees differs, which the estimates can bear)
+  std::vector<int32_t> start(r->dmax_b + 2, 0), num(n);
+  for (int v = 0; v < n; ++v) ++start[r->dmax_b - deg[v] + 1];
+  for (int d = 0; d <= r->dmax_b; ++d) start[d + 1] += start[d];
+  for (int v = 0; v < n; ++v) num[v] = start[r->dmax_b - deg[v]]++;
   std::vector<double> cost(n, 1.0);
   for (int v = 0; v < n; ++v)
     for (int32_t e = r->rp[v]; e < r->rp[v + 1]; ++e) {
       const int u = r->col[e];
-      const int lo = std::min(v, u), hi = std::max(v, u);
-      cost[lo] += of_sum[deg[lo] + deg[hi]];
+      cost[std::min(num[v], num[u])] += of_sum[deg[v] + deg[u]];
     }
   r->cum.assign(n + 1, 0.0);
   for (int v = 0; v < n; ++v) r->cum[v + 1] = r->cum[v] + cost[v];

@@ -41,7 +41,7 @@ struct mt_table {
 
 namespace mt {
 
-__constant__ uint8_t c_sjt[7][720];  // per k: transposition positions p (swap p, p+1)
+__constant__ uint8_t c_sjt[6][120];  // per k <= 5: transposition positions p (swap p, p+1)
 
 // Positions of the adjacent transpositions that take the identity through all
 // k! permutations (Steinhaus-Johnson-Trotter with directions).
@@ -253,7 +253,9 @@ static cudaError_t launch_rank(const uint32_t* bitmap, size_t ngroups, int32_t* 
 // prefix per 5-vertex digraph, connected or not) go through the k! orderings;
 // every other row of 1,024 slots is one of theirs with its slots permuted.
 // Measured on a GB300, table, count and read-out of one 800-vertex graph: 910
-// ms with all 2^30 keys walked (893 ms of it k_canon<6>), 18.4 ms this way.
+// ms with all 2^30 keys walked (893 ms of it k_canon<6>), 8.0 ms this way: 3.1
+// of it allocating and freeing 4 GiB, 1.1 writing the table (3.8 TB/s), 1.25 the
+// canonical masks, 1.1 the count.
 
 constexpr int kP5Keys = 1 << 20;      // 5-vertex prefix keys
 constexpr uint32_t kP5Classes = 9608; // 5-vertex digraphs up to isomorphism
@@ -297,11 +299,42 @@ __device__ __forceinline__ uint32_t mask5_to_key(uint32_t mask) {
   return key;
 }
 
+// Orderings that can reach a 6-vertex digraph's least mask.  The last vertex's
+// row is the mask's highest, so the last vertex has the least out-degree d and
+// its d successors come first: d! (5 - d)! orderings for each such vertex, 12 to
+// 120 instead of 720.  Per d, the adjacent transpositions that walk S_d on
+// positions 0..d-1 times S_(5-d) on positions d..4.
+struct LastWalks {
+  int32_t first[7];   // of d's transpositions in `at`; first[6] is the end
+  uint8_t at[320];
+};
+__constant__ LastWalks c_last;
+
+static LastWalks last_walks() {
+  LastWalks w{};
+  int n = 0;
+  for (int d = 0; d <= 5; ++d) {
+    w.first[d] = n;
+    const std::vector<uint8_t> left = sjt_sequence(d), right = sjt_sequence(5 - d);
+    for (size_t i = 0; i <= left.size(); ++i) {
+      for (uint8_t p : right) w.at[n++] = (uint8_t)(d + p);
+      if (i < left.size()) w.at[n++] = left[i];
+    }
+  }
+  w.first[6] = n;
+  return w;
+}
+
 // Canonical masks of the 6-vertex keys above the class prefixes (sub[class][z]);
 // marks the connected ones.  Disconnected patterns get mask 0, which is not
-// connected and so is never marked.
+// connected and so is never marked.  Bound by its integer operations: walking
+// all 720 orderings took 7.5 ms, these take 1.25 ms.
 __global__ void __launch_bounds__(256) k_sub_canon(uint32_t* sub, const uint32_t* masks5,
-                                                   uint32_t* bitmap, int nsteps) {
+                                                   uint32_t* bitmap) {
+  __shared__ LastWalks walks;
+  for (int i = threadIdx.x; i < (int)sizeof(LastWalks) / 4; i += blockDim.x)
+    ((uint32_t*)&walks)[i] = ((const uint32_t*)&c_last)[i];
+  __syncthreads();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (kP5Classes << kP5Low)) return;
   const uint32_t key =
@@ -309,10 +342,31 @@ __global__ void __launch_bounds__(256) k_sub_canon(uint32_t* sub, const uint32_t
   const uint64_t x0 = key_to_matrix(key, 6);
   uint32_t c = 0;
   if (matrix_connected(x0, 6)) {
-    uint64_t x = x0, best = x0;
-    for (int s = 0; s < nsteps; ++s) {
-      x = swap_adjacent(x, c_sjt[6][s]);
+    int d = 6;
+    for (int v = 0; v < 6; ++v) d = min(d, __popc((uint32_t)(x0 >> (8 * v)) & 0xFFu));
+    uint64_t best = ~0ull;
+    for (int v = 0; v < 6; ++v) {
+      const uint32_t succ = (uint32_t)(x0 >> (8 * v)) & 0xFFu;
+      if (__popc(succ) != d) continue;
+      // successors of v, the others, v: old vertex of each position, 4 bits each
+      uint32_t at = (uint32_t)v << 20;
+      int lo = 0, hi = d;
+      for (int u = 0; u < 6; ++u)
+        if (u != v) at |= (uint32_t)u << (4 * ((succ >> u) & 1u ? lo++ : hi++));
+      uint64_t x = 0;
+#pragma unroll
+      for (int p = 0; p < 6; ++p) {
+        const uint32_t row = (uint32_t)(x0 >> (8 * ((at >> (4 * p)) & 15u))) & 0xFFu;
+        uint32_t r = 0;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) r |= ((row >> ((at >> (4 * q)) & 15u)) & 1u) << q;
+        x |= (uint64_t)r << (8 * p);
+      }
       best = x < best ? x : best;
+      for (int s = walks.first[d]; s < walks.first[d + 1]; ++s) {
+        x = swap_adjacent(x, walks.at[s]);
+        best = x < best ? x : best;
+      }
     }
     c = matrix_to_mask(best, 6);
     const uint32_t bit = 1u << (c & 31u);
@@ -381,7 +435,7 @@ static mt_status upload_sjt(int k, cudaStream_t s, int* nsteps) {
   for (int i = 2; i <= k; ++i) fact *= i;
   if (seq.size() + 1 != fact || std::unique(seen.begin(), seen.end()) != seen.end())
     return MT_ECUDA;
-  MT_CUDA_TRY(cudaMemcpyToSymbolAsync(c_sjt, seq.data(), seq.size(), (size_t)k * 720,
+  MT_CUDA_TRY(cudaMemcpyToSymbolAsync(c_sjt, seq.data(), seq.size(), (size_t)k * 120,
                                       cudaMemcpyHostToDevice, s));
   *nsteps = (int)seq.size();
   return MT_OK;
@@ -441,17 +495,21 @@ static cudaError_t scratch_alloc(TableScratch* x, int k, cudaStream_t s) {
 
 // The 5-vertex classes and the dense ids above them (x->sub, x->class5,
 // x->sigma), and the class list.
-static cudaError_t launch_sub6(const TableScratch& x, uint32_t* class_masks, int nsteps5,
-                               int nsteps6, int sms, cudaStream_t s) {
+static cudaError_t launch_sub6(const TableScratch& x, uint32_t* class_masks, int nsteps5, int sms,
+                               cudaStream_t s) {
+  const LastWalks walks = last_walks();
+  cudaError_t e = cudaMemcpyToSymbolAsync(c_last, &walks, sizeof(walks), 0, cudaMemcpyHostToDevice,
+                                          s);
+  if (e != cudaSuccess) return e;
   k_prefix5<<<kP5Keys / 256, 256, 0, s>>>(x.class5, x.sigma, x.bitmap5, nsteps5);
-  cudaError_t e = launch_rank(x.bitmap5, x.ngroups5, x.tiles, x.prefix5, s);
+  e = launch_rank(x.bitmap5, x.ngroups5, x.tiles, x.prefix5, s);
   if (e != cudaSuccess) return e;
   const uint4* b5 = (const uint4*)x.bitmap5;
   const uint4* b6 = (const uint4*)x.bitmap;
   k_bit_list<<<32, 256, 0, s>>>(b5, x.ngroups5, x.prefix5, x.masks5, kP5Classes);
   k_assign<<<sms * 8, 256, 0, s>>>(x.class5, kP5Keys, b5, x.prefix5);
   const uint32_t nsub = kP5Classes << kP5Low;
-  k_sub_canon<<<(nsub + 255) / 256, 256, 0, s>>>(x.sub, x.masks5, x.bitmap, nsteps6);
+  k_sub_canon<<<(nsub + 255) / 256, 256, 0, s>>>(x.sub, x.masks5, x.bitmap);
   e = launch_rank(x.bitmap, x.ngroups, x.tiles, x.prefix, s);
   if (e != cudaSuccess) return e;
   k_assign<<<sms * 16, 256, 0, s>>>(x.sub, nsub, b6, x.prefix);
@@ -490,9 +548,8 @@ static mt_status table_done(mt_table* t, mt_table** out) {
 
 static mt_status build_table(int k, cudaStream_t s, mt_table** out) {
   const uint64_t nkeys = 1ull << (k * (k - 1));
-  int nsteps = 0, nsteps5 = 0;
-  MT_TRY(upload_sjt(k, s, &nsteps));
-  if (k == 6) MT_TRY(upload_sjt(5, s, &nsteps5));
+  int nsteps = 0;  // k = 6 walks the orderings of its 5-vertex prefixes
+  MT_TRY(upload_sjt(std::min(k, 5), s, &nsteps));
   mt_table* t = new mt_table();
   t->k = k;
   t->nkeys = nkeys;
@@ -505,7 +562,7 @@ static mt_status build_table(int k, cudaStream_t s, mt_table** out) {
     const int sms = sm_count();
     const int grid = (int)std::min<uint64_t>((nkeys + 255) / 256, (uint64_t)sms * 16);
     if (k == 6) {
-      e = launch_sub6(x, t->class_masks, nsteps5, nsteps, sms, s);
+      e = launch_sub6(x, t->class_masks, nsteps, sms, s);
       if (e == cudaSuccess)
         k_expand<<<sms * 8, 256, 0, s>>>(t->table, x.sub, x.class5, x.sigma, nullptr, kP5Keys);
     } else {
@@ -627,8 +684,7 @@ __global__ void k_xreps(const uint32_t* xbits, const int32_t* xrep, int32_t* rep
 }
 
 static mt_status build_compact6(cudaStream_t s, mt_table** out) {
-  int nsteps = 0, nsteps5 = 0;
-  MT_TRY(upload_sjt(6, s, &nsteps));
+  int nsteps5 = 0;
   MT_TRY(upload_sjt(5, s, &nsteps5));
   mt_table* t = new mt_table();
   t->k = 6;
@@ -654,7 +710,7 @@ static mt_status build_compact6(cudaStream_t s, mt_table** out) {
   int32_t nreps = 0;
   if (e == cudaSuccess) {
     const int sms = sm_count();
-    e = launch_sub6(x, t->class_masks, nsteps5, nsteps, sms, s);
+    e = launch_sub6(x, t->class_masks, nsteps5, sms, s);
     k_xprefix<<<kXKeys / 256, 256, 0, s>>>(xcanon, xsigma, xbits, xrep);
     k_xtables<<<kXKeys, 256, 0, s>>>(xcanon, xsigma, xbits, t->xclass, t->xmap);
     k_xreps<<<1, 32, 0, s>>>(xbits, xrep, x.reps);

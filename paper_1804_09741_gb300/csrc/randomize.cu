@@ -11,9 +11,10 @@
 // GPU mapping: one thread block per graph.  The arc array (src<<16 | dst) and a
 // hash set of the present arcs sit in shared memory (global memory for graphs
 // too large for it); the block fills them in parallel.  Then 256 threads run
-// the attempts in windows of 64, four threads per attempt (one per arc that it
-// looks up or replaces), while two warps draw the next attempts' positions,
-// which do not depend on the graph:
+// the attempts in windows of 64 (128 threads, 32 for small graphs), four threads
+// per attempt (one per arc that it looks up or replaces; a warp has new arcs or
+// old ones), while two warps draw the next attempts' positions, which do not
+// depend on the graph:
 //  * speculation: every attempt is evaluated against the state at the start of
 //    the window (the two arcs at its positions, the checks, whether the two new
 //    arcs are present);
@@ -29,9 +30,10 @@
 // The outcome is that of the attempts run one after another.  What bounds it is
 // the latency of one window after another: at m = 6,000 a window passes 44.5
 // attempts (two attempts of a window overlap with probability about 4 / m; 128
-// wide it would pass 50) and takes 1.5 us.  One graph of m = 6,000, 60,000
+// wide it would pass 50) and takes 1.4 us.  One graph of m = 6,000, 60,000
 // attempts: 7.2 ms with one warp, 32 attempts and bucket scans by every lane,
-// 2.3 ms now; 511 graphs of m = 1,500: 6.0 -> 1.5 ms.
+// 2.1 ms now; 511 graphs of m = 1,500: 6.0 ms, 1.5 in windows of 64, 1.1 in windows
+// of 32.
 //
 // Set: 2^bb buckets of 8 slots (two 16-byte reads), 2 to 4 keys per bucket on
 // average; a key lives in the first bucket of its probe sequence (home bucket,
@@ -167,9 +169,14 @@ struct BucketSet {
 };
 
 // Shared-memory working set of the windows.
-constexpr int kWindow = 64;      // attempts per window, four threads each
-constexpr int kRunners = 4 * kWindow;
-constexpr int kRandThreads = kRunners + 64;  // two warps draw
+constexpr int kWindow = 64;      // attempts per window at most, four threads each
+template <int WN>
+constexpr int kRunners = 4 * WN;
+template <int WN>
+constexpr int kRandThreads = kRunners<WN> + 64;  // two warps draw
+// Graphs of fewer arcs run windows of 32: little of a wider one passes (20 of 32
+// attempts at m = 1,500, 24 of 64), and it takes half the warps.
+constexpr int kWideArcs = 3000;
 constexpr int kDraws = 256;      // attempts per buffer of drawn positions
 constexpr int kKeyTab = 512, kPosTab = 512;
 struct RandWindow {
@@ -178,33 +185,46 @@ struct RandWindow {
   uint2 ktab[kKeyTab];           // bits of the accepted attempts by arc (hashed)
   uint2 ptab[kPosTab];           //   and by position
   uint2 draws[2][kDraws];
-  int first_bad[2];              // first unsafe attempt; windows alternate
+  uint32_t accepted[2][4];       // accepted attempts, a bit per even lane of the new keys'
+                                 // warps; windows alternate
+  int first_bad[2];              // first unsafe attempt
 };
 
 __device__ __forceinline__ uint32_t key_slot(uint32_t key) {
   return (key * 0x85EBCA6Bu) >> 23;  // 32 - log2(kKeyTab)
 }
 
-// Barrier of the threads that run the attempts.
-__device__ __forceinline__ void run_sync() {
-  asm volatile("bar.sync 1, %0;" ::"n"(kRunners) : "memory");
+// The even bits of x, together.
+__device__ __forceinline__ uint32_t squeeze(uint32_t x) {
+  x &= 0x55555555u;
+  x = (x | x >> 1) & 0x33333333u;
+  x = (x | x >> 2) & 0x0F0F0F0Fu;
+  x = (x | x >> 4) & 0x00FF00FFu;
+  return (x | x >> 8) & 0xFFFFu;
 }
 
-// Threads 0 .. kRunners-1: the attempts whose positions are draws[0..n), in
-// order, thread 4j + q holding key q of the window's attempt j (0, 1: the new
-// keys, to be absent; 2, 3: the old ones).  `Pol::make` derives from the two
-// entries an attempt's validity, its keys and the two new entries.
-template <class Pol, bool GM>
+// Barrier of the threads that run the attempts.
+template <int WN>
+__device__ __forceinline__ void run_sync() {
+  asm volatile("bar.sync 1, %0;" ::"n"(kRunners<WN>) : "memory");
+}
+
+// Threads 0 .. kRunners<WN> - 1: the attempts whose positions are draws[0..n), in
+// order.  Thread 2j + q of the first half holds new key q of the window's attempt
+// j (to be absent), of the second half old key q (a warp does one of the two).
+// `Pol::make` derives from the two entries an attempt's validity, its keys and
+// the two new entries.
+template <class Pol, bool GM, int WN>
 __device__ __forceinline__ void run_draws(const Pol& pol, uint32_t* ent, const BucketSet<GM>& S,
                                           RandWindow& W, const uint2* draws, int n) {
-  const int j = threadIdx.x >> 2, q = threadIdx.x & 3, quad = threadIdx.x & 28;
-  const bool fresh = q < 2;
+  const bool fresh = threadIdx.x < 2 * WN;
+  const int j = (threadIdx.x >> 1) & (WN - 1), q = threadIdx.x & 1;
   const int half = j >> 5;
   const unsigned bit = 1u << (j & 31);
   for (int t = 0, w = 0; t < n; w ^= 1) {
-    const int cnt = min(kWindow, n - t);
+    const int cnt = min(WN, n - t);
     // speculation; `valid`: the outcome depends on the graph, `tried`: its keys
-    // are looked up, `acc`: accepted
+    // are looked up
     uint2 e = make_uint2(0, 0);
     if (j < cnt) e = draws[t + j];
     const bool valid = e.x != e.y;
@@ -213,34 +233,49 @@ __device__ __forceinline__ void run_draws(const Pol& pol, uint32_t* ent, const B
     if (valid)
       tried = pol.make(state_read<GM>(ent + e.x), state_read<GM>(ent + e.y), k1, k2, o1, o2, w1,
                        w2);
-    const uint32_t key = fresh ? (q == 0 ? k1 : k2) : (q == 2 ? o1 : o2);
-    const uint32_t pos = q == 2 ? e.x : e.y;
-    // A new key: is it there, and a free slot of its home bucket.  An old one:
-    // its slot (only this attempt may erase it, so the slot stays valid).
+    const uint32_t key = fresh ? (q ? k2 : k1) : (q ? o2 : o1);
+    const uint32_t pos = q ? e.y : e.x;
+    const uint32_t ks = key_slot(key), ps = pos & (kPosTab - 1);
     const uint32_t h = S.home(key);
     const BucketRow r = S.row(h);
-    // (New keys of one window prefer different slots of a bucket.)
-    const unsigned slots = r.mask(fresh ? kEmpty : key);
-    const unsigned turned = fresh ? (slots | slots << 8) >> (j & 7) : slots;
-    const int at = slots ? (__ffs(turned) - 1 + (fresh ? j : 0)) & 7 : -1;
-    bool there = r.has(key);
-    if (tried && fresh && !there && S.passed(h)) there = S.contains_after(key, h);
-    const unsigned hit = __ballot_sync(kWarp, fresh && there) >> quad;
-    const bool acc = tried && (hit & 3u) == 0;
-    const uint32_t ks = key_slot(key), ps = pos & (kPosTab - 1);
-    if (acc) {
-      if (q == 0) W.keys[j] = make_uint4(k1, k2, o1, o2);
-      if (q == 1) W.pos[j] = e;
-      atomicOr((uint32_t*)&W.ktab[ks] + half, bit);
-      if (!fresh) atomicOr((uint32_t*)&W.ptab[ps] + half, bit);
+    int at;  // new key: a free slot of its home bucket; old key: its slot (only
+             // this attempt may erase it, so the slot stays valid)
+    if (fresh) {
+      // new keys of one window prefer different slots of a bucket
+      const unsigned slots = r.mask(kEmpty);
+      at = slots ? (__ffs((slots | slots << 8) >> (j & 7)) - 1 + j) & 7 : -1;
+      bool there = r.has(key);
+      if (tried && !there && S.passed(h)) there = S.contains_after(key, h);
+      const unsigned hit = __ballot_sync(kWarp, there);
+      const bool acc = tried && ((hit >> (threadIdx.x & 30)) & 3u) == 0;
+      const unsigned accs = __ballot_sync(kWarp, acc && q == 0);
+      if ((threadIdx.x & 31) == 0) W.accepted[w][threadIdx.x >> 5] = accs;
+      if (acc) {
+        if (q == 0) W.pos[j] = e;
+        else W.keys[j] = make_uint4(k1, k2, o1, o2);
+        atomicOr((uint32_t*)&W.ktab[ks] + half, bit);
+      }
+    } else {
+      // marked whether accepted or not; whoever reads the marks looks at
+      // `accepted`
+      at = r.find(key);
+      if (tried) {
+        atomicOr((uint32_t*)&W.ktab[ks] + half, bit);
+        atomicOr((uint32_t*)&W.ptab[ps] + half, bit);
+      }
     }
-    run_sync();
+    run_sync<WN>();
+    // the accepted attempts: one bit per pair of lanes of the new keys' warps
+    const uint4 av = *(const uint4*)W.accepted[w];
+    const uint32_t alo = squeeze(av.x) | squeeze(av.y) << 16;
+    const uint32_t ahi = squeeze(av.z) | squeeze(av.w) << 16;
+    const bool acc = ((half ? ahi : alo) & bit) != 0;
     // earlier accepted attempts that may overlap: by arc for the new keys, by
     // position for the old ones
     bool unsafe = false;
     if (fresh ? tried : valid) {
       const uint2 c = fresh ? W.ktab[ks] : W.ptab[ps];
-      uint32_t lo = c.x, hi = c.y;
+      uint32_t lo = c.x & alo, hi = c.y & ahi;
       if (half == 0) {
         lo &= bit - 1u;
         hi = 0;
@@ -267,40 +302,43 @@ __device__ __forceinline__ void run_draws(const Pol& pol, uint32_t* ent, const B
     }
     const unsigned bad = __ballot_sync(kWarp, unsafe);
     if (bad && (threadIdx.x & 31) == 0)
-      atomicMin(&W.first_bad[w], (int)(threadIdx.x >> 2) + ((__ffs(bad) - 1) >> 2));
-    run_sync();
+      atomicMin(&W.first_bad[w], j + ((__ffs(bad) - 1) >> 1));
+    run_sync<WN>();
     // attempts before the first unsafe one (the first of a window is never
     // unsafe) are applied, and the marks go.  A free slot that another key took,
     // or a bucket without one, sends a key the slow way.
     const int p = min(W.first_bad[w], cnt);
     if (threadIdx.x == 0) W.first_bad[w ^ 1] = kWindow;
-    if (acc) {
-      W.ktab[ks] = make_uint2(0, 0);
-      if (!fresh) W.ptab[ps] = make_uint2(0, 0);
-      if (j < p) {
-        if (!fresh) {
-          ent[pos] = q == 2 ? w1 : w2;
-          if (at >= 0) S.t[8 * h + at] = kEmpty;
-          else S.erase_after(key, h);
-        } else if (at < 0 || atomicCAS(&S.t[8 * h + at], kEmpty, key) != kEmpty) {
-          S.insert(key);
-        }
+    const bool apply = acc && j < p;
+    if (fresh) {
+      if (acc) W.ktab[ks] = make_uint2(0, 0);
+      if (apply && (at < 0 || atomicCAS(&S.t[8 * h + at], kEmpty, key) != kEmpty)) S.insert(key);
+    } else {
+      if (tried) {
+        W.ktab[ks] = make_uint2(0, 0);
+        W.ptab[ps] = make_uint2(0, 0);
+      }
+      if (apply) {
+        ent[pos] = q ? w2 : w1;
+        if (at >= 0) S.t[8 * h + at] = kEmpty;
+        else S.erase_after(key, h);
       }
     }
-    run_sync();
+    run_sync<WN>();
     t += p;
   }
 }
 
 // The attempts of one graph, by the whole block: kRunners threads run the drawn
 // attempts of one buffer while the others draw the next buffer's positions.
-template <class Pol, bool GM>
+template <int WN, class Pol, bool GM>
 __device__ void run_attempts(const Pol& pol, uint32_t* ent, const BucketSet<GM>& S, RandWindow& W,
                              uint64_t attempts) {
   const int tid = threadIdx.x;
   for (int i = tid; i < kKeyTab; i += blockDim.x) W.ktab[i] = make_uint2(0, 0);
   for (int i = tid; i < kPosTab; i += blockDim.x) W.ptab[i] = make_uint2(0, 0);
   if (tid < 2) W.first_bad[tid] = kWindow;
+  if (tid < 8) W.accepted[tid >> 2][tid & 3] = 0;  // the words of absent warps stay 0
   auto draw = [&](uint64_t t0, int buf, int first, int step) {
     for (int j = first; j < kDraws && t0 + j < attempts; j += step)
       pol.draw(t0 + j, W.draws[buf][j].x, W.draws[buf][j].y);
@@ -309,12 +347,12 @@ __device__ void run_attempts(const Pol& pol, uint32_t* ent, const BucketSet<GM>&
   __syncthreads();
   int buf = 0;
   for (uint64_t t0 = 0; t0 < attempts; t0 += kDraws, buf ^= 1) {
-    if (tid < kRunners) {
+    if (tid < kRunners<WN>) {
       const int n = (int)(attempts - t0 < (uint64_t)kDraws ? attempts - t0 : kDraws);
-      run_draws(pol, ent, S, W, W.draws[buf], n);
+      run_draws<Pol, GM, WN>(pol, ent, S, W, W.draws[buf], n);
       if (tid == 0) W.first_bad[0] = kWindow;
     } else {
-      draw(t0 + kDraws, buf ^ 1, tid - kRunners, blockDim.x - kRunners);
+      draw(t0 + kDraws, buf ^ 1, tid - kRunners<WN>, blockDim.x - kRunners<WN>);
     }
     __syncthreads();
   }
@@ -360,8 +398,8 @@ __device__ __forceinline__ int row_of(const int32_t* row_ptr, int n, int e) {
   return lo;
 }
 
-template <bool GM>
-__global__ void __launch_bounds__(kRandThreads) k_randomize(RandArgs a) {
+template <bool GM, int WN>
+__global__ void __launch_bounds__(kRandThreads<WN>) k_randomize(RandArgs a) {
   extern __shared__ __align__(16) uint32_t rsm[];
   __shared__ RandWindow W;
   const int g = blockIdx.x;
@@ -378,7 +416,7 @@ __global__ void __launch_bounds__(kRandThreads) k_randomize(RandArgs a) {
   __syncthreads();
   if (m > 0) {
     const ArcSwap pol{a.seeds[g], (uint64_t)m};
-    run_attempts(pol, arcs, S, W, a.swaps);
+    run_attempts<WN>(pol, arcs, S, W, a.swaps);
   }
   __syncthreads();
   for (int e = threadIdx.x; e < m; e += blockDim.x)
@@ -449,8 +487,8 @@ struct DyadSwap {
   }
 };
 
-template <bool GM>
-__global__ void __launch_bounds__(kRandThreads) k_randomize_dyads(DyadArgs a) {
+template <bool GM, int WN>
+__global__ void __launch_bounds__(kRandThreads<WN>) k_randomize_dyads(DyadArgs a) {
   extern __shared__ __align__(16) uint32_t dsm[];
   __shared__ RandWindow W;
   __shared__ int scan_tmp[33];
@@ -495,7 +533,7 @@ __global__ void __launch_bounds__(kRandThreads) k_randomize_dyads(DyadArgs a) {
   __syncthreads();
   if (S + D > 0) {
     const DyadSwap pol{a.seeds[g], (uint64_t)S, (uint64_t)D};
-    run_attempts(pol, lists, Sset, W, a.attempts);
+    run_attempts<WN>(pol, lists, Sset, W, a.attempts);
   }
   __syncthreads();
   // arcs back into the rows of the fixed out-CSR shape (order inside a row is
@@ -528,14 +566,15 @@ size_t rand_gscratch_words(int32_t m, int G) {
 }
 
 template <typename Args>
-static cudaError_t launch_rand(void (*in_smem)(Args), void (*in_global)(Args), Args& a, int32_t m,
-                               int G, uint32_t* gscratch, cudaStream_t s) {
+static cudaError_t launch_rand(void (*narrow)(Args), void (*wide)(Args), void (*in_global)(Args),
+                               Args& a, int32_t m, int G, uint32_t* gscratch, cudaStream_t s) {
   a.gscratch = gscratch;
   if (!rand_fits_smem(m)) {
     if (!gscratch) return cudaErrorInvalidValue;
-    in_global<<<G, kRandThreads, 0, s>>>(a);
+    in_global<<<G, kRandThreads<64>, 0, s>>>(a);
     return cudaGetLastError();
   }
+  void (*in_smem)(Args) = m < kWideArcs ? narrow : wide;
   const size_t smem = rand_smem_bytes(m);
   // the limit is the function's, shared by launches of other sizes: always the
   // largest this rule lets through
@@ -547,7 +586,7 @@ static cudaError_t launch_rand(void (*in_smem)(Args), void (*in_global)(Args), A
     e = cudaFuncSetAttribute((const void*)in_smem, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              max_smem - (int)sizeof(RandWindow) - 2048);
   if (e != cudaSuccess) return e;
-  in_smem<<<G, kRandThreads, smem, s>>>(a);
+  in_smem<<<G, m < kWideArcs ? kRandThreads<32> : kRandThreads<64>, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -559,7 +598,8 @@ cudaError_t launch_randomize_dyads(int32_t n, int32_t m, int G, const int32_t* r
   a.n = n; a.m = m; a.G = G;
   a.row_ptr = row_ptr; a.col0 = col0; a.seeds = seeds; a.attempts = attempts;
   a.col_out = col_out; a.scratch = scratch;
-  return launch_rand(k_randomize_dyads<false>, k_randomize_dyads<true>, a, m, G, gscratch, s);
+  return launch_rand(k_randomize_dyads<false, 32>, k_randomize_dyads<false, 64>,
+                     k_randomize_dyads<true, 64>, a, m, G, gscratch, s);
 }
 
 // Enqueue G randomisations of the graph (row_ptr, col0) into col_out.
@@ -570,7 +610,7 @@ cudaError_t launch_randomize(int32_t n, int32_t m, int G, const int32_t* row_ptr
   a.n = n; a.m = m; a.G = G;
   a.row_ptr = row_ptr; a.col0 = col0; a.seeds = seeds; a.swaps = swaps;
   a.col_out = col_out;
-  return launch_rand(k_randomize<false>, k_randomize<true>, a, m, G, gscratch, s);
+  return launch_rand(k_randomize<false, 32>, k_randomize<false, 64>, k_randomize<true, 64>, a, m, G, gscratch, s);
 }
 
 }  // namespace mt

@@ -30,6 +30,13 @@ def test_window_and_buffer_edges(lib, model, attempts):
 
 
 @pytest.mark.parametrize("model", MODELS)
+@pytest.mark.parametrize("m,attempts", [(2999, 31), (2999, 33), (2999, 30000), (3000, 30000)])
+def test_both_window_widths(lib, model, m, attempts):
+    lib.load_library()
+    check(lib, syn.chung_lu_digraph(700, m, 2.2, None, 0.2, 4), model, 13, attempts)
+
+
+@pytest.mark.parametrize("model", MODELS)
 @pytest.mark.parametrize("n,p", [(5, 0.5), (8, 0.6), (12, 0.9), (40, 0.5), (90, 0.7)])
 def test_overlapping_windows_and_full_buckets(lib, model, n, p):
     lib.load_library()

@@ -262,16 +262,16 @@ def run_ours(args, world, rank, local):
 
         def step():
             batch.run(seeds, hists, z)
-        launches_per_step = 9
+        # randomise; scatter, rows, lengths, place; entry counts; plan (totals,
+        # items, and degree sums for cells at k >= 5); count; z-scores
+        launches_per_step = 10 + (1 if method and k >= 5 else 0)
     else:
         hists = torch.empty(C, dtype=torch.int64, device="cuda")
 
         def step():
-            if tuning is None:
-                mt.count(dg, table, hists)
-            else:
-                mt.count_tuned(dg, table, out=hists, method=method)
-        launches_per_step = 5
+            mt.count_tuned(dg, table, out=hists, method=method)
+        # plan, count, and the histogram copies' fold at k = 6
+        launches_per_step = 3 + (1 if method and k >= 5 else 0) + (1 if k == 6 else 0)
 
     for _ in range(max(args.warmup, 3)):
         step()
@@ -344,6 +344,7 @@ def run_ours(args, world, rank, local):
             dist.all_reduce(te, op=dist.ReduceOp.MAX)
             e2e_s = float(te.item())
         e2e = {"value": all_subgraphs / e2e_s, "unit": "subgraphs/s",
+               "method": "automatic (the calls' default: cells)",
                "h2d_bytes_per_step": int(h2d), "d2h_bytes_per_step": int(d2h),
                "ms_per_step": 1000 * e2e_s}
 
@@ -632,11 +633,12 @@ def measure_plain_vs_batched(mt, torch, dg, table, g, batched_graphs_per_s, npla
     graphs = [dg] + [mt.randomize(dg, s, 10 * g.m) for s in range(1, nplain + 1)]
     out = torch.empty(table.num_classes, dtype=torch.int64, device="cuda")
     for gr in graphs:
-        mt.count(gr, table, out)
+        mt.count_tuned(gr, table, out=out, method=mt.METHOD_ENUMERATE)
     torch.cuda.synchronize()
     flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
     it = iter(range(10**9))
-    ms = _timed(torch, lambda: mt.count(graphs[next(it) % len(graphs)], table, out),
+    ms = _timed(torch, lambda: mt.count_tuned(graphs[next(it) % len(graphs)], table, out=out,
+                                                 method=mt.METHOD_ENUMERATE),
                 len(graphs), flush)
     plain = len(graphs) / (ms / 1000.0)
     return {"plain_graphs_per_s": plain, "batched_graphs_per_s": batched_graphs_per_s,
@@ -709,7 +711,7 @@ def measure_serving(mt, torch, have_tables, num=32, seed=0, method=0, round_cost
             "requests": num, "round_cost": round_cost,
             "k_mix": {str(k): ks.count(k) for k in (3, 4, 5, 6)},
             "n_range": [int(min(g.n for _, g in reqs)), int(max(g.n for _, g in reqs))],
-            "all_ok": ok, "method": "cells" if method else "enumerate"}
+            "all_ok": ok, "method": "cells" if method else "automatic (cells)"}
 
 
 def ops_per_subgraph(k: int) -> int:

@@ -1729,8 +1729,9 @@ mt_status count_configure_tuned(CountPlan* p, int K, int G, int nmax, int dmax, 
   p->keep = keep && K >= 5 && p->comb && p->gcache && p->lab_smem && G >= 8 &&
             dmax >= (K == 5 ? kKeepDegree5 : kKeepDegree6);
   const void* kern = pick_kernel(*p);
-  MT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)p->smem_bytes));
+  // the limit belongs to the kernel, not to this plan: a smaller plan made before
+  // a batch runs must not lower it
+  MT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
   int occ = 0;
   MT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, p->warps_per_block * 32,
                                                             p->smem_bytes));

@@ -129,3 +129,24 @@ def test_kept_lists_that_do_not_fit(lib, name):
          "dense_hub": lambda: syn.disjoint_union(syn.random_small_digraph(75, 0.35, 0.5, 2),
                                                  _hub(200, 80, 300, 3))}[name]()
     _batch_equals_single_counts(lib, g, 5, 8)
+
+
+@pytest.mark.parametrize("k", [3, 5, 6])
+def test_smaller_plans_between_a_batch_and_its_run(lib, k):
+    """Plans of one kernel with different shared-memory sizes, the largest made
+    first and run last."""
+    lib.load_library()
+    t = lib.table_build(k)
+    large = lib.graph_from(syn.chung_lu_digraph(400, 1200, 2.3, 40, 0.1, k))
+    small = lib.graph_from(syn.chung_lu_digraph(60, 150, 2.3, 20, 0.1, k))
+    want = lib.count_host(large, t)
+    b = lib.Batch(large, t, 2, 100)
+    bs = lib.Batch(small, t, 2, 100)
+    seeds = np.array([1, 2], dtype=np.uint64)
+    ws = lib.count_host(small, t)
+    np.testing.assert_array_equal(lib.to_numpy_u64(b.run(seeds)[0])[0], want)
+    np.testing.assert_array_equal(lib.to_numpy_u64(bs.run(seeds)[0])[0], ws)
+    assert b.error() == 0 and bs.error() == 0
+    b.free()
+    bs.free()
+    t.free()

@@ -242,7 +242,7 @@ def run_ours(args, world, rank, local):
     swaps = 10 * g.m
 
     method = mt.METHOD_CELLS if args.method == "cells" else mt.METHOD_ENUMERATE
-    tuning = mt.make_tuning(method=method) if method else None
+    tuning = mt.make_tuning(method=method)  # the method by name, also without the autotuner
     tuned = None
     if R and not args.no_autotune:
         from paper_1804_09741_gb300 import autotune

@@ -888,7 +888,8 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
     };
 
     // Exclusive neighbours of lanes' list members, per code, to the counters of
-    // their cells' numbers.
+    // their cells' numbers.  Both forms add atomically, like the kept lists'
+    // corrections: votes and shuffles order no memory between the lanes.
     auto add_exclusive = [&](uint32_t num, uint32_t n1, uint32_t n2, uint32_t n3) {
       const bool some = (n1 | n2 | n3) != 0;
       const uint32_t num0 = __shfl_sync(kFull, num, 0);
@@ -896,11 +897,10 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
         const uint32_t s12 = __reduce_add_sync(kFull, n1 | (n2 << 16));
         const uint32_t s3 = __reduce_add_sync(kFull, n3);
         if (lane == 0) {
-          xs[3 * num0] += s12 & 0xFFFFu;
-          xs[3 * num0 + 1] += s12 >> 16;
-          xs[3 * num0 + 2] += s3;
+          red_add_shared((int*)&xs[3 * num0], (int)(s12 & 0xFFFFu));
+          red_add_shared((int*)&xs[3 * num0 + 1], (int)(s12 >> 16));
+          red_add_shared((int*)&xs[3 * num0 + 2], (int)s3);
         }
-        __syncwarp();
       } else if (some) {
         if (n1) atomicAdd(&xs[3 * num], n1);
         if (n2) atomicAdd(&xs[3 * num + 1], n2);

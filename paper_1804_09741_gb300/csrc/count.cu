@@ -1353,6 +1353,7 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
             const bool v0 = idx < lc;
             const int u0 = v0 ? buf[c + 1 + idx] : 0;
             const uint32_t lt = v0 ? (uint32_t)lab[u0] : 0u;
+            __syncwarp();  // the other choices' lanes read the word too
             if (v0 && h == 0) lab[u0] = (LT)(lt & LM);
             const uint32_t lb = cpt ? (uint32_t)xmw[lt & LM] : (lt & LM);
             for (int p0 = 0; p0 < ng; p0 += P) {

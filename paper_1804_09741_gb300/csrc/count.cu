@@ -2049,7 +2049,9 @@ mt_status mt_set_workspace(mt_graph* g, void* ws, size_t bytes) {
       return MT_EINVAL;
     }
   }
-  // an earlier count may still use the current scratch, on any stream
+  // an earlier count may still use the current scratch, on any stream of the
+  // graph's device
+  DeviceScope on(g->device);
   MT_CUDA_TRY(cudaDeviceSynchronize());
   if (g->ws && g->ws_owned) pool_free(g->ws, nullptr);
   g->ws = ws;

@@ -401,12 +401,11 @@ mt_status graph_alloc(int32_t n, int32_t m, cudaStream_t s, mt_graph** out) {
 
 // Free a graph's memory on `s`, behind everything that uses it there.
 static void graph_free_on(mt_graph* g, cudaStream_t s) {
-  int dev = g->device;
-  cudaGetDevice(&dev);
-  if (dev != g->device) cudaSetDevice(g->device);
-  pool_free(g->mem, s);
-  if (g->ws && g->ws_owned) pool_free(g->ws, s);
-  if (dev != g->device) cudaSetDevice(dev);
+  {
+    DeviceScope on(g->device);
+    pool_free(g->mem, s);
+    if (g->ws && g->ws_owned) pool_free(g->ws, s);
+  }
   if (g->ev0) cudaEventDestroy(g->ev0);
   if (g->ev1) cudaEventDestroy(g->ev1);
   delete g;
@@ -653,7 +652,10 @@ mt_status mt_graph_load_csr(int32_t n, int32_t m, const int32_t* row_ptr, const 
 
 mt_status mt_graph_free(mt_graph* g) {
   if (!g) return MT_OK;
-  cudaDeviceSynchronize();  // counts on any stream may still use it
+  // counts on any stream of the graph's device may still use it, and the pool
+  // orders memory it takes back behind the freeing stream's work only
+  DeviceScope on(g->device);
+  cudaDeviceSynchronize();
   graph_free_on(g, nullptr);
   return MT_OK;
 }

@@ -51,6 +51,24 @@ struct mt_graph {
 
 namespace mt {
 
+// Makes `device` the current one while in scope: what is waited for and the
+// legacy stream that memory is returned on are the current device's.
+class DeviceScope {
+ public:
+  explicit DeviceScope(int device) {
+    if (cudaGetDevice(&before_) != cudaSuccess) before_ = device;
+    if (before_ != device) cudaSetDevice(device);
+    device_ = device;
+  }
+  ~DeviceScope() {
+    if (before_ != device_) cudaSetDevice(before_);
+  }
+  DeviceScope(const DeviceScope&) = delete;
+  DeviceScope& operator=(const DeviceScope&) = delete;
+
+ private:
+  int before_ = 0, device_ = 0;
+};
 
 // Pointers of G graphs of equal degrees laid out with fixed strides.
 struct BuildArgs {

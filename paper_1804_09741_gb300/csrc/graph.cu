@@ -284,9 +284,13 @@ void handle_born() {
 
 void handle_died() {
   std::lock_guard<std::mutex> lock(g_pool_mu);
-  if (--g_live_handles == 0)
-    for (cudaMemPool_t p : g_pools)
-      if (p) cudaMemPoolTrimTo(p, 0);
+  if (--g_live_handles > 0) return;
+  for (int d = 0; d < kPoolDevices; ++d)
+    if (g_pools[d]) {
+      DeviceScope on(d);
+      cudaDeviceSynchronize();  // the frees are stream-ordered: until then nothing can be trimmed
+      cudaMemPoolTrimTo(g_pools[d], 0);
+    }
 }
 
 cudaError_t pool_alloc(void** out, size_t bytes, cudaStream_t s) {

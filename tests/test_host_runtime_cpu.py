@@ -118,3 +118,25 @@ def test_set_workspace_waits_for_the_graphs_device(fake):
     fake.mt_graph_free(g)
     fake.mt_table_free(t)
     fake.fake_free(hist)
+
+
+def test_pools_are_trimmed_after_their_frees_have_run(fake):
+    """Memory freed in stream order is the pool's only once the stream gets there:
+    with the last handle each device is waited for before its pool is trimmed."""
+    fake.cudaSetDevice(1)
+    g1, g2 = fake.graph(*PATH), fake.graph(*PATH)
+    fake.cudaSetDevice(0)
+    g0 = fake.graph(*PATH)
+    fake.mt_graph_free(g1)
+    fake.mt_graph_free(g0)
+    fake.log()
+    fake.mt_graph_free(g2)  # the last one
+    log = calls(fake.log(), "sync", "free_async", "trim")
+    trims = [i for i, e in enumerate(log) if e[0] == "trim"]
+    assert {log[i][1] for i in trims} == {0, 1}
+    for i in trims:
+        last_free = max(j for j, e in enumerate(log[:i]) if e[0] == "free_async")
+        assert ("sync", log[i][1]) in [e[:2] for e in log[last_free:i]]
+    dev = ctypes.c_int()
+    fake.cudaGetDevice(ctypes.byref(dev))
+    assert dev.value == 0

@@ -28,6 +28,11 @@
  * - A handle may be used by one host thread at a time.  Counting calls on one
  *   graph handle share its scratch memory: order them on one stream (or
  *   synchronise between them).
+ * - Counts into a device histogram can be captured into a CUDA graph once an
+ *   earlier count has allocated the handle's scratch (MT_ECUDA otherwise).
+ *   Replays use that scratch, the handle and `hist`: keep them alive (the library
+ *   keeps its own scratch with the handle, also when later counts need more) and
+ *   order replays with the handle's other counts.
  * - Graphs: n vertices numbered 0..n-1 (1 <= n <= 65535), m arcs given as an
  *   int32 CSR of out-neighbours (row_ptr[n+1], col[m]); rows may be unsorted;
  *   self-loops, duplicate arcs, ids outside [0,n) and non-monotone row_ptr are

@@ -257,7 +257,7 @@ static mt_status batch_enqueue(mt_batch* b, cudaStream_t s) {
   MT_CUDA_TRY(cudaGetLastError());
   MT_CUDA_TRY(cudaEventRecordWithFlags(b->ev[1], s, cudaEventRecordExternal));
   MT_CUDA_TRY(cudaMemsetAsync(b->d_hists, 0, (size_t)(R + 1) * b->C * 8, s));
-  if (n >= b->K) MT_TRY(count_enqueue(b->plan, b->ws, b->d_graphs, table_view(b->t), 0, n, s));
+  if (n >= b->K) MT_TRY(count_enqueue(b->plan, b->ws, b->d_graphs, nullptr, table_view(b->t), 0, n, s));
   else MT_CUDA_TRY(cudaMemsetAsync(count_err_ptr(b->plan, b->ws), 0, 4, s));  // no launch sets it
   MT_CUDA_TRY(cudaEventRecordWithFlags(b->ev[2], s, cudaEventRecordExternal));
   if (b->C <= kWarpClasses)

@@ -74,6 +74,8 @@ struct GraphPlan {
   uint32_t qhead, pad;
 };
 
+static_assert(sizeof(GraphPlan) % 8 == 0, "zeroed in 8-byte words");
+
 constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr int kTargetItemsPerWarp = 64;
 // Cell method: an item's least estimated work, below which fetching it and
@@ -1769,8 +1771,19 @@ uint32_t* count_nitems_ptr(const CountPlan& p, void* ws) {
   return &((GraphPlan*)((char*)ws + p.off_gp))->count;
 }
 
+// Start of a one-graph launch: its descriptor, which travels as a kernel argument
+// so that a captured launch holds it and reads no host memory at replay, and
+// zeros in header and plan (`words` 8-byte words).  One kernel for both: in place
+// of the header's memset it costs nothing, beside it a k = 3 count of n = 300 took
+// 76 us, not 69.
+__global__ void __launch_bounds__(32) k_begin(DevGraph* dst, DevGraph src,
+                                              unsigned long long* hdr, int words) {
+  if (threadIdx.x == 0) *dst = src;
+  for (int i = threadIdx.x; i < words; i += blockDim.x) hdr[i] = 0;
+}
+
 template <int K>
-static cudaError_t enqueue_k(const CountPlan& p, void* ws, const DevGraph* graphs,
+static cudaError_t enqueue_k(const CountPlan& p, void* ws, DevGraph* graphs, const DevGraph* one,
                              const TableView& table, int32_t rb, int32_t re, cudaStream_t s,
                              unsigned long long* copies_base, int copies, uint32_t copy_stride) {
   char* base = (char*)ws;
@@ -1779,8 +1792,13 @@ static cudaError_t enqueue_k(const CountPlan& p, void* ws, const DevGraph* graph
   Item* items = (Item*)(base + p.off_items);
   void* lab = base + p.off_lab;
   // header and graph plans are neighbours
-  cudaError_t e = cudaMemsetAsync(base + p.off_hdr, 0,
-                                  p.off_gp - p.off_hdr + (size_t)p.G * sizeof(GraphPlan), s);
+  const size_t zeros = p.off_gp - p.off_hdr + (size_t)p.G * sizeof(GraphPlan);
+  cudaError_t e = cudaSuccess;
+  if (one)
+    k_begin<<<1, 32, 0, s>>>(graphs, *one, (unsigned long long*)(base + p.off_hdr),
+                             (int)(zeros / 8));
+  else
+    e = cudaMemsetAsync(base + p.off_hdr, 0, zeros, s);
   if (e != cudaSuccess) return e;
   SplitArgs sa;
   sa.split_cost = p.split_cost;
@@ -1847,18 +1865,19 @@ static cudaError_t enqueue_k(const CountPlan& p, void* ws, const DevGraph* graph
   return cudaLaunchKernel(pick_kernel(p), dim3(p.blocks), dim3(threads), args, p.smem_bytes, s);
 }
 
-mt_status count_enqueue(const CountPlan& p, void* ws, const DevGraph* graphs,
+mt_status count_enqueue(const CountPlan& p, void* ws, DevGraph* graphs, const DevGraph* one,
                         const TableView& table, int32_t root_begin, int32_t root_end,
                         cudaStream_t s, unsigned long long* copies_base, int copies,
                         uint32_t copy_stride) {
   if (copies > 1 && (p.K != 6 || p.G != 1 || !copies_base)) return MT_EINVAL;
+  if (one && p.G != 1) return MT_EINVAL;
   cudaError_t e;
   switch (p.K) {
-    case 3: e = enqueue_k<3>(p, ws, graphs, table, root_begin, root_end, s, nullptr, 1, 0); break;
-    case 4: e = enqueue_k<4>(p, ws, graphs, table, root_begin, root_end, s, nullptr, 1, 0); break;
-    case 5: e = enqueue_k<5>(p, ws, graphs, table, root_begin, root_end, s, nullptr, 1, 0); break;
+    case 3: e = enqueue_k<3>(p, ws, graphs, one, table, root_begin, root_end, s, nullptr, 1, 0); break;
+    case 4: e = enqueue_k<4>(p, ws, graphs, one, table, root_begin, root_end, s, nullptr, 1, 0); break;
+    case 5: e = enqueue_k<5>(p, ws, graphs, one, table, root_begin, root_end, s, nullptr, 1, 0); break;
     default:
-      e = enqueue_k<6>(p, ws, graphs, table, root_begin, root_end, s, copies_base, copies,
+      e = enqueue_k<6>(p, ws, graphs, one, table, root_begin, root_end, s, copies_base, copies,
                        copy_stride);
       break;
   }
@@ -1878,6 +1897,19 @@ static size_t count_scratch_bytes(const CountPlan& p, uint32_t C) {
   return p.ws_bytes + 256 + (size_t)count_hist_copies(p) * round16((size_t)C * 8);
 }
 
+// Give up g's scratch: the library's own goes back to the pool on `s`, or stays
+// with the handle when a captured count uses it.  The caller has waited for the
+// counts that use it.
+static void drop_scratch(mt_graph* g, cudaStream_t s) {
+  if (g->ws && g->ws_owned) {
+    if (g->ws_captured) g->captured_ws.push_back(g->ws);
+    else pool_free(g->ws, s);
+    g->ws_captured = false;
+  }
+  g->ws = nullptr;
+  g->ws_bytes = 0;
+}
+
 // Plain one-graph count with the workspace cached in the graph handle.
 static mt_status count_one(const mt_graph* gc, const mt_table* t, uint64_t* hist,
                            int32_t rb, int32_t re, const mt_tuning* tuning, cudaStream_t s) {
@@ -1894,24 +1926,22 @@ static mt_status count_one(const mt_graph* gc, const mt_table* t, uint64_t* hist
                    " bytes, this count needs " + std::to_string(need));
     return MT_EINVAL;
   }
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  MT_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
+  const bool captured = cap != cudaStreamCaptureStatusNone;
   if (g->ws_bytes < need) {
     // scratch outlives a captured launch, so it is not allocated by one
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    MT_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
-    if (cap != cudaStreamCaptureStatusNone) {
+    if (captured) {
       set_last_error("the first count of a graph allocates scratch: not under stream capture");
       return MT_ECUDA;
     }
-    if (g->ws) {
-      // an earlier count may still use the old scratch, on any stream
-      MT_CUDA_TRY(cudaDeviceSynchronize());
-      pool_free(g->ws, s);
-      g->ws = nullptr;
-      g->ws_bytes = 0;
-    }
+    // an earlier count may still use the old scratch, on any stream
+    if (g->ws) MT_CUDA_TRY(cudaDeviceSynchronize());
+    drop_scratch(g, s);
     MT_CUDA_TRY(pool_alloc(&g->ws, need, s));
     g->ws_bytes = need;
   }
+  if (captured && g->ws_owned) g->ws_captured = true;
   if (!g->ev0) {
     MT_CUDA_TRY(cudaEventCreate(&g->ev0));
     MT_CUDA_TRY(cudaEventCreate(&g->ev1));
@@ -1939,8 +1969,7 @@ static mt_status count_one(const mt_graph* gc, const mt_table* t, uint64_t* hist
     if (original_scratch_bytes(g) > p.ws_bytes - p.off_items) return MT_EOVERFLOW;
     MT_TRY(graph_build_original(g, base + p.off_items, s));  // before the items are written
   }
-  DevGraph hg = dev_view(g, dh, part);
-  MT_CUDA_TRY(cudaMemcpyAsync(dg, &hg, sizeof(DevGraph), cudaMemcpyHostToDevice, s));
+  const DevGraph hg = dev_view(g, dh, part);
   MT_CUDA_TRY(cudaMemsetAsync(dh, 0, (size_t)C * 8, s));
   if (g->n >= K && rb < re) {
     const int copies = count_hist_copies(p);
@@ -1949,7 +1978,7 @@ static mt_status count_one(const mt_graph* gc, const mt_table* t, uint64_t* hist
     MT_CUDA_TRY(cudaEventRecord(g->ev0, s));
     if (copies > 1)
       MT_CUDA_TRY(cudaMemsetAsync(cbase, 0, (size_t)(copies - 1) * stride * 8, s));
-    MT_TRY(count_enqueue(p, g->ws, dg, table_view(t), rb, re, s, cbase, copies, stride));
+    MT_TRY(count_enqueue(p, g->ws, dg, &hg, table_view(t), rb, re, s, cbase, copies, stride));
     if (copies > 1) {
       const unsigned fb = (unsigned)std::min<uint32_t>((C + 255) / 256, 152u * 8u);
       k_fold_copies<<<fb, 256, 0, s>>>(dh, cbase, copies - 1, C, stride);
@@ -2053,7 +2082,7 @@ mt_status mt_set_workspace(mt_graph* g, void* ws, size_t bytes) {
   // graph's device
   DeviceScope on(g->device);
   MT_CUDA_TRY(cudaDeviceSynchronize());
-  if (g->ws && g->ws_owned) pool_free(g->ws, nullptr);
+  drop_scratch(g, nullptr);
   g->ws = ws;
   g->ws_bytes = ws ? bytes : 0;
   g->ws_owned = ws == nullptr;

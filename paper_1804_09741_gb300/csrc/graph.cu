@@ -409,6 +409,7 @@ static void graph_free_on(mt_graph* g, cudaStream_t s) {
     DeviceScope on(g->device);
     pool_free(g->mem, s);
     if (g->ws && g->ws_owned) pool_free(g->ws, s);
+    for (void* p : g->captured_ws) pool_free(p, s);
   }
   if (g->ev0) cudaEventDestroy(g->ev0);
   if (g->ev1) cudaEventDestroy(g->ev1);

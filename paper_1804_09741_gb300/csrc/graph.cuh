@@ -2,6 +2,8 @@
 // undirected CSR) shared by the loader, the randomiser and the batch path.
 #pragma once
 
+#include <vector>
+
 #include "common.cuh"
 
 namespace mt {
@@ -40,9 +42,13 @@ struct mt_graph {
 
   // Counting scratch, grown on demand by mt_count, or the caller's buffer
   // attached by mt_set_workspace (ws_owned false: never grown or freed here).
+  // Scratch that a captured count uses stays until the handle goes: its CUDA
+  // graph may be replayed after a larger count has moved on to another buffer.
   void* ws = nullptr;
   size_t ws_bytes = 0;
   bool ws_owned = true;
+  bool ws_captured = false;         // a captured count uses ws
+  std::vector<void*> captured_ws;   // earlier ones
   // Where the last count left its error word and item count inside `ws`.
   bool stats_valid = false;
   size_t off_err = 0, off_nitems = 0;

@@ -54,9 +54,6 @@ static mt_status scratch_address(void** out) {
   return MT_OK;
 }
 
-// Writes the graph descriptor into the fixed scratch (no host staging copy).
-__global__ void k_put_graph(DevGraph* dst, DevGraph src) { *dst = src; }
-
 static mt_status count_noalloc(const mt_graph* g, const mt_table* t, uint64_t* hist,
                                cudaStream_t s) {
   int dev = 0;
@@ -95,11 +92,10 @@ static mt_status count_noalloc(const mt_graph* g, const mt_table* t, uint64_t* h
     return MT_EUNSUPPORTED;
   }
   DevGraph* dg = (DevGraph*)((char*)scratch + desc_off);
-  k_put_graph<<<1, 1, 0, s>>>(dg, dev_view(g, (unsigned long long*)hist));
-  MT_CUDA_TRY(cudaGetLastError());
+  const DevGraph hg = dev_view(g, (unsigned long long*)hist);
   MT_CUDA_TRY(cudaMemsetAsync(hist, 0, (size_t)C * 8, s));
   if (g->n >= K) {
-    MT_TRY(count_enqueue(p, scratch, dg, table_view(t), 0, g->n, s));
+    MT_TRY(count_enqueue(p, scratch, dg, &hg, table_view(t), 0, g->n, s));
   } else {
     // no launch: clear the status word a previous call left behind
     MT_CUDA_TRY(cudaMemsetAsync(count_err_ptr(p, scratch), 0, 4, s));

@@ -476,8 +476,8 @@ static mt_status step(mt_server* s, int32_t* completed) {
     for (int ki = 0; ki < 4; ++ki) {
       if (by_k[ki].empty()) continue;
       MT_CUDA_TRY(cudaStreamWaitEvent(s->kstream[ki], s->fork_ev, 0));
-      MT_TRY(count_enqueue(plans[ki], s->ws[ki], s->d_graphs[ki], table_view(s->tables[ki]), 0,
-                           nmaxs[ki], s->kstream[ki]));
+      MT_TRY(count_enqueue(plans[ki], s->ws[ki], s->d_graphs[ki], nullptr,
+                           table_view(s->tables[ki]), 0, nmaxs[ki], s->kstream[ki]));
       MT_CUDA_TRY(cudaMemcpyAsync(R.h_err + ki, count_err_ptr(plans[ki], s->ws[ki]), 4,
                                   cudaMemcpyDeviceToHost, s->kstream[ki]));
       MT_CUDA_TRY(cudaEventRecord(s->kdone_ev[ki], s->kstream[ki]));

@@ -140,3 +140,32 @@ def test_pools_are_trimmed_after_their_frees_have_run(fake):
     dev = ctypes.c_int()
     fake.cudaGetDevice(ctypes.byref(dev))
     assert dev.value == 0
+
+
+def test_captured_count_holds_no_host_memory_and_keeps_its_scratch(fake):
+    """What a captured count uploads is read at every replay, so it uploads nothing
+    from the host; and the scratch it uses stays, whatever later counts need."""
+    g, t3, t4 = fake.graph(*PATH), fake.table(3), fake.table(4)
+    hist = fake.fake_alloc(8 * 199)
+    assert fake.mt_count(g, t3, hist, STREAM) == mt.MT_OK
+    fake.fake_set_capturing(STREAM)
+    fake.log()
+    assert fake.mt_count(g, t3, hist, STREAM) == mt.MT_OK
+    assert fake.mt_count_roots(g, t3, 1, 3, hist, STREAM) == mt.MT_OK
+    log = fake.log()
+    assert not calls(log, "captured_upload")
+    assert not calls(log, "malloc", "free_async", "sync", "sync_stream")
+    # nothing is allocated under capture
+    assert fake.mt_count(g, t4, hist, STREAM) == mt.MT_ECUDA
+    fake.fake_set_capturing(None)
+    fake.log()
+    assert fake.mt_count(g, t4, hist, STREAM) == mt.MT_OK  # moves on to more scratch
+    log = fake.log()
+    assert calls(log, "malloc") and not calls(log, "free_async")
+    assert fake.mt_set_workspace(g, None, 0) == mt.MT_OK  # gives that back, not the captured one
+    assert len(calls(fake.log(), "free_async")) == 1
+    fake.mt_graph_free(g)
+    assert len(calls(fake.log(), "free_async")) == 2  # the arrays and the captured scratch
+    fake.mt_table_free(t3)
+    fake.mt_table_free(t4)
+    fake.fake_free(hist)

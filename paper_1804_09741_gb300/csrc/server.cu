@@ -234,58 +234,17 @@ static void drop_load(mt_server* s, SrvRequest* r, mt_status st) {
   r->t_done = now_ms(s);
 }
 
-// The loads of a round's admissions are enqueued one after another and waited
-// for once.
-static void admit(mt_server* s) {
-  std::vector<SrvRequest*> loading;
-  while (!s->pending.empty() && (int)s->active.size() < s->max_slots) {
-    SrvRequest* r = s->pending.front();
-    const uint32_t C = table_classes(s->tables[r->k - 3]);
-    r->bytes = request_bytes(r, C);
-    if (r->bytes > s->budget) {  // can never fit
-      s->pending.pop_front();
-      r->state = 3;
-      r->status = MT_EBUSY;
-      r->t_done = now_ms(s);
-      continue;
-    }
-    // the scratch r's k needs with r active, against what k holds now
-    const int ki = r->k - 3;
-    const size_t need_k = std::max(s->reserved[ki], scratch_need(s, ki, r));
-    if (r->bytes + need_k > s->budget) {  // can never fit, even alone
-      s->pending.pop_front();
-      r->state = 3;
-      r->status = MT_EBUSY;
-      r->t_done = now_ms(s);
-      continue;
-    }
-    if (s->used + r->bytes + reserved_total(s) - s->reserved[ki] + need_k > s->budget) break;
-    s->pending.pop_front();
-    mt_status st = graph_load_begin(r->n, r->m, r->rp.data(), r->col.data(), s->load_stream,
-                                    s->h_stats + loading.size(), &r->g);
-    if (st == MT_OK) st = acquire_pinned(s, r->k, C, &r->h_result);
-    if (st == MT_OK) {
-      cudaError_t e = pool_alloc((void**)&r->d_hist, (size_t)C * 8, s->load_stream);
-      if (e == cudaSuccess) e = cudaMemsetAsync(r->d_hist, 0, (size_t)C * 8, s->load_stream);
-      if (e != cudaSuccess) {
-        set_last_error(cudaGetErrorString(e));
-        st = MT_ECUDA;
-      }
-    }
-    if (st != MT_OK) {
-      drop_load(s, r, st);
-      continue;
-    }
-    s->used += r->bytes;
-    s->reserved[ki] = need_k;
-    r->state = 1;
-    r->t_admit = now_ms(s);
-    r->next_root = 0;
-    s->active.push_back(r);
-    loading.push_back(r);
-  }
-  if (loading.empty()) return;
+// Free k's round scratch once no active request of k is left (stream-ordered
+// behind every launch enqueued so far) and drop its reservation.
+static void release_idle_scratch(mt_server* s);
+
+// Wait for the loads enqueued so far.  A load that failed leaves nothing charged:
+// its request's memory, its slot, and what it added to its k's reservation
+// (`before` = the reservations without the loads).  Returns whether any failed.
+static bool settle_loads(mt_server* s, std::vector<SrvRequest*>& loading, size_t before[4]) {
+  if (loading.empty()) return false;
   const cudaError_t e = cudaStreamSynchronize(s->load_stream);
+  bool failed[4] = {false, false, false, false}, any = false;
   for (size_t i = 0; i < loading.size(); ++i) {
     SrvRequest* r = loading[i];
     std::vector<int32_t>().swap(r->rp);
@@ -295,8 +254,74 @@ static void admit(mt_server* s) {
       s->active.erase(std::find(s->active.begin(), s->active.end(), r));
       s->used -= std::min(s->used, r->bytes);
       drop_load(s, r, st);
+      failed[r->k - 3] = any = true;
     }
   }
+  for (int ki = 0; ki < 4; ++ki) {
+    if (failed[ki]) s->reserved[ki] = std::max(before[ki], scratch_need(s, ki, nullptr));
+    before[ki] = s->reserved[ki];
+  }
+  if (any) release_idle_scratch(s);
+  loading.clear();
+  return any;
+}
+
+// The loads of a round's admissions are enqueued one after another and waited
+// for once: when nothing more is admitted.  If some failed, what they held is free
+// for the requests behind them.
+static void admit(mt_server* s) {
+  std::vector<SrvRequest*> loading;
+  size_t before[4];
+  std::copy(s->reserved, s->reserved + 4, before);
+  do {
+    while (!s->pending.empty() && (int)s->active.size() < s->max_slots) {
+      SrvRequest* r = s->pending.front();
+      const uint32_t C = table_classes(s->tables[r->k - 3]);
+      r->bytes = request_bytes(r, C);
+      if (r->bytes > s->budget) {  // can never fit
+        s->pending.pop_front();
+        r->state = 3;
+        r->status = MT_EBUSY;
+        r->t_done = now_ms(s);
+        continue;
+      }
+      // the scratch r's k needs with r active, against what k holds now
+      const int ki = r->k - 3;
+      const size_t need_k = std::max(s->reserved[ki], scratch_need(s, ki, r));
+      if (r->bytes + need_k > s->budget) {  // can never fit, even alone
+        if (settle_loads(s, loading, before)) continue;
+        s->pending.pop_front();
+        r->state = 3;
+        r->status = MT_EBUSY;
+        r->t_done = now_ms(s);
+        continue;
+      }
+      if (s->used + r->bytes + reserved_total(s) - s->reserved[ki] + need_k > s->budget) break;
+      s->pending.pop_front();
+      mt_status st = graph_load_begin(r->n, r->m, r->rp.data(), r->col.data(), s->load_stream,
+                                      s->h_stats + loading.size(), &r->g);
+      if (st == MT_OK) st = acquire_pinned(s, r->k, C, &r->h_result);
+      if (st == MT_OK) {
+        cudaError_t e = pool_alloc((void**)&r->d_hist, (size_t)C * 8, s->load_stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(r->d_hist, 0, (size_t)C * 8, s->load_stream);
+        if (e != cudaSuccess) {
+          set_last_error(cudaGetErrorString(e));
+          st = MT_ECUDA;
+        }
+      }
+      if (st != MT_OK) {
+        drop_load(s, r, st);
+        continue;
+      }
+      s->used += r->bytes;
+      s->reserved[ki] = need_k;
+      r->state = 1;
+      r->t_admit = now_ms(s);
+      r->next_root = 0;
+      s->active.push_back(r);
+      loading.push_back(r);
+    }
+  } while (settle_loads(s, loading, before));
 }
 
 // Grow k's round scratch to this round's plan.  The admitted requests' plan
@@ -319,8 +344,6 @@ static mt_status ensure_capacity(mt_server* s, int ki, size_t ws_need, size_t gr
   return MT_OK;
 }
 
-// Free k's round scratch once no active request of k is left (stream-ordered
-// behind every launch enqueued so far) and drop its reservation.
 static void release_idle_scratch(mt_server* s) {
   for (int ki = 0; ki < 4; ++ki) {
     bool any = false;

@@ -169,3 +169,113 @@ def test_captured_count_holds_no_host_memory_and_keeps_its_scratch(fake):
     fake.mt_table_free(t3)
     fake.mt_table_free(t4)
     fake.fake_free(hist)
+
+
+class FakeServer:
+    def __init__(self, fake, tables, budget, slots=8):
+        self.fake = fake
+        h = ctypes.c_void_p()
+        ts = [tables.get(k) for k in (3, 4, 5, 6)]
+        assert fake.mt_server_create(*ts, budget, slots, 1e9, ctypes.byref(h)) == mt.MT_OK
+        self.h = h.value
+
+    def submit(self, k, n, rp, col):
+        rp, col = np.array(rp, np.int32), np.array(col, np.int32)
+        rid = ctypes.c_uint64()
+        assert self.fake.mt_server_submit(self.h, k, n, int(rp[-1]), rp.ctypes.data,
+                                          col.ctypes.data, ctypes.byref(rid)) == mt.MT_OK
+        return rid.value
+
+    def step(self):
+        assert self.fake.mt_server_step(self.h, None, None, None) == mt.MT_OK
+
+    def state(self, rid):
+        """(state, status) without taking the result."""
+        st = ctypes.c_int32()
+        status = self.fake.mt_server_result(self.h, rid, ctypes.byref(st), None, None)
+        return st.value, status
+
+    def used(self):
+        u = ctypes.c_size_t()
+        assert self.fake.mt_server_used_bytes(self.h, ctypes.byref(u)) == mt.MT_OK
+        return u.value
+
+    def free(self):
+        self.fake.mt_server_free(self.h)
+
+
+def _used_by_one(fake, tables, k):
+    s = FakeServer(fake, tables, 1 << 40)
+    s.submit(k, *PATH)
+    s.step()
+    used = s.used()
+    s.free()
+    return used
+
+
+@pytest.mark.parametrize("good_first", [False, True])
+def test_failed_load_leaves_no_charge(fake, good_first):
+    """A duplicate arc is found on the device, after the request and its k's
+    scratch have been charged: both charges go with it, and requests of another k
+    are admitted under a budget that holds one k's scratch at a time."""
+    tables = {k: fake.table(k) for k in (3, 4)}
+    one = {k: _used_by_one(fake, tables, k) for k in (3, 4)}
+    s = FakeServer(fake, tables, max(one.values()) + 4096)
+    if good_first:  # after rounds have run, too
+        rid = s.submit(3, *PATH)
+        for _ in range(3):
+            s.step()
+        assert s.state(rid) == (2, mt.MT_OK)
+    fake.fake_poke(16, 8, 2)  # the next build finds a duplicate arc
+    bad = s.submit(3, 4, [0, 2, 2, 2, 2], [1, 1])
+    for _ in range(2):
+        s.step()
+    assert s.state(bad)[1] == mt.MT_EINVAL
+    assert s.used() == 0
+    good = s.submit(4, *PATH)
+    for _ in range(4):
+        s.step()
+    assert s.state(good) == (2, mt.MT_OK)
+    assert s.used() == 0
+    s.free()
+    for t in tables.values():
+        fake.mt_table_free(t)
+
+
+def test_failed_load_beside_a_good_one_is_charged_no_more(fake):
+    """Of two requests of one k admitted together the failed one's share of the
+    scratch is given back at once."""
+    tables = {3: fake.table(3)}
+    one = _used_by_one(fake, tables, 3)
+    s = FakeServer(fake, tables, 1 << 40)
+    fake.fake_poke(16, 8, 2)
+    big = 400
+    bad = s.submit(3, big + 1, [0] + [big] * (big + 1), list(range(1, big)) + [1])
+    good = s.submit(3, *PATH)
+    s.step()
+    assert s.state(bad)[1] == mt.MT_EINVAL
+    assert s.used() == one
+    for _ in range(3):
+        s.step()
+    assert s.state(good) == (2, mt.MT_OK) and s.used() == 0
+    s.free()
+    fake.mt_table_free(tables[3])
+
+
+@pytest.mark.parametrize("slots", [1, 8])
+def test_failed_load_does_not_refuse_the_requests_behind_it(fake, slots):
+    """A request that fits the budget alone is not refused, nor left out of a
+    round, for the memory or the slot of one whose load fails."""
+    tables = {3: fake.table(3)}
+    s = FakeServer(fake, tables, _used_by_one(fake, tables, 3) + 64, slots)
+    fake.fake_poke(16, 8, 2)
+    bad = s.submit(3, 4, [0, 2, 2, 2, 2], [1, 1])
+    good = s.submit(3, *PATH)
+    s.step()
+    assert s.state(bad)[1] == mt.MT_EINVAL
+    assert s.state(good) == (1, mt.MT_OK)
+    for _ in range(2):
+        s.step()
+    assert s.state(good) == (2, mt.MT_OK) and s.used() == 0
+    s.free()
+    fake.mt_table_free(tables[3])

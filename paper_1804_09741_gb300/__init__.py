@@ -18,6 +18,7 @@ Names follow the C ABI with the ``mt_`` prefix dropped:
 from __future__ import annotations
 
 import ctypes
+import enum
 import os
 
 import numpy as np
@@ -36,7 +37,13 @@ class Tuning(ctypes.Structure):
                 ("method", ctypes.c_int)]
 
 
-METHOD_ENUMERATE, METHOD_CELLS = 0, 1
+class Method(enum.IntEnum):
+    """mt_method."""
+    ENUMERATE = 0
+    CELLS = 1
+
+
+METHOD_ENUMERATE, METHOD_CELLS = Method
 NULL_ARC_SWAP, NULL_DYAD_SWAP = 0, 1
 
 

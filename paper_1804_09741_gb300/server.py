@@ -8,13 +8,17 @@ import time
 
 import numpy as np
 
-from . import MT_OK, _check, _ptr, load_library
+from . import MT_OK, Method, _check, _ptr, load_library
 
 _vp = ctypes.c_void_p
 
 
 class Server:
-    """Continuous-batching server over resident per-k tables."""
+    """Continuous-batching server over resident per-k tables.
+
+    `method`: a counting method by its name, METHOD_ENUMERATE or METHOD_CELLS;
+    the default, a plain 0, leaves the choice to the library (the names are enum
+    members, so METHOD_ENUMERATE is told from it although its value is 0)."""
 
     def __init__(self, tables: dict, memory_budget: int = 8 << 30, max_slots: int = 64,
                  round_cost: float = 1.6e9, method: int = 0):
@@ -25,7 +29,7 @@ class Server:
         _check(self.lib.mt_server_create(*ts, int(memory_budget), int(max_slots),
                                          float(round_cost), ctypes.byref(h)), "mt_server_create")
         self.handle = h.value
-        if method:
+        if method or isinstance(method, Method):
             _check(self.lib.mt_server_set_method(self.handle, int(method)),
                    "mt_server_set_method")
 

@@ -126,3 +126,19 @@ def test_batches(lib, tables, k):
             np.testing.assert_array_equal(h[r], oracle_dense(oracle.count(gr, k)[0],
                                                              t.class_masks()))
         b.free()
+
+
+def test_server_by_name(lib, tables):
+    """Rounds of per-subgraph launches, over all k and with a compact table."""
+    from paper_1804_09741_gb300.server import Server, run_stream
+    ts = {3: tables(3), 4: tables(4), 5: tables(5), 6: tables(6, True)}
+    reqs = [(k, syn.chung_lu_digraph(n, 3 * n, 2.3, 25, 0.2, 10 * k + n))
+            for k in (3, 4, 5, 6) for n in ([40, 200, 600] if k < 6 else [30, 60, 110])]
+    srv = Server(ts, memory_budget=2 << 30, max_slots=6, round_cost=2e6,
+                 method=lib.METHOD_ENUMERATE)
+    out, _, _ = run_stream(srv, reqs)
+    for (k, g), (st, hist, status) in zip(reqs, out):
+        assert st == 2, status
+        np.testing.assert_array_equal(hist, per_subgraph(lib, lib.graph_from(g), ts[k]))
+    assert srv.used_bytes() == 0
+    srv.free()

@@ -279,3 +279,31 @@ def test_failed_load_does_not_refuse_the_requests_behind_it(fake, slots):
     assert s.state(good) == (2, mt.MT_OK) and s.used() == 0
     s.free()
     fake.mt_table_free(tables[3])
+
+
+@pytest.mark.parametrize("method,want", [(None, []), (0, []), (mt.METHOD_ENUMERATE, [0]),
+                                         (mt.METHOD_CELLS, [1]), (1, [1])])
+def test_python_server_follows_a_method_asked_for_by_name(fake, monkeypatch, method, want):
+    from paper_1804_09741_gb300 import server
+
+    class Table:
+        handle = fake.table(3)
+
+    class Recording:
+        calls = []
+
+        def __getattr__(self, name):
+            if name == "mt_server_set_method":
+                return lambda h, m: self.calls.append(m) or fake.mt_server_set_method(h, m)
+            return getattr(fake, name)
+    Recording.calls = []
+    monkeypatch.setattr(server, "load_library", Recording)
+    srv = server.Server({3: Table}) if method is None else server.Server({3: Table}, method=method)
+    assert Recording.calls == want
+    srv.free()
+    fake.mt_table_free(Table.handle)
+
+
+def test_methods_are_the_abi_values():
+    assert (mt.METHOD_ENUMERATE, mt.METHOD_CELLS) == (0, 1)
+    assert mt.make_tuning(method=mt.METHOD_CELLS).method == 1

@@ -181,22 +181,39 @@ __global__ void __launch_bounds__(256) k_place(BuildArgs a) {
   }
 }
 
-cudaError_t launch_build(const BuildArgs& a, cudaStream_t s) {
-  if (a.G <= 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(a.cursor, 0, (size_t)a.G * a.n * 4, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(a.stats, 0, (size_t)a.G * sizeof(BuildStats), s);
-  if (e != cudaSuccess) return e;
-  const int most = std::max(1, 8192 / a.G);  // blocks per graph
-  if (a.m > 0) k_scatter<<<dim3(std::min((a.m + 255) / 256, most), a.G), 256, 0, s>>>(a);
+// The launches' y dimension is the graph, of which a grid has at most 65,535.
+constexpr int kGridGraphs = 65535;
+
+cudaError_t launch_build(const BuildArgs& all, cudaStream_t s) {
+  if (all.G <= 0) return cudaSuccess;
+  cudaError_t e = cudaMemsetAsync(all.cursor, 0, (size_t)all.G * all.n * 4, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(all.stats, 0, (size_t)all.G * sizeof(BuildStats), s);
   // 8 warps of bitmaps, 4 for graphs of more than 48,000 vertices
-  const size_t per_warp = (size_t)bitmap_words(a.n) * 8;
+  const size_t per_warp = (size_t)bitmap_words(all.n) * 8;
   const int warps = per_warp * 8 > 96 * 1024 ? 4 : 8;
-  e = cudaFuncSetAttribute((const void*)k_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           96 * 1024);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute((const void*)k_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             96 * 1024);
   if (e != cudaSuccess) return e;
-  k_rows<<<dim3(std::min((a.n + warps - 1) / warps, most), a.G), warps * 32, per_warp * warps, s>>>(a);
-  k_lengths<<<a.G, 1024, 0, s>>>(a);
-  k_place<<<dim3(std::min((a.n + 7) / 8, most), a.G), 256, 0, s>>>(a);
+  for (int g0 = 0; g0 < all.G; g0 += kGridGraphs) {
+    BuildArgs a = all;
+    a.G = std::min(all.G - g0, kGridGraphs);
+    const size_t n0 = (size_t)g0 * a.n, m0 = (size_t)g0 * a.m;
+    a.col_in += m0;
+    a.tmp += 2 * m0;
+    a.cursor += n0;
+    a.urow += n0 + g0;
+    a.ucol += 2 * m0;
+    a.usrc += 2 * m0;
+    a.ufwd += n0;
+    a.stats += g0;
+    const int most = std::max(1, 8192 / a.G);  // blocks per graph
+    if (a.m > 0) k_scatter<<<dim3(std::min((a.m + 255) / 256, most), a.G), 256, 0, s>>>(a);
+    k_rows<<<dim3(std::min((a.n + warps - 1) / warps, most), a.G), warps * 32, per_warp * warps,
+             s>>>(a);
+    k_lengths<<<a.G, 1024, 0, s>>>(a);
+    k_place<<<dim3(std::min((a.n + 7) / 8, most), a.G), 256, 0, s>>>(a);
+  }
   return cudaGetLastError();
 }
 

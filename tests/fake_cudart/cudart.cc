@@ -23,6 +23,7 @@ std::map<char*, std::pair<size_t, int>> g_mem;  // device memory: bytes, device
 std::deque<Poke> g_pokes;
 std::map<const void*, std::string> g_kernels;
 int g_device = 0;
+cudaError_t g_error = cudaSuccess;  // of a launch
 void* g_capturing = nullptr;  // stream under capture
 uintptr_t g_next = 0x1000;    // streams, events, pools
 
@@ -91,7 +92,11 @@ cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
   return cudaSuccess;
 }
 const char* cudaGetErrorString(cudaError_t) { return "fake"; }
-cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaGetLastError() {
+  const cudaError_t e = g_error;
+  g_error = cudaSuccess;
+  return e;
+}
 
 // ---- memory
 cudaError_t cudaMalloc(void** p, size_t n) { *p = device_alloc(n); note("malloc", *p); return cudaSuccess; }
@@ -132,10 +137,10 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t s, cudaStreamCaptureStatus* st) {
   *st = g_capturing && s == g_capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
   return cudaSuccess;
 }
-cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaErrorNotSupported; }
-cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t*) { return cudaErrorNotSupported; }
-cudaError_t cudaGraphInstantiate(cudaGraphExec_t*, cudaGraph_t, unsigned long long) { return cudaErrorNotSupported; }
-cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaErrorNotSupported; }
+cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaSuccess; }
+cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) { *g = handle<cudaGraph_t>(); return cudaSuccess; }
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t, unsigned long long) { *e = handle<cudaGraphExec_t>(); return cudaSuccess; }
+cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
 cudaError_t cudaEventCreate(cudaEvent_t* e) { *e = handle<cudaEvent_t>(); return cudaSuccess; }
@@ -154,7 +159,9 @@ cudaError_t cudaLaunchKernel(const void* f, dim3 grid, dim3, void**, size_t, cud
   snprintf(line, sizeof(line), "grid=%ux%ux%u ", grid.x, grid.y, grid.z);
   const auto it = g_kernels.find(f);
   note((std::string("launch ") + line + (it == g_kernels.end() ? "?" : it->second)).c_str());
-  return grid.y > 65535 || grid.z > 65535 ? cudaErrorInvalidConfiguration : cudaSuccess;
+  if (grid.x < 1 || grid.y < 1 || grid.z < 1 || grid.y > 65535 || grid.z > 65535)
+    g_error = cudaErrorInvalidConfiguration;
+  return g_error;
 }
 cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3 b, void** a, size_t sm, cudaStream_t s) {
   return cudaLaunchKernel((const void*)k, g, b, a, sm, s);

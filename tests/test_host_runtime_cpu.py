@@ -307,3 +307,23 @@ def test_python_server_follows_a_method_asked_for_by_name(fake, monkeypatch, met
 def test_methods_are_the_abi_values():
     assert (mt.METHOD_ENUMERATE, mt.METHOD_CELLS) == (0, 1)
     assert mt.make_tuning(method=mt.METHOD_CELLS).method == 1
+
+
+@pytest.mark.parametrize("R", [65535, 65536, 140000])
+def test_batches_past_a_grid_dimension(fake, R):
+    """The builder's launches have a graph per step of the grid's y dimension,
+    which ends at 65,535; a batch of more null graphs (too small to hold a k-set,
+    so nothing is counted) is built in parts."""
+    g, t = fake.graph(2, [0, 1, 1], [1]), fake.table(3)
+    h = ctypes.c_void_p()
+    assert fake.mt_batch_create(g, t, R, 1, ctypes.byref(h)) == mt.MT_OK
+    seeds = np.zeros(R, np.uint64)
+    hist = fake.fake_alloc((R + 1) * 13 * 8)
+    fake.log()
+    assert fake.mt_batch_run(h.value, seeds.ctypes.data, hist, None, None) == mt.MT_OK
+    grids = [re.match(r"launch grid=(\d+)x(\d+)x(\d+) .*k_scatter", e[0]) for e in fake.log()]
+    assert sum(int(m[2]) for m in grids if m) == R
+    fake.mt_batch_free(h.value)
+    fake.mt_graph_free(g)
+    fake.mt_table_free(t)
+    fake.fake_free(hist)

@@ -406,6 +406,12 @@ mt_status mt_batch_phase_ms(const mt_batch* b, float out[3]);
  * device. */
 mt_status mt_batch_error(const mt_batch* b, uint32_t* err);
 
+/* The batch's counting launch, as mt_count_launch_info; layout bit 8 = the cell
+ * method keeps lists (what the sets below one list share is read once).
+ * Errors: MT_EINVAL. */
+mt_status mt_batch_launch_info(const mt_batch* b, int32_t* warps_per_block, int32_t* blocks,
+                               int32_t* stack_cap, uint32_t* layout);
+
 /* One-shot form of the batch: create, run, free. */
 mt_status mt_count_batch(const mt_graph* g, const mt_table* t, const uint64_t* seeds, int R,
                          uint64_t swaps, uint64_t* hists, double* z, void* stream);

@@ -87,6 +87,7 @@ SIGNATURES = {
     "mt_batch_run": (ctypes.c_int, [_vp, _vp, _vp, _vp, _vp]),
     "mt_batch_phase_ms": (ctypes.c_int, [_vp, _P(ctypes.c_float)]),
     "mt_batch_error": (ctypes.c_int, [_vp, _P(_u32)]),
+    "mt_batch_launch_info": (ctypes.c_int, [_vp, _P(_i32), _P(_i32), _P(_i32), _P(_u32)]),
     "mt_count_batch": (ctypes.c_int, [_vp, _vp, _vp, ctypes.c_int, _u64, _vp, _vp, _vp]),
     "mt_probe_rates": (ctypes.c_int, [_u64, _u64, _P(_f64), _P(_f64)]),
     "mt_server_create": (ctypes.c_int, [_vp, _vp, _vp, _vp, ctypes.c_size_t, ctypes.c_int, _f64,
@@ -326,13 +327,17 @@ def count_noalloc_error(stream=None) -> int:
     return int(err.value)
 
 
-def launch_info(g: Graph, k: int) -> dict:
-    """The automatic counting launch for `g` at k (mt_count_launch_info)."""
-    w, b, cap, lay = _i32(), _i32(), _i32(), _u32()
-    _check(_lib.mt_count_launch_info(g.handle, int(k), w, b, cap, lay), "mt_count_launch_info")
+def _launch(w, b, cap, lay) -> dict:
     return {"warps_per_block": w.value, "blocks": b.value, "stack_cap": cap.value,
             "graph_in_smem": bool(lay.value & 1), "words_in_smem": bool(lay.value & 2),
             "stacks_in_global": bool(lay.value & 4)}
+
+
+def launch_info(g: Graph, k: int) -> dict:
+    """The automatic counting launch for `g` at k (mt_count_launch_info)."""
+    info = _i32(), _i32(), _i32(), _u32()
+    _check(_lib.mt_count_launch_info(g.handle, int(k), *info), "mt_count_launch_info")
+    return _launch(*info)
 
 
 def workspace_query(g: Graph, k: int) -> int:
@@ -444,6 +449,12 @@ class Batch:
         out = (ctypes.c_float * 3)()
         _check(_lib.mt_batch_phase_ms(self.handle, out), "mt_batch_phase_ms")
         return list(out)
+
+    def launch_info(self) -> dict:
+        """The batch's counting launch (mt_batch_launch_info)."""
+        info = _i32(), _i32(), _i32(), _u32()
+        _check(_lib.mt_batch_launch_info(self.handle, *info), "mt_batch_launch_info")
+        return {**_launch(*info), "keeps_lists": bool(info[3].value & 8)}
 
     def error(self) -> int:
         e = _u32()

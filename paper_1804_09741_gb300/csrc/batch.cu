@@ -390,6 +390,13 @@ mt_status mt_batch_error(const mt_batch* b, uint32_t* err) {
   return MT_OK;
 }
 
+mt_status mt_batch_launch_info(const mt_batch* b, int32_t* warps_per_block, int32_t* blocks,
+                               int32_t* stack_cap, uint32_t* layout) {
+  if (!b) return MT_EINVAL;
+  plan_info(b->plan, warps_per_block, blocks, stack_cap, layout);
+  return MT_OK;
+}
+
 mt_status mt_count_batch(const mt_graph* g, const mt_table* t, const uint64_t* seeds, int R,
                          uint64_t swaps, uint64_t* hists, double* z, void* stream) {
   TraceRange tr("mt_count_batch");

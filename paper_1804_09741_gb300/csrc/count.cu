@@ -61,9 +61,8 @@
 namespace mt {
 
 struct Hdr {
-  uint32_t head;
   uint32_t err;
-  uint32_t pad0, pad1;
+  uint32_t pad[3];
 };
 
 // The planner's result for one graph: its estimated work, and its items
@@ -532,7 +531,7 @@ struct CountArgs {
   unsigned long long* hist_copies;  // copies 1 .. copies-1 of a one-graph k = 6 histogram
   int copies;                // 1 = every block adds into the graph's own histogram
   uint32_t copy_stride;      // elements between two copies
-  int G, nmax, nu_cap, cap;
+  int G, nmax, cap;
   uint32_t classes;
   int graph_bytes, hist_bytes, lab_bytes, buf_bytes, cell_bytes, map_bytes;
   unsigned long long idle_ns;  // a warp waiting for donated work gives up after this
@@ -1764,6 +1763,16 @@ mt_status count_configure_tuned(CountPlan* p, int K, int G, int nmax, int dmax, 
   return MT_OK;
 }
 
+void plan_info(const CountPlan& p, int32_t* warps_per_block, int32_t* blocks, int32_t* stack_cap,
+               uint32_t* layout) {
+  if (warps_per_block) *warps_per_block = p.warps_per_block;
+  if (blocks) *blocks = p.blocks;
+  if (stack_cap) *stack_cap = p.cap;
+  if (layout)
+    *layout = (p.gcache ? 1u : 0u) | (p.lab_smem ? 2u : 0u) | (p.stack_global ? 4u : 0u) |
+              (p.keep ? 8u : 0u);
+}
+
 uint32_t* count_err_ptr(const CountPlan& p, void* ws) {
   return &((Hdr*)((char*)ws + p.off_hdr))->err;
 }
@@ -1852,7 +1861,6 @@ static cudaError_t enqueue_k(const CountPlan& p, void* ws, DevGraph* graphs, con
   a.copy_stride = copy_stride;
   a.G = p.G;
   a.nmax = p.nmax;
-  a.nu_cap = p.nu_cap;
   a.cap = p.cap;
   a.classes = p.classes;
   a.graph_bytes = (int)p.graph_bytes;
@@ -2058,11 +2066,7 @@ mt_status mt_count_launch_info(const mt_graph* g, int k, int32_t* warps_per_bloc
   CountPlan p;
   MT_TRY(count_configure_tuned(&p, k, 1, g->n, g->dmax, g->nu / 2 + 1, std::max(g->nu, 1),
                                kNumClasses[k], nullptr));
-  if (warps_per_block) *warps_per_block = p.warps_per_block;
-  if (blocks) *blocks = p.blocks;
-  if (stack_cap) *stack_cap = p.cap;
-  if (layout)
-    *layout = (p.gcache ? 1u : 0u) | (p.lab_smem ? 2u : 0u) | (p.stack_global ? 4u : 0u);
+  plan_info(p, warps_per_block, blocks, stack_cap, layout);
   return MT_OK;
 }
 

@@ -5,7 +5,6 @@
 
 namespace mt {
 
-const uint32_t* table_device(const mt_table* t);
 int table_k(const mt_table* t);
 uint32_t table_classes(const mt_table* t);
 TableView table_view(const mt_table* t);
@@ -68,6 +67,10 @@ mt_status count_enqueue(const CountPlan& p, void* ws, DevGraph* graphs, const De
                         const TableView& table, int32_t root_begin, int32_t root_end,
                         cudaStream_t s, unsigned long long* copies_base = nullptr,
                         int copies = 1, uint32_t copy_stride = 0);
+
+// A plan for mt_count_launch_info and mt_batch_launch_info.
+void plan_info(const CountPlan& p, int32_t* warps_per_block, int32_t* blocks, int32_t* stack_cap,
+               uint32_t* layout);
 
 // Read the launch's error word and item count from the workspace (device
 // pointers into `ws`).  The header holding the error word is at offset 0 of

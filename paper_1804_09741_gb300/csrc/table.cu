@@ -756,7 +756,6 @@ TableView table_view(const mt_table* t) {
 }
 bool table_compact(const mt_table* t) { return t->compact; }
 
-const uint32_t* table_device(const mt_table* t) { return t->table; }
 int table_k(const mt_table* t) { return t->k; }
 uint32_t table_classes(const mt_table* t) { return t->classes; }
 

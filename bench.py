@@ -270,8 +270,8 @@ def run_ours(args, world, rank, local):
 
         def step():
             mt.count_tuned(dg, table, out=hists, method=method)
-        # plan, count, and the histogram copies' fold at k = 6
-        launches_per_step = 3 + (1 if method and k >= 5 else 0) + (1 if k == 6 else 0)
+        # descriptor, plan, count, and the histogram copies' fold at k = 6
+        launches_per_step = 4 + (1 if method and k >= 5 else 0) + (1 if k == 6 else 0)
 
     for _ in range(max(args.warmup, 3)):
         step()
@@ -395,7 +395,8 @@ def run_ours(args, world, rank, local):
             "note": "same workloads counted with MT_METHOD_CELLS (Algorithm 1 of Sec. 3: the "
                     "last two vertices counted per cell pair); histograms identical"}
         extra["serving"] = measure_serving(mt, torch, {5: table})
-        extra["serving_cells"] = measure_serving(mt, torch, {5: table}, method=1)
+        extra["serving_per_subgraph"] = measure_serving(mt, torch, {5: table},
+                                                        method=mt.METHOD_ENUMERATE)
 
     gar = None
     if rank == 0 and R and count_ms:
@@ -438,9 +439,11 @@ def _timed(torch, fn, steps, flush):
 
 
 def _ceilings(mt, k, sub_rate, method="enumerate", workload=None):
-    """The count kernel's global-memory work against the measured ceilings of
+    """The count kernel's global-memory work against the measured rates of
     random 4 B reads from a table of 2^(k(k-1)) words (the k-vertex table) and
     random 64-bit atomic adds into the class count's power of two of counters.
+    The rates are references, not ceilings: the kernel's reads have locality
+    (neighbouring slots below one prefix), so a fraction can be above 1.
 
     The kernel does not read the table once per subgraph: it reads once per
     group of equal keys.  So the reads and reductions it actually issues per
@@ -471,6 +474,7 @@ def _ceilings(mt, k, sub_rate, method="enumerate", workload=None):
     out["note"] = ("issued global-load and global-reduction sectors per classified subgraph "
                    "(ncu, a smaller batch on the same code path) x the kernel's subgraphs/s, over the "
                    "measured random-read and random-atomic rates (mt_probe_rates, this run); "
+                   "reads with locality can pass the random rate; "
                    + cap.get("reading", ""))
     return out
 
@@ -666,16 +670,18 @@ def serving_requests(num, seed):
     return out
 
 
-def measure_serving(mt, torch, have_tables, num=32, seed=0, method=0, round_cost=1.6e9):
+def measure_serving(mt, torch, have_tables, num=32, seed=0, method=None, round_cost=1.6e9):
     """Continuous-batching server on a seeded stream of mixed-k requests:
-    closed-loop capacity first, then Poisson arrivals at 80% of it."""
+    closed-loop capacity first, then Poisson arrivals at 80% of it.  `method`: None,
+    the calls' own choice, or a method by name."""
     from paper_1804_09741_gb300.server import Server, poisson_arrivals, run_stream
     reqs = serving_requests(num, seed)
     tables = dict(have_tables)
     for k in (3, 4, 5, 6):
         if k not in tables:
             tables[k] = mt.table_build(k)
-    srv = Server(tables, memory_budget=16 << 30, max_slots=32, round_cost=round_cost, method=method)
+    srv = Server(tables, memory_budget=16 << 30, max_slots=32, round_cost=round_cost,
+                 method=0 if method is None else method)
     run_stream(srv, reqs[:4])  # warm-up
     res, lat, wall = run_stream(srv, reqs)
     cap = num / wall
@@ -688,7 +694,7 @@ def measure_serving(mt, torch, have_tables, num=32, seed=0, method=0, round_cost
     # back to the host, one request after another
     def plain(k, g):
         dg = mt.graph_from(g)
-        if method:
+        if method is not None:
             h = mt.to_numpy_u64(mt.count_tuned(dg, tables[k], method=method))
         else:
             h = mt.count_host(dg, tables[k])
@@ -711,7 +717,7 @@ def measure_serving(mt, torch, have_tables, num=32, seed=0, method=0, round_cost
             "requests": num, "round_cost": round_cost,
             "k_mix": {str(k): ks.count(k) for k in (3, 4, 5, 6)},
             "n_range": [int(min(g.n for _, g in reqs)), int(max(g.n for _, g in reqs))],
-            "all_ok": ok, "method": "cells" if method else "automatic (cells)"}
+            "all_ok": ok, "method": "automatic (cells)" if method is None else method.name.lower()}
 
 
 def ops_per_subgraph(k: int) -> int:

@@ -223,18 +223,20 @@ mt_status mt_count_roots(const mt_graph* g, const mt_table* t, int32_t root_begi
  *   and partitions the pairs above it). */
 typedef enum { MT_METHOD_ENUMERATE = 0, MT_METHOD_CELLS = 1 } mt_method;
 
-/* Launch tuning of the enumerator (all fields 0 = automatic).
+/* Launch tuning of the enumerator (0 = automatic, except `method`, whose 0 is
+ * MT_METHOD_ENUMERATE: a call without a tuning, which counts by cells, is faster
+ * than one with every field 0).
  * - split_cost: estimated work (classified subgraphs, or list entries of the
  *   cell method) above which a first-level
  *   extension branch of a root is split into second-level work items, and the
  *   target size of first-level items; the root-split threshold.
  * - split_scale: when split_cost is 0, a multiplier of the automatic threshold
  *   (the graph's total estimate spread over 64 items per resident warp).
- *   The threshold is never set below 1/5 of the automatic one, which bounds the
- *   number of work items.
+ *   The threshold is never set below 1/5 of the automatic one (the one without
+ *   the cell method's least item), which bounds the number of work items.
  * - warps_per_block: block size in warps, 1..32.
  * - stack_cap: candidate-stack entries per warp (the stack depth).  Automatic is
- *   (k-1) * max degree + 32, which cannot overflow; a smaller value saves shared
+ *   (k-2) * max degree + 32, which cannot overflow; a smaller value saves shared
  *   memory, and an overflow is detected and reported as MT_EOVERFLOW.
  * - method: an mt_method. */
 typedef struct {
@@ -360,8 +362,8 @@ mt_status mt_randomize(const mt_graph* src, uint64_t seed, uint64_t swaps, void*
  * unless the entries coincide, a == c, b == d, a == d, c == b, or a new pair is
  * already adjacent in either direction.  In- and out-degrees, each vertex's
  * number of mutual partners and the dyad census are preserved.  Synchronises
- * `stream`.  Graphs whose arc set does not fit shared memory (m above about
- * 17,000) keep it in global memory.  Errors: MT_EINVAL, MT_ENOMEM, MT_ECUDA. */
+ * `stream`.  Graphs whose arc set does not fit shared memory (m above 16,384)
+ * keep it in global memory, here and in mt_randomize.  Errors: MT_EINVAL, MT_ENOMEM, MT_ECUDA. */
 mt_status mt_randomize_dyads(const mt_graph* src, uint64_t seed, uint64_t attempts, void* stream,
                              mt_graph** out);
 
@@ -374,7 +376,8 @@ mt_status mt_batch_create(const mt_graph* g, const mt_table* t, int R, uint64_t 
                           mt_batch** out);
 mt_status mt_batch_free(mt_batch* b);
 
-/* mt_batch_create with explicit tuning of the counting launch (NULL = automatic). */
+/* mt_batch_create with explicit tuning of the counting launch (NULL = automatic,
+ * by cells; see mt_tuning). */
 mt_status mt_batch_create_tuned(const mt_graph* g, const mt_table* t, int R, uint64_t swaps,
                                 const mt_tuning* tuning, mt_batch** out);
 

@@ -36,7 +36,7 @@
 //    three choices at a time instead (see kWideTailBlocksPerGraph); at k = 6,
 //    short candidate lists let several choices share one pass, a (choice,
 //    candidate) pair per lane;
-//  * MT_METHOD_CELLS, the automatic choice at k = 5 and 6, stops one level
+//  * MT_METHOD_CELLS, the automatic choice at every k, stops one level
 //    earlier and counts the last two vertices per pair of cells (Algorithm 1 of
 //    Sec. 3; see pair_level below);
 //  * histograms: per-block shared-memory 32-bit counters for k <= 5 (13 / 199
@@ -88,8 +88,13 @@ constexpr double kCellsItemFloor = K == 3 ? 1024.0 : 128.0;
 // Adds one warp may make to a shared 32-bit histogram between two flushes of
 // it by exchange (enumeration path, k <= 5; see `ladd` in k_count).
 constexpr int kLeafBudget = 1 << 25;
-// The same for the cell method, whose adds also come in larger steps: a counter
-// stays below warps x (2^24 + one list's pairs (at most 2^24) + 32 rows' adds).
+// The same for the cell method, whose adds also come in larger steps: one list's
+// pairs (at most 2^24, or they go to the graph's counters), 32 rows' arcs, and the
+// list's exclusive counts.  Those are charged as the rows are read but added at the
+// list's end, so a flush in between leaves them uncharged: at most one list's per
+// warp, each below 2^20 (larger ones go to the graph's counters), and one class
+// takes few of a list's (cell, code) counts.  So a counter stays below 32 warps x
+// (2 x 2^24 and a few 2^20) < 2^31.
 constexpr int kCellBudget = 1 << 24;
 // Items a block's warps can hand to each other at once (work donation).
 constexpr int kDonSlots = 32;
@@ -394,7 +399,8 @@ using LabT = typename std::conditional<
 // Neighbour entries as the enumerator reads them: the graph's 32-bit entries
 // (vertex in bits 0..29, arc code in bits 30..31) or, in the shared-memory copy
 // the cell method makes of graphs of fewer than 2^14 vertices, 16-bit ones
-// (vertex in bits 0..13, code in bits 14..15).
+// (vertex in bits 0..13, code in bits 14..15).  2^14 is what the format holds; the
+// layout rule stops making copies earlier (near n = 4,000 at two arcs per vertex).
 __device__ __forceinline__ int ent_vertex(uint32_t e) { return (int)(e & kVertexMask); }
 __device__ __forceinline__ uint32_t ent_code(uint32_t e) { return e >> 30; }
 constexpr int kMaxVertices16 = 1 << 14;
@@ -919,7 +925,7 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) k_count(CountArgs a
     // cell and the arc code between y and u, so exclusive neighbours are
     // counted per (cell, code).
     // Bound by instruction issue (75% of cycles on the k = 5 workload: 68
-    // candidates, 6 cells and 830 row entries per X).  A lane per row segment
+    // candidates and 6 cells per X).  A lane per row segment
     // needs one search and no ballots for 8 entries where a lane per entry
     // needed a 5-step search and a match for each 32; the k = 5 batch (257 graphs)
     // went from 260 to 187 ms, the k = 6 one (65 graphs) from 112 to 71 ms.

@@ -250,9 +250,10 @@ __global__ void __launch_bounds__(256) k_degrees(int n, int m, const int32_t* __
 // (degrees of 4,095 and more are one class), and the places of their rows before
 // merging.  A set belongs to its smallest number, so hubs are roots: their
 // neighbours are off the lists of every later root, and the rows that a list's
-// members are read for are the short ones.  On the k = 5 workload (ids half
-// in this order already) a (k-2)-set's rows shrink from 818 to 530 entries: the
-// 257-graph batch counts in 138 ms, 194 in the original numbering.
+// members are read for are the short ones.  On the k = 5 workload graph (ids half
+// in this order already) the rows of a 3-set's choices hold 453 entries above the
+// root, 742 in the original numbering: the 257-graph batch counted in 138 ms, 194
+// in the original numbering.
 constexpr int kDegreeBins = 4096;
 __global__ void __launch_bounds__(1024) k_rank(int n, const int32_t* __restrict__ deg,
                                                int32_t* rank, int32_t* off) {

@@ -144,7 +144,10 @@ static mt_status batch_create(const mt_graph* g0, const mt_table* t, int R, uint
   b->null_model = null_model;
   mt_status st = count_configure_tuned(&b->plan, K, R + 1, n, dbound,
                                        (int64_t)(R + 1) * std::max(m, 1),
-                                       2 * (int64_t)std::max(m, 1), C, tuning, table_compact(t));
+                                       2 * (int64_t)std::max(m, 1), C, tuning, table_compact(t),
+                                       kAutoMethod,
+                                       (R + 1) * estimate_sets(K, n, deg.data(), rp.data(),
+                                                               col.data()));
   if (st != MT_OK) {
     delete b;
     return st;

@@ -550,15 +550,28 @@ template <int K>
 constexpr int kCells = 1 << (2 * (K - 2));
 constexpr int kNumbered = 64;
 // Kept lists (see keep_list): arcs of one list, and the choices and members that
-// a list must have for it to be worth noting.  Launches use them over 8 and more
-// graphs (the items of fewer have too few choices of one list) of these degrees.
-// Measured on a GB300, count phase without and with: k = 5, n = 1,500, degree 287,
-// 257 graphs 141 : 102 ms, 33 graphs 18.3 : 13.6; degree 142 21.0 : 16.3; 106 10.7 :
-// 9.3; 70 8.4 : 7.9; 61 4.3 : 4.3; 57 3.3 : 3.6.  k = 6: degree 53 72.6 : 69.1, 45
-// 28.5 : 27.7, 42 10.9 : 11.1.  Kernels of their own: the tests for kept lists in
-// the common one cost the other lists 8 to 13%.
+// a list must have for it to be worth noting.  Launches over 8 and more graphs use
+// them (for one graph they lost, 756 : 837 us; 2 to 7 are untried, but for 4 at k = 6,
+// 4.6 : 4.5 ms) when the degrees give long lists and an item holds enough sets to
+// share one.  Measured on a GB300, count phase without and with, ms:
+//  * by degree, 257 graphs, k = 5: 142 21.0 : 16.3, 106 10.7 : 9.3, 70 8.4 : 7.9, 61
+//    4.3 : 4.3, 57 3.3 : 3.6; 65 graphs, k = 6: 53 72.6 : 69.1, 45 28.5 : 27.7, 42
+//    10.9 : 11.1;
+//  * by estimated sets per item, k = 5: the workload graph (n = 1,500) at 6.7 (8 graphs)
+//    3.86 : 4.00, 7.6 4.30 : 4.29, 8.4 4.77 : 4.56, 13 7.4 : 5.8, 217 (257 graphs) 116 :
+//    85; n = 700 at 7 3.79 : 3.85, 10 4.97 : 4.38; n = 400 at 7 2.70 : 2.86, 14 5.2 : 4.8; a
+//    hub of degree 400 in a sparse background at 2.8 1.85 : 1.95, 12 6.4 : 5.3; hubs of 64 to
+//    200 and small graphs, at 0.4 to 4, lost 5 to 8%;
+//  * k = 6: the workload graph (n = 800) at 26 (8 graphs) 8.9 : 8.5, 210 (65) 71.3 : 67.9;
+//    n = 500 at 15 5.18 : 5.02; a hub of degree 150 at 16 5.3 : 5.1; hubs of 44 and 80, at 1 to
+//    12, lost 6 to 10%; n = 300, degree 46, at 17 to 109 0.984 to 0.993.  Dense graphs,
+//    whose lists have more arcs than are kept, lose 2%.
+// Server rounds are indifferent (1,420 : 1,415 requests/s).  Kernels of their own: the
+// tests for kept lists in the common one cost the other lists 8 to 13%.
 constexpr int kKeptArcs = 1024;
+constexpr int kKeepGraphs = 8;
 constexpr int kKeepDegree5 = 64, kKeepDegree6 = 44;
+constexpr double kKeepSets5 = 8.0, kKeepSets6 = 16.0;  // per item
 constexpr int kKeepChoices = 8, kKeepLength = 32;
 
 // Persistent enumerator.  A thread block works on one graph at a time: its
@@ -1618,7 +1631,7 @@ static const void* pick_kernel(const CountPlan& p) {
 
 mt_status count_configure_tuned(CountPlan* p, int K, int G, int nmax, int dmax, int64_t fwd_bound,
                                 int64_t entry_stride, uint32_t classes, const mt_tuning* tuning,
-                                bool compact, int method, bool keep) {
+                                bool compact, int method, double sets) {
   if (tuning) method = tuning->method;
   if (K < 3 || K > 6 || G < 1 || nmax < 1) return MT_EINVAL;
   const double split_cost = tuning ? tuning->split_cost : 0.0;
@@ -1734,8 +1747,11 @@ mt_status count_configure_tuned(CountPlan* p, int K, int G, int nmax, int dmax, 
   p->lab_bytes = lab_bytes;
   p->buf_bytes = buf_bytes - cell_bytes - kLevelBytes - p->map_bytes;
   p->cell_bytes = cell_bytes;
-  p->keep = keep && K >= 5 && p->comb && p->gcache && p->lab_smem && G >= 8 &&
-            dmax >= (K == 5 ? kKeepDegree5 : kKeepDegree6);
+  // (one block per SM, as in every layout that keeps lists)
+  p->keep = K >= 5 && p->comb && p->gcache && p->lab_smem && G >= kKeepGraphs &&
+            dmax >= (K == 5 ? kKeepDegree5 : kKeepDegree6) &&
+            sets >= (K == 5 ? kKeepSets5 : kKeepSets6) * sms * p->warps_per_block *
+                        kTargetItemsPerWarp;
   const void* kern = pick_kernel(*p);
   // the limit belongs to the kernel, not to this plan: a smaller plan made before
   // a batch runs must not lower it
@@ -1767,6 +1783,20 @@ mt_status count_configure_tuned(CountPlan* p, int K, int G, int nmax, int dmax, 
   }
   p->ws_bytes = off + 256;
   return MT_OK;
+}
+
+double estimate_sets(int K, int n, const int32_t* deg, const int32_t* row_ptr, const int32_t* col) {
+  double sets = 0.0;
+  if (K == 5)
+    for (int v = 0; v < n; ++v) sets += 0.5 * deg[v] * (deg[v] - 1.0);
+  if (K == 6)
+    for (int v = 0; v < n; ++v) {
+      const double d = deg[v];
+      double ends = 0.0;
+      for (int32_t e = row_ptr[v]; e < row_ptr[v + 1]; ++e) ends += deg[col[e]] - 1.0;
+      sets += d * (d - 1.0) * (d - 2.0) / 6.0 + (d - 1.0) * ends;
+    }
+  return sets;
 }
 
 void plan_info(const CountPlan& p, int32_t* warps_per_block, int32_t* blocks, int32_t* stack_cap,

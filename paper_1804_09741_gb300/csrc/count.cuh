@@ -47,13 +47,19 @@ struct CountPlan {
 // `tuning` as in include/motifs.h (nullptr = automatic, with the
 // counting method `method`: an mt_method, or kAutoMethod for the library's
 // choice).  `compact`: the table is the compact k = 6 form (an explicit
-// MT_METHOD_CELLS is then MT_EUNSUPPORTED).  `keep`: let the cell method keep
-// lists' arcs in the workspace (about 8 KB per warp, tens of MB).
+// MT_METHOD_CELLS is then MT_EUNSUPPORTED).  `sets`: estimated (k-2)-sets of the
+// launch, by which the cell method keeps lists' arcs in the workspace (about 8 KB
+// per warp, tens of MB) or not; 0: it does not.
 constexpr int kAutoMethod = -1;
 mt_status count_configure_tuned(CountPlan* p, int K, int G, int nmax, int dmax, int64_t fwd_bound,
                                 int64_t entry_stride, uint32_t classes, const mt_tuning* tuning,
                                 bool compact = false, int method = kAutoMethod,
-                                bool keep = true);
+                                double sets = 0.0);
+
+// (k-2)-sets of one graph at k = 5 and 6 (0 below), estimated from its degrees
+// (in + out): paths of two edges, stars and paths of three.  Sets with triangles
+// count more than once.
+double estimate_sets(int K, int n, const int32_t* deg, const int32_t* row_ptr, const int32_t* col);
 
 // Enqueue planner + enumerator.  `graphs` is a device array of G DevGraph whose
 // hist pointers are already zeroed (the launch adds into them).  `one` (G = 1

@@ -80,7 +80,7 @@ static mt_status count_noalloc(const mt_graph* g, const mt_table* t, uint64_t* h
   size_t desc_off = 0, need = 0;
   for (const int method : {kAutoMethod, (int)MT_METHOD_ENUMERATE}) {
     MT_TRY(count_configure_tuned(&p, K, 1, g->n, g->dmax, g->nu / 2 + 1, g->nu > 0 ? g->nu : 1, C,
-                                 nullptr, table_compact(t), method, false));
+                                 nullptr, table_compact(t), method));
     desc_off = (p.ws_bytes + 255) & ~(size_t)255;
     need = desc_off + 256;
     if (need <= kNoAllocScratchBytes) break;

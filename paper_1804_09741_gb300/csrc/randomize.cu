@@ -175,7 +175,10 @@ constexpr int kRunners = 4 * WN;
 template <int WN>
 constexpr int kRandThreads = kRunners<WN> + 64;  // two warps draw
 // Graphs of fewer arcs run windows of 32: little of a wider one passes (20 of 32
-// attempts at m = 1,500, 24 of 64), and it takes half the warps.
+// attempts at m = 1,500, 24 of 64), and it takes half the warps.  Randomise phase of
+// 1 and 511 null graphs, 32 against 64, ms: m = 1,500 0.72 : 0.85 and 1.00 : 1.45, 2,500
+// 1.01 : 1.08 and 2.25 : 2.52, 3,000 1.32 : 1.36 and 2.90 : 3.08, 3,500 1.72 : 1.68 and
+// 3.83 : 3.79, 4,000 2.18 : 2.01 and 4.85 : 4.61, 6,000 2.39 : 2.20 and 5.36 : 5.34.
 constexpr int kWideArcs = 3000;
 constexpr int kDraws = 256;      // attempts per buffer of drawn positions
 constexpr int kKeyTab = 512, kPosTab = 512;

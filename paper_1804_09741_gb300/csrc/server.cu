@@ -45,6 +45,7 @@ struct SrvRequest {
   int32_t n = 0, m = 0;
   std::vector<int32_t> rp, col;  // host copy until admitted
   std::vector<double> cum;       // cumulative per-root cost estimate (n+1)
+  double sets = 0;               // estimated (k-2)-sets (k = 5 and 6)
   int32_t dmax_b = 0;            // bounds for planning before the device build:
   int32_t nu_b = 0;              //   largest in+out degree, 2m undirected entries
   uint32_t taint = 0;            // device error bits of launches its chunks ran in
@@ -120,6 +121,7 @@ static void root_costs(SrvRequest* r) {
   r->dmax_b = 1;
   for (int v = 0; v < n; ++v) r->dmax_b = std::max(r->dmax_b, deg[v]);
   r->nu_b = std::max(2 * r->m, 1);
+  r->sets = estimate_sets(r->k, n, deg.data(), r->rp.data(), r->col.data());
   std::vector<double> of_sum(2 * (size_t)r->dmax_b + 1);
   for (size_t d = 0; d < of_sum.size(); ++d) of_sum[d] = 1.0 + choose_d((double)d, r->k - 2);
   // the numbering of the roots: by descending degree, as the device build's (the
@@ -155,7 +157,9 @@ static mt_status plan_for(const mt_server* s, int ki, const SrvRequest* extra, C
                           int* G) {
   int nmax = 1, dmax = 1, numax = 1, g = 0;
   int64_t fwd = 0;
+  double sets = 0;
   auto add = [&](const SrvRequest* r) {
+    sets += r->sets;
     nmax = std::max(nmax, r->n);
     dmax = std::max(dmax, r->dmax_b);
     numax = std::max(numax, r->nu_b);
@@ -169,7 +173,8 @@ static mt_status plan_for(const mt_server* s, int ki, const SrvRequest* extra, C
   if (g == 0) return MT_OK;
   return count_configure_tuned(p, ki + 3, g, nmax, dmax, fwd, numax,
                                table_classes(s->tables[ki]), nullptr,
-                               table_compact(s->tables[ki]), s->method, keep_lists(s));
+                               table_compact(s->tables[ki]), s->method,
+                               keep_lists(s) ? sets : 0.0);
 }
 
 // Round scratch of k's launch (planner and work queue, graph descriptors) for
@@ -455,7 +460,10 @@ static mt_status step(mt_server* s, int32_t* completed) {
       const uint32_t C = table_classes(t);
       int nmax = 1, dmax = 1, numax = 1;
       int64_t fwd = 0;
+      double sets = 0;
       for (auto& c : chunks) {
+        const std::vector<double>& cum = c.r->cum;
+        sets += c.r->sets * (cum[c.b] - cum[c.a]) / cum[c.r->n];
         nmax = std::max(nmax, c.r->g->n);
         dmax = std::max(dmax, c.r->g->dmax);
         numax = std::max(numax, c.r->g->nu);
@@ -464,7 +472,7 @@ static mt_status step(mt_server* s, int32_t* completed) {
       CountPlan p;
       mt_status cst = count_configure_tuned(&p, K, (int)chunks.size(), nmax, dmax, fwd, numax, C,
                                             nullptr, table_compact(t), s->method,
-                                            keep_lists(s));
+                                            keep_lists(s) ? sets : 0.0);
       if (cst == MT_OK) cst = ensure_capacity(s, ki, p.ws_bytes, chunks.size());
       if (cst == MT_OK)  // charge what is held, should the plan outgrow the reservation
         s->reserved[ki] = std::max(s->reserved[ki],

@@ -53,8 +53,9 @@ def _two_hubs(leaves, arcs, seed):
     return syn.csr_from_arcs(2 + leaves, a[:, 0], a[:, 1])
 
 
-@pytest.mark.parametrize("leaves", [1020, 1023, 1024, 1060])
-def test_rows_at_the_limit_of_kept_counts(lib, leaves):
+@pytest.mark.parametrize("leaves,R", [(1020, 8), (1023, 8), (1023, 7), (1023, 6), (1024, 8),
+                                      (1060, 8)])
+def test_rows_at_the_limit_of_kept_counts(lib, leaves, R):
     """A kept list's counts hold rows of up to 1,023 entries; with a longer row in
     it (the second hub's, in the list below the first hub and a leaf) the sets
     read all rows."""
@@ -65,50 +66,59 @@ def test_rows_at_the_limit_of_kept_counts(lib, leaves):
     assert dg.max_degree == leaves
     want = lib.to_numpy_u64(lib.count_tuned(dg, t, method=lib.METHOD_ENUMERATE))
     assert lib.count_stats(dg)[1] == 0
-    b = lib.Batch(dg, t, 8, 0)  # no swaps: nine times the same graph
-    assert b.launch_info()["keeps_lists"]
-    h = lib.to_numpy_u64(b.run(np.arange(1, 9, dtype=np.uint64))[0])
+    b = lib.Batch(dg, t, R, 0)  # no swaps: the same graph R + 1 times
+    assert b.launch_info()["keeps_lists"] == (R >= 7)  # from 8 graphs on
+    h = lib.to_numpy_u64(b.run(np.arange(1, R + 1, dtype=np.uint64))[0])
     assert b.error() == 0
-    for r in range(9):
+    for r in range(R + 1):
         np.testing.assert_array_equal(h[r], want)
     b.free()
     dg.free()
     t.free()
 
 
-@pytest.mark.parametrize("k,n,p", [(5, 90, 0.3), (6, 64, 0.4)])
-def test_lists_of_more_arcs_than_are_kept(lib, k, n, p):
+@pytest.mark.parametrize("k,n,p,R", [(5, 90, 0.3, 31), (6, 64, 0.4, 7)])
+def test_lists_of_more_arcs_than_are_kept(lib, k, n, p, R):
     """Dense graphs: lists with more than the 1,024 arcs that fit."""
     lib.load_library()
     t = lib.table_build(k)
     g = syn.random_small_digraph(n, p, 0.3, 8)
     dg = lib.graph_from(g)
     want = lib.to_numpy_u64(lib.count_tuned(dg, t, method=lib.METHOD_ENUMERATE))
-    b = lib.Batch(dg, t, 7, 0)
+    b = lib.Batch(dg, t, R, 0)
     assert b.launch_info()["keeps_lists"]
-    h = lib.to_numpy_u64(b.run(np.arange(1, 8, dtype=np.uint64))[0])
+    h = lib.to_numpy_u64(b.run(np.arange(1, R + 1, dtype=np.uint64))[0])
     assert b.error() == 0
-    for r in range(8):
+    for r in range(R + 1):
         np.testing.assert_array_equal(h[r], want)
     b.free()
     dg.free()
     t.free()
 
 
-@pytest.mark.parametrize("R,keeps", [(6, False), (7, True)])
-def test_batches_around_the_graphs_it_takes_to_keep_lists(lib, R, keeps):
+@pytest.mark.parametrize("k,n,m,dmax,R,keeps", [
+    (5, 900, 5000, None, 7, False), (5, 900, 5000, None, 15, True),   # sets per item
+    (5, 700, 3000, None, 15, False), (5, 700, 3000, None, 31, True),
+    (5, 700, 3000, 20, 63, False),                                    # degrees
+    (6, 300, 1100, 40, 15, False), (6, 300, 1100, 40, 31, True),
+    (6, 300, 1100, 25, 63, False)])
+def test_both_sides_of_the_rule_for_keeping_lists(lib, k, n, m, dmax, R, keeps):
+    """Every row against the single count of the same null graph, which reads the
+    rows each time, and one against per-subgraph classification."""
     lib.load_library()
-    t = lib.table_build(5)
-    g = syn.chung_lu_digraph(200, 800, 2.2, None, 0.1, 4)
+    t = lib.table_build(k)
+    g = syn.chung_lu_digraph(n, m, 2.2 if k == 5 else 2.4, dmax, 0.1, 5)
     dg = lib.graph_from(g)
     b = lib.Batch(dg, t, R, 2 * g.m)
     assert b.launch_info()["keeps_lists"] == keeps
     h = lib.to_numpy_u64(b.run(np.arange(1, R + 1, dtype=np.uint64))[0])
     assert b.error() == 0
-    cm = t.class_masks()
-    for r in (0, R):
-        gr = g if r == 0 else syn.Graph(g.n, *oracle.randomize(g, r, 2 * g.m)[:2])
-        np.testing.assert_array_equal(h[r], oracle_dense(oracle.count(gr, 5)[0], cm))
+    for r in range(R + 1):
+        one = dg if r == 0 else lib.randomize(dg, r, 2 * g.m)
+        np.testing.assert_array_equal(
+            h[r], lib.to_numpy_u64(lib.count_tuned(one, t, method=lib.METHOD_CELLS)))
+    np.testing.assert_array_equal(
+        h[R], lib.to_numpy_u64(lib.count_tuned(one, t, method=lib.METHOD_ENUMERATE)))
     b.free()
     dg.free()
     t.free()

@@ -560,7 +560,7 @@ constexpr int kNumbered = 64;
 //  * by estimated sets per item, k = 5: the workload graph (n = 1,500) at 6.7 (8 graphs)
 //    3.86 : 4.00, 7.6 4.30 : 4.29, 8.4 4.77 : 4.56, 13 7.4 : 5.8, 217 (257 graphs) 116 :
 //    85; n = 700 at 7 3.79 : 3.85, 10 4.97 : 4.38; n = 400 at 7 2.70 : 2.86, 14 5.2 : 4.8; a
-//    hub of degree 400 in a sparse background at 2.8 1.85 : 1.95, 12 6.4 : 5.3; hubs of 64 to
+//    hub of degree 400 in a sparse background at 3 1.85 : 1.95, 12 6.4 : 5.3; hubs of 64 to
 //    200 and small graphs, at 0.4 to 4, lost 5 to 8%;
 //  * k = 6: the workload graph (n = 800) at 26 (8 graphs) 8.9 : 8.5, 210 (65) 71.3 : 67.9;
 //    n = 500 at 15 5.18 : 5.02; a hub of degree 150 at 16 5.3 : 5.1; hubs of 44 and 80, at 1 to

@@ -142,3 +142,17 @@ def test_server_by_name(lib, tables):
         np.testing.assert_array_equal(hist, per_subgraph(lib, lib.graph_from(g), ts[k]))
     assert srv.used_bytes() == 0
     srv.free()
+
+
+@pytest.mark.parametrize("name", ["uniform_k3", "chunglu_k4", "nullmodel_k5", "nullmodel_k6"])
+def test_workload_graphs(lib, tables, name):
+    """The four workload graphs, hubs and rows of many batches among them: the
+    cell method's histogram, and at k = 3 and 4 the oracle's."""
+    k = syn.WORKLOADS[name]["k"]
+    g = syn.workload_graph(name)
+    t = tables(k)
+    dg = lib.graph_from(g)
+    got = per_subgraph(lib, dg, t)
+    np.testing.assert_array_equal(got, lib.count_host(dg, t))
+    if k <= 4:
+        np.testing.assert_array_equal(got, oracle_dense(oracle.count(g, k)[0], t.class_masks()))

@@ -21,7 +21,7 @@
  * - Handles (mt_graph, mt_table, mt_batch) own device memory the library
  *   allocated; the caller frees them with the matching *_free.  Graphs and
  *   scratch come from a memory pool per device, which keeps up to 128 MiB of
- *   freed memory for the next ones while any graph or table is alive.  Buffers passed
+ *   freed memory for the next ones while any graph or table there is alive.  Buffers passed
  *   in by the caller stay the caller's.  Pointers documented as "device or host"
  *   are inspected with cudaPointerGetAttributes: a device pointer keeps the call
  *   asynchronous, a host pointer makes the call copy and synchronise the stream.

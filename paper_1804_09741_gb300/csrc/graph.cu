@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(1024) k_rank(int n, const int32_t* __restrict_
 // ------------------------------------------------------------------ device memory of the handles
 
 // Graphs, their scratch and the builder's come from a pool per device that keeps
-// up to kPoolKeep bytes between allocations while any graph or table is alive:
+// up to kPoolKeep bytes between allocations while any graph or table there is alive:
 // with the runtime's own calls one load, count and free of a small graph spent
 // 0.4 ms in cudaMalloc, cudaFree (50 us each) and in returning stream-ordered
 // scratch to the system at every synchronisation (85 us).  What the pool keeps goes
@@ -292,23 +292,21 @@ constexpr int kPoolDevices = 64;
 namespace {
 std::mutex g_pool_mu;
 cudaMemPool_t g_pools[kPoolDevices] = {};
-int64_t g_live_handles = 0;
+int64_t g_live_handles[kPoolDevices] = {};
 }  // namespace
 
-void handle_born() {
+void handle_born(int device) {
   std::lock_guard<std::mutex> lock(g_pool_mu);
-  ++g_live_handles;
+  if (device >= 0 && device < kPoolDevices) ++g_live_handles[device];
 }
 
-void handle_died() {
+void handle_died(int device) {
   std::lock_guard<std::mutex> lock(g_pool_mu);
-  if (--g_live_handles > 0) return;
-  for (int d = 0; d < kPoolDevices; ++d)
-    if (g_pools[d]) {
-      DeviceScope on(d);
-      cudaDeviceSynchronize();  // the frees are stream-ordered: until then nothing can be trimmed
-      cudaMemPoolTrimTo(g_pools[d], 0);
-    }
+  if (device < 0 || device >= kPoolDevices || --g_live_handles[device] > 0 || !g_pools[device])
+    return;
+  DeviceScope on(device);
+  cudaDeviceSynchronize();  // the frees are stream-ordered: until then nothing can be trimmed
+  cudaMemPoolTrimTo(g_pools[device], 0);
 }
 
 cudaError_t pool_alloc(void** out, size_t bytes, cudaStream_t s) {
@@ -396,7 +394,7 @@ static mt_status graph_alloc_impl(int32_t n, int32_t m, bool pooled, cudaStream_
     set_last_error(cudaGetErrorString(e));
     return e == cudaErrorMemoryAllocation ? MT_ENOMEM : MT_ECUDA;
   }
-  handle_born();
+  handle_born(g->device);
   g->mem_stats = (BuildStats*)g->mem;
   int32_t* p = (int32_t*)((char*)g->mem + 256);
   g->row_ptr = p; p += n + 1;  // row_ptr, rank and off are copied together
@@ -431,8 +429,9 @@ static void graph_free_on(mt_graph* g, cudaStream_t s) {
   }
   if (g->ev0) cudaEventDestroy(g->ev0);
   if (g->ev1) cudaEventDestroy(g->ev1);
+  const int device = g->device;
   delete g;
-  handle_died();
+  handle_died(device);
 }
 
 void graph_release(mt_graph* g, cudaStream_t s) {

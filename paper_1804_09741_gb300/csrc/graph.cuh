@@ -107,8 +107,8 @@ mt_status graph_build_original(mt_graph* g, void* scratch, cudaStream_t s);
 // Device memory of handles and their scratch, in the order of stream `s`.
 cudaError_t pool_alloc(void** out, size_t bytes, cudaStream_t s);
 void pool_free(void* p, cudaStream_t s);
-void handle_born();
-void handle_died();
+void handle_born(int device);
+void handle_died(int device);
 
 DevGraph dev_view(const mt_graph* g, unsigned long long* hist, bool original = false);
 

@@ -29,6 +29,7 @@
 struct mt_table {
   int k = 0;
   uint32_t classes = 0;
+  int device = 0;
   uint64_t nkeys = 0;
   uint32_t* table = nullptr;        // device, nkeys
   uint32_t* class_masks = nullptr;  // device, classes
@@ -541,7 +542,8 @@ static void table_drop(mt_table* t) {
 }
 
 static mt_status table_done(mt_table* t, mt_table** out) {
-  handle_born();
+  cudaGetDevice(&t->device);
+  handle_born(t->device);
   *out = t;
   return MT_OK;
 }
@@ -787,9 +789,11 @@ mt_status mt_table_is_compact(const mt_table* t, int* compact) {
 
 mt_status mt_table_free(mt_table* t) {
   if (!t) return MT_OK;
+  const int device = t->device;
+  DeviceScope on(device);
   cudaDeviceSynchronize();
   table_drop(t);
-  handle_died();
+  handle_died(device);
   return MT_OK;
 }
 

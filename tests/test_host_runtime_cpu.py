@@ -122,21 +122,27 @@ def test_set_workspace_waits_for_the_graphs_device(fake):
 
 def test_pools_are_trimmed_after_their_frees_have_run(fake):
     """Memory freed in stream order is the pool's only once the stream gets there:
-    with the last handle each device is waited for before its pool is trimmed."""
+    with its last handle a device is waited for before its pool is trimmed, and no
+    other device is."""
     fake.cudaSetDevice(1)
-    g1, g2 = fake.graph(*PATH), fake.graph(*PATH)
+    g1, g2, t1 = fake.graph(*PATH), fake.graph(*PATH), fake.table(3)
     fake.cudaSetDevice(0)
     g0 = fake.graph(*PATH)
-    fake.mt_graph_free(g1)
-    fake.mt_graph_free(g0)
-    fake.log()
-    fake.mt_graph_free(g2)  # the last one
-    log = calls(fake.log(), "sync", "free_async", "trim")
-    trims = [i for i, e in enumerate(log) if e[0] == "trim"]
-    assert {log[i][1] for i in trims} == {0, 1}
-    for i in trims:
-        last_free = max(j for j, e in enumerate(log[:i]) if e[0] == "free_async")
-        assert ("sync", log[i][1]) in [e[:2] for e in log[last_free:i]]
+
+    def freed(free, handle):
+        fake.log()
+        assert free(handle) == mt.MT_OK
+        log = calls(fake.log(), "sync", "free_async", "trim")
+        return [e[:2] for e in log]
+    assert "trim" not in [e[0] for e in freed(fake.mt_graph_free, g1)]
+    for free, last, device in ((fake.mt_graph_free, g0, 0), (fake.mt_graph_free, g2, None),
+                               (fake.mt_table_free, t1, 1)):
+        log = freed(free, last)
+        if device is None:
+            assert "trim" not in [e[0] for e in log]
+            continue
+        assert log[-2:] == [("sync", device), ("trim", device)]
+        assert {d for _, d in log} == {device}
     dev = ctypes.c_int()
     fake.cudaGetDevice(ctypes.byref(dev))
     assert dev.value == 0

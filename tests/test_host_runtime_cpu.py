@@ -4,7 +4,6 @@ be trimmed, what a server's budget is charged.  The library's objects are linked
 with a CUDA runtime that runs no kernel and logs the calls (fake_cudart/), so
 nothing here needs a GPU."""
 import ctypes
-import glob
 import os
 import re
 import shutil
@@ -65,16 +64,17 @@ def fake(tmp_path_factory):
     gxx = shutil.which("g++")
     if gxx is None or not os.path.exists(os.path.join(CUDA, "include", "cuda_runtime_api.h")):
         pytest.skip("no host compiler or CUDA headers")
-    if not b.up_to_date():
+    objects = [os.path.join(b.BUILD, os.path.basename(src)[:-3] + ".o") for src in b._sources()]
+    if not b.up_to_date() or not all(os.path.exists(o) for o in objects):
         if not os.path.exists(b.NVCC):
             pytest.skip("nvcc not available to build the library")
-        b.build()
+        b.build(force=True)
     out = str(tmp_path_factory.mktemp("fake") / "libmotifs_fake.so")
     # -Bsymbolic: the library's calls go to this runtime, whatever else is loaded
     subprocess.check_call([gxx, "-std=c++17", "-O1", "-fPIC", "-shared", "-Wl,-Bsymbolic",
                            "-I", os.path.join(CUDA, "include"),
                            os.path.join(HERE, "fake_cudart", "cudart.cc"),
-                           *sorted(glob.glob(os.path.join(b.BUILD, "*.o"))), "-o", out])
+                           *objects, "-o", out])
     return Fake(out)
 
 

@@ -262,11 +262,10 @@ static bool settle_loads(mt_server* s, std::vector<SrvRequest*>& loading, size_t
       failed[r->k - 3] = any = true;
     }
   }
-  for (int ki = 0; ki < 4; ++ki) {
+  for (int ki = 0; ki < 4; ++ki)
     if (failed[ki]) s->reserved[ki] = std::max(before[ki], scratch_need(s, ki, nullptr));
-    before[ki] = s->reserved[ki];
-  }
   if (any) release_idle_scratch(s);
+  std::copy(s->reserved, s->reserved + 4, before);
   loading.clear();
   return any;
 }
